@@ -564,24 +564,25 @@ def kernel_rooflines(precision, st, phase_ms, peaks, peak_kind):
                      "peak_source": ("bf16_tflops (%s)" % peak_kind) if bound == "tensor" else
                      "FP32 FFMA: 152 SMs x 128 lanes x 2 FLOP x %.0f MHz (derived)" % sm_max})
 
+    def x6_row(name, phase, units):
+        # six BF16 tensor products per hidden-layer product (executed FLOP)
+        ms = phase_ms.get(phase)
+        if not ms or units <= 0:
+            return
+        fl = units * 6 * 2 * 5 * 256 * 256
+        ach = fl / (ms / 1e3) / 1e12
+        rows.append({"kernel": name, "bound": "tensor", "achieved": ach, "peak": bf16_peak, "unit": "TFLOP/s",
+                     "frac": ach / bf16_peak, "traffic": ncu_traffic(name, units), "kernel_ms": ms,
+                     "flop_per_launch": fl, "units_per_launch": units,
+                     "peak_source": "bf16_tflops (%s)" % peak_kind})
+
     if precision in ("bf16", "bf16x6"):
         row("k_mlp_bf16<256,0,2>", "hop", st["hop_evals"], "tensor")
         row("k_mlp_bf16<256,1,2>", "vertices", st["unique_vertices"], "tensor")
-        if precision == "bf16":
-            row("k_pts_mlp_fp32<256,1>", "refine", st["refined_vertices"], "alu")
-        elif phase_ms.get("refine"):
-            # six BF16 tensor products per hidden-layer product (executed FLOP)
-            fl = st["refined_vertices"] * 6 * 2 * 5 * 256 * 256
-            ms = phase_ms["refine"]
-            ach = fl / (ms / 1e3) / 1e12
-            rows.append({"kernel": "k_mlp_x6<256,0>", "bound": "tensor", "achieved": ach, "peak": bf16_peak,
-                         "unit": "TFLOP/s", "frac": ach / bf16_peak, "traffic": ncu_traffic("k_mlp_x6<256,0>",
-                         st["refined_vertices"]), "kernel_ms": ms, "flop_per_launch": fl,
-                         "units_per_launch": st["refined_vertices"],
-                         "peak_source": "bf16_tflops (%s)" % peak_kind})
+        x6_row("k_mlp_x6<256,2>", "refine", st["refined_vertices"])
     else:
-        row("k_hop_mlp_fp32<256>", "hop", st["hop_evals"], "alu")
-        row("k_pts_mlp_fp32<256,0>", "vertices", st["unique_vertices"], "alu")
+        x6_row("k_mlp_x6<256,0>", "hop", st["hop_evals"])
+        x6_row("k_mlp_x6<256,1>", "vertices", st["unique_vertices"])
     mc = mesh_write_row(st, WORKLOAD["N"], phase_ms.get("mc"), peaks, peak_kind)
     if mc:
         rows.append(mc)
@@ -625,7 +626,7 @@ def companion(gh, torch, sdb, N, bufs, stream, flush, precision="fp32", eps=None
         ach = tensor / (ph["refine"] / 1e3) / 1e12
         bf = float(peaks.get("bf16_tflops", 1917.8))
         out["refine_roofline"] = {
-            "kernel": "k_mlp_x6<256,0>", "bound": "tensor", "achieved": ach, "peak": bf, "unit": "TFLOP/s",
+            "kernel": "k_mlp_x6<256,2>", "bound": "tensor", "achieved": ach, "peak": bf, "unit": "TFLOP/s",
             "frac": ach / bf, "traffic": None, "kernel_ms": ph["refine"], "units_per_launch": st["refined_vertices"],
             "flop_per_launch": tensor, "peak_source": "bf16_tflops (%s)" % peak_kind,
             "fp32_equivalent_tflops": st["refined_vertices"] * FLOP_PER_EVAL / (ph["refine"] / 1e3) / 1e12}

@@ -124,16 +124,19 @@ typedef struct {
     float hi[3];  /* three axes (a cube, Sec. 2)                            */
 } gh_grid;
 
-#define GH_FP32 0        /* every evaluation in FP32                           */
+#define GH_FP32 0        /* every evaluation at FP32 accuracy                  */
 #define GH_BF16_REFINE 1 /* neural SDB: hop in BF16 with an error bound eps,   */
-                         /* corners of candidate cells re-evaluated in FP32    */
-/* GH_BF16_REFINE_X6: as GH_BF16_REFINE, but the corners are re-evaluated on
- * the tensor cores with split-BF16 products instead of FP32 FMAs: every FP32
- * operand of a hidden layer is split exactly into three BF16 parts and the
- * six part products of size >= 2^-16 of the product are accumulated in FP32
- * (the dropped three are below about 2^-23 of it).  Not FP32 arithmetic:
- * its error against exact arithmetic is of FP32's size, not bit-identical to
- * GH_FP32.  gh_eval takes it too (points evaluated that way). */
+                         /* corners of candidate cells re-evaluated as GH_FP32 */
+/* How GH_FP32 evaluates a neural SDB of up to 8 hidden layers: on the tensor
+ * cores with split-BF16 products.  Every FP32 operand of a hidden layer is
+ * split exactly into three BF16 parts, the six part products of size >=
+ * 2^-16 of the product are accumulated in FP32 (the dropped three are below
+ * about 2^-23 of it), and the mean truncation of the tensor core's accumulator
+ * is added back; its error against exact arithmetic is below that of a chain
+ * of FP32 FMAs.  A hidden activation that overflows float32 makes f NaN
+ * (GH_ERR_NONFINITE).  Deeper networks run on FP32 FMAs.
+ * GH_BF16_REFINE_X6: as GH_BF16_REFINE; it names the split-BF16 evaluator
+ * explicitly (networks it does not take are refused), gh_eval takes it too. */
 #define GH_BF16_REFINE_X6 2
 /* The BF16 modes support widths 64, 128 and 256 with at most 8 hidden layers
  * (n_mid), 7 at width 256, and the split-BF16 evaluator at most 8; other

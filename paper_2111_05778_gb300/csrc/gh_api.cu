@@ -348,13 +348,14 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     // in place from the uploaded block
     const size_t WW = (size_t)W * W;
     float *d_wt, *d_wtb, *d_bm;
-    uint16_t *d_wbf, *d_wx6;
+    uint16_t *d_wbf, *d_wx6, *d_wx6t;
     if (dev_alloc(s, &s->d_params, (size_t)np) || dev_alloc(s, &d_wt, (size_t)h.n_mid * WW) ||
         dev_alloc(s, &d_wtb, (size_t)h.n_mid * WW) || dev_alloc(s, &d_bm, (size_t)h.n_mid * W) ||
-        dev_alloc(s, &d_wbf, (size_t)h.n_mid * WW) || dev_alloc(s, &d_wx6, (size_t)3 * h.n_mid * WW))
+        dev_alloc(s, &d_wbf, (size_t)h.n_mid * WW) || dev_alloc(s, &d_wx6, (size_t)3 * h.n_mid * WW) ||
+        dev_alloc(s, &d_wx6t, (size_t)3 * h.n_mid * WW))
         return GH_ERR_CUDA;
     GH_CUDA(cudaMemcpy(s->d_params, P, sizeof(float) * np, cudaMemcpyHostToDevice));
-    launch_prep_mlp(s->d_params, W, h.n_mid, d_wt, d_wtb, d_wbf, d_wx6, d_bm, 0);
+    launch_prep_mlp(s->d_params, W, h.n_mid, d_wt, d_wtb, d_wbf, d_wx6, d_wx6t, d_bm, 0);
     GH_CUDA(cudaGetLastError());
     GH_CUDA(cudaStreamSynchronize(0));  // the layouts are complete before any stream uses them
     const float *d_w0 = s->d_params, *d_b0 = s->d_params + 3 * W;
@@ -376,6 +377,7 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     m.bout = wout[W];
     m.wbf = d_wbf;
     m.wx6 = d_wx6;
+    m.wx6t = d_wx6t;
     s->nparam = np;
     return GH_OK;
 }
@@ -638,6 +640,22 @@ static inline void mark_phase(int i, cudaStream_t st) {
 static constexpr int LAUNCHES_HOP = 2, LAUNCHES_LISTS = 8, LAUNCHES_VERTS = 1, LAUNCHES_REFINE = 4,
                      LAUNCHES_MC = 2;
 
+// FP32 evaluation of a neural SDB: on the tensor cores with split-BF16
+// products (k_mlp_x6.cu; error below sequential FP32 FMAs', 2^20 points in
+// 2.32 / 0.65 / 0.29 ms at width 256 / 128 / 64 against 10.0 / 2.82 / 0.81), on
+// the FFMA engine for networks deeper than that engine's shared memory takes.
+static bool fp32_on_tensor(const MlpDev &m) { return m.n_mid <= x6_max_mid(); }
+
+static void hop_mlp_fp32(const gh_sdb *first, const Item *di, int n, int nsm, cudaStream_t st) {
+    if (fp32_on_tensor(first->mlp)) launch_hop_mlp_x6(di, n, first->mlp.width, nsm, st);
+    else launch_hop_mlp_fp32(di, n, first->mlp.width, nsm, st);
+}
+
+static void vertices_mlp_fp32(const gh_sdb *first, const Item *di, int n, int nsm, bool refine_list, cudaStream_t st) {
+    if (fp32_on_tensor(first->mlp)) launch_eval_vertices_mlp_x6(di, n, first->mlp.width, nsm, refine_list, st);
+    else launch_eval_vertices_mlp_fp32(di, n, first->mlp.width, nsm, refine_list, st);
+}
+
 static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh_mesh &out, int nsm,
                         cudaStream_t st) {
     Scratch &c = s->scr;
@@ -650,6 +668,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
     if (o.method == GH_METHOD_ENUM) {
         // Sec. 2 enumeration: every lattice point, every cell
         if (s->kind == GH_SDB_CSG) launch_lattice_csg(s->d_prims, s->nprim, g, c, st);
+        else if (fp32_on_tensor(s->mlp)) launch_lattice_mlp_x6(s->d_item, s->mlp.width, nsm, st);
         else launch_lattice_mlp_fp32(s->d_item, s->mlp.width, nsm, st);
         launch_enum_stats(g, c, st);
         for (int p = 1; p <= 5; ++p) mark_phase(p, st);
@@ -671,11 +690,11 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(4, st);
         mark_phase(5, st);
     } else if (o.precision == GH_FP32) {
-        launch_hop_mlp_fp32(s->d_item, 1, s->mlp.width, nsm, st);
+        hop_mlp_fp32(s, s->d_item, 1, nsm, st);
         mark_phase(1, st);
         launch_build_lists(g, c, st);
         mark_phase(2, st);
-        launch_eval_vertices_mlp_fp32(s->d_item, 1, s->mlp.width, nsm, false, st);
+        vertices_mlp_fp32(s, s->d_item, 1, nsm, false, st);
         mark_phase(3, st);
         mark_phase(4, st);
         mark_phase(5, st);
@@ -688,8 +707,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(3, st);
         launch_refine_select(g, c, st);
         mark_phase(4, st);
-        if (o.precision == GH_BF16_REFINE_X6) launch_refine_mlp_x6(s->d_item, 1, s->mlp.width, nsm, st);
-        else launch_eval_vertices_mlp_fp32(s->d_item, 1, s->mlp.width, nsm, true, st);
+        vertices_mlp_fp32(s, s->d_item, 1, nsm, true, st);
         mark_phase(5, st);
         launches += LAUNCHES_REFINE;
     }
@@ -856,7 +874,8 @@ extern "C" int gh_eval(const gh_sdb *s, const float *p, int64_t n, float *out, i
     if (s->kind == GH_SDB_CSG) {
         launch_eval_points_csg(s->d_prims, s->nprim, p, n, out, st);
     } else if (precision == GH_FP32) {
-        launch_eval_points_mlp_fp32(s->mlp, p, n, out, nsm, st);
+        if (fp32_on_tensor(s->mlp)) launch_eval_points_mlp_x6(s->mlp, p, n, out, nsm, st);
+        else launch_eval_points_mlp_fp32(s->mlp, p, n, out, nsm, st);
     } else if (precision == GH_BF16_REFINE) {
         if (!bf16_supported(s->mlp.width) || s->mlp.n_mid > bf16_max_mid(s->mlp.width))
             return fail(GH_ERR_UNIMPLEMENTED, "no BF16 path for this width / depth");
@@ -1000,7 +1019,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             for (int q = gr.first; q < gr.second; ++q) mx = sd[P.order[q]]->nprim > mx ? sd[P.order[q]]->nprim : mx;
             launch_hop_csg(di, n, mx, nsm, o.ray_block, st);
         } else if (o.precision == GH_FP32) {
-            launch_hop_mlp_fp32(di, n, first->mlp.width, nsm, st);
+            hop_mlp_fp32(first, di, n, nsm, st);
         } else {
             launch_hop_mlp_bf16(di, n, first->mlp.width, nsm, tiles, st);
         }
@@ -1016,7 +1035,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         const Item *di = P.d_items + gr.first;
         const int n = gr.second - gr.first;
         ++launches;
-        if (o.precision == GH_FP32) launch_eval_vertices_mlp_fp32(di, n, first->mlp.width, nsm, false, st);
+        if (o.precision == GH_FP32) vertices_mlp_fp32(first, di, n, nsm, false, st);
         else launch_eval_vertices_mlp_bf16(di, n, first->mlp.width, nsm, tiles, st);
     }
     if (any_mlp && o.precision != GH_FP32) {
@@ -1028,8 +1047,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             const Item *di = P.d_items + gr.first;
             const int n = gr.second - gr.first;
             ++launches;
-            if (o.precision == GH_BF16_REFINE_X6) launch_refine_mlp_x6(di, n, first->mlp.width, nsm, st);
-            else launch_eval_vertices_mlp_fp32(di, n, first->mlp.width, nsm, true, st);
+            vertices_mlp_fp32(first, di, n, nsm, true, st);
         }
     }
     launch_mc_b(P.d_items, B, nsm, st);

@@ -1,4 +1,5 @@
-// Neural SDB in FP32 on the FFMA pipe.
+// Neural SDB in FP32 on the FFMA pipe: the evaluator of networks deeper than
+// the split-BF16 tensor engine takes (k_mlp_x6.cu, 2.8 to 4.4 times as fast).
 //
 // f(p) = (|p| - r0 + alpha g(p)) / beta / lambda with g a ReLU MLP (the
 // neural SDB of Sec. 5.2, Eq. 7).  A CTA of 256 threads evaluates a tile of

@@ -1,33 +1,48 @@
-// Neural SDB on the tensor cores at FP32-level accuracy: split-BF16 products
-// ("x6"), used for the refinement of the BF16 path and, through gh_eval, for
-// point lists.
+// Neural SDB on the tensor cores at FP32 accuracy: split-BF16 products.  This
+// is the FP32 evaluator of networks up to x6_max_mid() hidden layers (deeper
+// ones run on the FFMA engine, k_mlp_fp32.cu): FP32 hopping, vertex values,
+// the refinement of the BF16 path, point lists, the enumeration lattice and
+// the adjoint's forward pass and delta chain.
 //
 // Every FP32 operand x of a hidden layer is split exactly into three BF16
 // parts, x = x_h + x_m + x_l (x_h = bf16(x), x_m = bf16(x - x_h), x_l =
-// bf16(x - x_h - x_m); each difference is exact in FP32 and the three parts
-// carry 24 significant bits).  Of the nine part products of a * w the six
+// bf16(x - x_h - x_m)); each difference is exact in FP32 and the three parts
+// carry 24 significant bits.  Of the nine part products of a * w the six
 // whose size is at least 2^-16 |a w| are formed on the tensor core (hh, hm,
 // mh, hl, lh, mm) with FP32 accumulation in tensor memory; the three dropped
 // (ml, lm, ll) are below 2^-23 |a w| together, the size of one FP32 rounding.
-// Products are accumulated from the smallest to the largest: per layer the
-// weight parts stream in the order low, middle, high, and within the high
-// part's K-block the activation parts low, middle, high.  Layer 0 (3 -> W) and
-// the output layer (W -> 1) run on CUDA cores in FP32, in the FP32 engine's
-// operation order.
+// The accumulator adds the products from the smallest to the largest in four
+// passes over the layer's inputs: x_h w_l; x_m w_m and x_h w_m; x_l w_h and
+// x_m w_h; x_h w_h.  Only the last pass's W/16 updates are at the size of the
+// result.  The accumulator is truncated toward zero: on layers of like-signed
+// terms it was short by 0.50 / 0.62 / 1.50 units in the last place on average
+// at width 64 / 128 / 256 (0.63 / 1.1 / 2.3 with mixed signs; deviation 0.3 /
+// 0.4 / 0.6), which the epilogue adds back on average (KAPPA).  What remains
+// is below the error of a chain of FP32 FMAs (deviation 1.2 / 1.6 / 2.2).
+// The last two passes share the high part's stages in the ring.  Layer 0
+// (3 -> W) and the output layer (W -> 1) run on CUDA cores in FP32.
 //
-// One persistent CTA per SM, 384 threads, one 128-row tile at a time:
+// Persistent CTAs, one 128-row tile at a time each, 64 + 2 W threads:
 //   warp 0       bulk-copy producer: K-blocks (64 inputs x W outputs) of one
 //                weight part per stage, stored pre-swizzled in global
 //                memory, into a 4-stage shared-memory ring.
 //   warp 1       allocates TMEM (2W columns); one lane issues tcgen05.mma
-//                (M = 128, N = W, K = 16): A = x_h from shared memory, or
-//                x_m / x_l from tensor memory.
-//   warps 4..11  epilogue, two threads per row (column halves): layer 0,
-//                TMEM -> registers -> bias, ReLU, the exact three-way split ->
-//                x_h into 128B-swizzled shared memory and x_m, x_l into
-//                tensor memory (the next layer's A operands); the output
-//                dot product; the store of f.
-// TMEM columns: [0, W) accumulator, [W, 3W/2) x_m, [3W/2, 2W) x_l (two BF16
+//                (M = 128, N = W, K = 16): A = x_h or x_m from tensor memory,
+//                or x_l from shared memory.
+//   warps 2..    epilogue, W/64 threads per row, 64 columns (one K-block of
+//                the next layer) each: layer 0, TMEM -> registers -> bias,
+//                ReLU, the exact three-way split -> x_h and x_m into tensor
+//                memory, x_l into 128B-swizzled shared memory (the next
+//                layer's A operands); the output dot product; the hop step of
+//                Algorithm 1 or the store of f.
+// A thread holds its 64 columns in registers, so the accumulator is free and
+// the next layer's first pass (x_h only) starts as soon as x_h is stored; the
+// middle and low parts are computed under it (barriers a_h and a_ml).
+// x_l, which only one of the six products reads, is the part in shared memory:
+// its port carries the weights' copies and the B operands already, and runs
+// of products with A in shared memory took 183 cycles each at width 256,
+// with A in tensor memory 122.
+// TMEM columns: [0, W) accumulator, [W, 3W/2) x_h, [3W/2, 2W) x_m (two BF16
 // per 32-bit column, K ascending).  Every wait is bounded as in the BF16
 // engine; a timeout sets the error flag, every role leaves, copies in flight
 // land and MMAs complete before TMEM is freed.
@@ -43,38 +58,71 @@ namespace {
 using namespace tc;
 
 constexpr int TM = 128;   // rows per tile
-constexpr int NST = 4;    // weight ring stages
-constexpr int EPI = 256;  // epilogue threads (warps 4..11)
+constexpr int NPASS = 4;  // weight passes per layer: low, middle, high (with x_l, x_m), high (with x_h)
+constexpr int EPI_T0 = 64;  // first epilogue thread (warp 2)
 constexpr int MAXMID = 8;
+constexpr unsigned FULL = 0xFFFFFFFFu;
+constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
 constexpr int BAR_EPI = 1;  // named barrier of the epilogue threads
 
-enum { XMODE_REFINE = 0, XMODE_POINTS = 1 };
+enum { XM_HOP = 0, XM_VERTS = 1, XM_REFINE = 2, XM_POINTS = 3, XM_LATTICE = 4, XM_ADJ = 5 };
+
+// Resident CTAs per SM the registers are budgeted for: TMEM (2W of 512
+// columns) and shared memory (217 / 105 / 53 KB) allow 1, 2 and 4; at width
+// 64 three CTAs leave the threads the registers that four would spill.
+template <int W>
+constexpr int ctas_of() {
+    return W == 256 ? 1 : (W == 128 ? 2 : 3);
+}
+
+// Weight ring stages: a divisor of the 3 W/64 stages of a layer, so that the
+// K-blocks of every layer fall on the same stages and the issuing thread's
+// loop over a layer is straight-line code with constant stage addresses and
+// barriers.  (Computing them per stage cost that thread about 400 cycles: 728
+// cycles for a stage of four products instead of the 512 of the products.)
+template <int W>
+constexpr int nst_of() {
+    return W == 256 ? 4 : 3;
+}
+
+// Mean shortfall of a truncated accumulator in units of its last place, as a
+// factor of the accumulator's power of two (2^e of its value m 2^e, 1 <= m < 2).
+template <int W>
+constexpr float kappa_of() {
+    return (W == 256 ? 1.9f : (W == 128 ? 0.8f : 0.5f)) * 1.1920929e-7f;
+}
+__device__ __forceinline__ float pow2_of(float v) { return __uint_as_float(__float_as_uint(v) & 0xFF800000u); }
 
 template <int W>
 struct SmemX {
-    uint8_t ah[W / 64][TM * 128];  // x_h: K-blocks of 128 rows x 128 B (1024-aligned)
+    static constexpr int NST = nst_of<W>();
+    uint8_t al[W / 64][TM * 128];  // x_l: K-blocks of 128 rows x 128 B (1024-aligned)
     uint8_t w[NST][W * 128];       // weight ring: one K-block of one part per stage
-    float4 w0b[W];                 // layer-0 rows and biases by output pairs (as the BF16 engine)
+    float4 w0b[W];                 // layer-0 rows and biases by output pairs
     float bmid[MAXMID * W];        // hidden-layer biases
     float wout[W];                 // output-layer weights
-    float red[2][TM];              // output dot products of the two column halves
-    unsigned long long full[NST], empty[NST], acc_full, a_full, item_ready, drain;
+    float4 pt[TM];                 // the tile's points
+    float red[3][W / 64][TM];      // per column group: output dot products (adjoint: grad_x g)
+    unsigned long long full[NST], empty[NST], acc_full, a_h, a_ml, item_ready, drain;
     const uint16_t *cur_w;         // split weights of the current item
-    unsigned long long base, total;
     int done;
     uint32_t tmem_base;
     int ctl;
 };
 
-// x = h + m + l exactly, each part BF16 (rounded to nearest even); two values
-// at a time, packed (lo value in the low half).
-__device__ __forceinline__ void split3(float x0, float x1, uint32_t &h, uint32_t &m, uint32_t &l) {
+// BF16 parts of two values, packed (x0 in the low half): the high part ...
+__device__ __forceinline__ uint32_t part_h(float x0, float x1) {
+    uint32_t h;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(x1), "f"(x0));
+    return h;
+}
+// ... and the middle and low ones: x = h + m + l, every difference exact.
+__device__ __forceinline__ void parts_ml(float x0, float x1, uint32_t &m, uint32_t &l) {
+    const uint32_t h = part_h(x0, x1);
     const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(r1), "f"(r0));
-    const float s0 = r0 - __uint_as_float(m << 16), s1 = r1 - __uint_as_float(m & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(s1), "f"(s0));
+    m = part_h(r0, r1);
+    l = part_h(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xFFFF0000u));
 }
 
 __device__ __forceinline__ float outer_f(const MlpDev &m, float x, float y, float z, float g) {
@@ -82,10 +130,10 @@ __device__ __forceinline__ float outer_f(const MlpDev &m, float x, float y, floa
     return (fmaf(m.alpha, g, m.radial * r - m.r0) / m.beta) * m.inv_lam;
 }
 
-// Loads item it's layer-0 rows, biases and output weights (epilogue threads).
+// Loads an item's layer-0 rows, biases and output weights (epilogue threads).
 template <int W>
 __device__ __forceinline__ void load_params(SmemX<W> &sm, const MlpDev &mm, int e) {
-    for (int o = e; o < W; o += EPI) {
+    for (int o = e; o < W; o += 2 * W) {
         float *q = reinterpret_cast<float *>(&sm.w0b[o & ~1]) + (o & 1);
         q[0] = mm.w0[3 * o];
         q[2] = mm.w0[3 * o + 1];
@@ -93,33 +141,104 @@ __device__ __forceinline__ void load_params(SmemX<W> &sm, const MlpDev &mm, int 
         q[6] = mm.b0[o];
         sm.wout[o] = mm.wout[o];
     }
-    for (int i = e; i < mm.n_mid * W; i += EPI) sm.bmid[i] = mm.bm[i];
+    for (int i = e; i < mm.n_mid * W; i += 2 * W) sm.bmid[i] = mm.bm[i];
 }
 
+// x[64] (this thread's row, columns 64 grp .., ReLU'd when RELU) -> x_h into
+// tensor memory (32 columns of two inputs each).  The ReLU is the conversion's,
+// so that x_h, which the next layer's first products wait for, takes as few
+// instructions as can be.
+template <bool RELU>
+__device__ __forceinline__ void put_h(const float (&x)[64], uint32_t th) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t h[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            h[p] = RELU ? pack_relu_bf16(x[16 * c + 2 * p], x[16 * c + 2 * p + 1])
+                        : part_h(x[16 * c + 2 * p], x[16 * c + 2 * p + 1]);
+        tmem_st8(th + 8 * c, h);
+    }
+    tmem_wait_st();
+}
+
+// x_m into tensor memory, x_l into K-block grp of the shared-memory operand
+template <bool RELU>
+__device__ __forceinline__ void put_ml(const float (&x)[64], uint32_t tm, uint32_t lrow, int sw) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t m[8], l[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+            const float x0 = x[16 * c + 2 * p], x1 = x[16 * c + 2 * p + 1];
+            parts_ml(RELU ? relu_nan(x0) : x0, RELU ? relu_nan(x1) : x1, m[p], l[p]);
+        }
+        tmem_st8(tm + 8 * c, m);
+        sts128(lrow + (uint32_t)(((2 * c) ^ sw) << 4), l[0], l[1], l[2], l[3]);
+        sts128(lrow + (uint32_t)(((2 * c + 1) ^ sw) << 4), l[4], l[5], l[6], l[7]);
+    }
+    tmem_wait_st();
+}
+
+// bit c set where x[c] > 0
+__device__ __forceinline__ uint2 relu_bits(const float (&x)[64]) {
+    uint2 b = make_uint2(0u, 0u);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        b.x |= (x[c] > 0.f ? 1u : 0u) << c;
+        b.y |= (x[c + 32] > 0.f ? 1u : 0u) << c;
+    }
+    return b;
+}
+
+// 64 floats of a row to global memory (16-byte aligned)
+__device__ __forceinline__ void store_row(float *dst, const float (&x)[64]) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+        reinterpret_cast<float4 *>(dst)[c] = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+}
+
+// The adjoint's buffers (XM_ADJ): activations relu(z_l) into A + l*ldl and
+// deltas delta_l into D + l*ldl (row-major [vertex][W]), ReLU masks, s_v.
+struct AdjOut {
+    const float *dL;
+    float *A, *D, *s;
+    uint2 *mask;  // [(l * rows + row) * (W/64) + group], rows = tiles * 128
+    long long ldl;
+    const uint16_t *wt6;  // split transposed weights, last layer first
+};
+
 template <int W, int MODE>
-__global__ void __launch_bounds__(384, 1)
-    k_mlp_x6(const Item *__restrict__ items, int n_items, const float *__restrict__ pts, long long npts,
-             float *__restrict__ outv, unsigned long long wait_ns) {
+__global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
+    k_mlp_x6(const Item *__restrict__ items_in, int n_items, const __grid_constant__ Item single,
+             const float *__restrict__ pts, long long npts, float *__restrict__ outv, AdjOut adj,
+             unsigned long long wait_ns) {
+    // point lists and the adjoint: the one descriptor comes with the launch
+    const Item *items = MODE == XM_POINTS || MODE == XM_ADJ ? &single : items_in;
     extern __shared__ uint8_t smem_raw[];
-    constexpr int KB = W / 64;                 // K-blocks per layer
+    constexpr int G = W / 64;                  // K-blocks per layer = column groups
+    constexpr int NST = nst_of<W>();
+    constexpr int EPI = 2 * W;                 // epilogue threads
     constexpr uint32_t STAGE_BYTES = W * 128;  // one K-block of one part
     constexpr uint32_t TMEM_COLS = 2 * W;      // 128, 256 or 512
-    constexpr uint32_t AM = W, AL = W + W / 2; // TMEM columns of x_m and x_l
+    constexpr uint32_t AH = W, AM = W + W / 2; // TMEM columns of x_h and x_m
     constexpr uint32_t IDESC = idesc_bf16(TM, W);
     SmemX<W> &sm = *reinterpret_cast<SmemX<W> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *ctl = &sm.ctl;
     Counters *ctr0 = items[0].s.ctr;  // error flags of a timeout go to the first item
     const int n_mid = items[0].m.n_mid;
+    const int n_gemm = MODE == XM_ADJ ? 2 * n_mid : n_mid;  // products per tile (adjoint: there and back)
 
-    if (tid >= 128) load_params<W>(sm, items[0].m, tid - 128);
+    if (tid >= EPI_T0) load_params<W>(sm, items[0].m, tid - EPI_T0);
     if (tid == 0) {
         for (int i = 0; i < NST; ++i) {
             mbar_init(&sm.full[i], 1);
             mbar_init(&sm.empty[i], 1);
         }
         mbar_init(&sm.acc_full, 1);
-        mbar_init(&sm.a_full, EPI);
+        mbar_init(&sm.a_h, EPI);
+        mbar_init(&sm.a_ml, EPI);
         mbar_init(&sm.item_ready, 1);
         mbar_init(&sm.drain, 1);
         sm.cur_w = items[0].m.wx6;
@@ -140,34 +259,34 @@ __global__ void __launch_bounds__(384, 1)
     volatile int *vdone = &sm.done;
 
     if (warp == 0) {
-        // ---- producer: per tile, n_mid layers x 3 parts x KB K-blocks ----------
+        // ---- producer: per tile, n_gemm layers x 3 parts x G K-blocks ----------
         if (lane == 0) {
-            long long issued = 0;
+            uint32_t issued = 0;
             uint32_t pir = 0;
             bool go = true;
             while (go) {
                 if (!wait_bar(&sm.item_ready, pir, ctl, CTL_ABORT, ctr0, wait_ns)) break;
                 pir ^= 1u;
                 if (*vdone) break;
-                const uint8_t *src = reinterpret_cast<const uint8_t *>(*(const uint16_t *volatile *)&sm.cur_w);
-                const int nst = n_mid * 3 * KB;
-                for (int s = 0; s < nst; ++s) {
-                    const int st = (int)(issued % NST);
-                    const uint32_t par = (uint32_t)(((issued / NST) & 1) ^ 1);
-                    if (!wait_bar(&sm.empty[st], par, ctl, CTL_ABORT, ctr0, wait_ns)) {
-                        go = false;
-                        break;
+                const uint8_t *wf = reinterpret_cast<const uint8_t *>(*(const uint16_t *volatile *)&sm.cur_w);
+                for (int l = 0; l < n_gemm && go; ++l) {
+                    const uint8_t *src = MODE == XM_ADJ && l >= n_mid ? reinterpret_cast<const uint8_t *>(adj.wt6) : wf;
+                    src += (size_t)(MODE == XM_ADJ && l >= n_mid ? l - n_mid : l) * 3 * G * STAGE_BYTES;
+                    for (int s = 0; s < 3 * G; ++s) {  // parts low, middle, high; the last pass finds high in the ring
+                        const uint32_t st = issued % NST, par = ((issued / NST) & 1) ^ 1;
+                        if (!wait_bar(&sm.empty[st], par, ctl, CTL_ABORT, ctr0, wait_ns)) {
+                            go = false;
+                            break;
+                        }
+                        mbar_expect_tx(&sm.full[st], STAGE_BYTES);
+                        bulk_g2s(sm.w[st], src + (size_t)s * STAGE_BYTES, STAGE_BYTES, &sm.full[st]);
+                        ++issued;
                     }
-                    mbar_expect_tx(&sm.full[st], STAGE_BYTES);
-                    bulk_g2s(sm.w[st], src + (size_t)s * STAGE_BYTES, STAGE_BYTES, &sm.full[st]);
-                    ++issued;
                 }
             }
             // the copies still in flight land before the CTA may exit
-            for (long long i = issued - NST; i < issued; ++i) {
-                if (i < 0) continue;
-                wait_bar(&sm.full[i % NST], (uint32_t)((i / NST) & 1), ctl, 0, ctr0);
-            }
+            for (uint32_t i = issued < NST ? 0 : issued - NST; i < issued; ++i)
+                wait_bar(&sm.full[i % NST], (i / NST) & 1, ctl, 0, ctr0);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -175,47 +294,53 @@ __global__ void __launch_bounds__(384, 1)
         // (lean issue loop: descriptors built once and advanced by fixed steps,
         // a stage that has landed taken without a call; k_mlp_bf16.cu)
         if (lane == 0) {
-            long long consumed = 0;
-            uint32_t pa = 0;
+            uint32_t pa = 0, pf = 0;  // phases: of the operand barriers, of the ring at the layer's first stage
             bool go = true;
             constexpr unsigned long long A_KB = (TM * 128) >> 4, W_ST = STAGE_BYTES >> 4;
-            const unsigned long long ahd = sdesc(su32(&sm.ah[0][0])), wd0 = sdesc(su32(sm.w[0]));
+            const unsigned long long ald = sdesc(su32(&sm.al[0][0])), wd0 = sdesc(su32(sm.w[0]));
             while (go) {
-                for (int l = 0; l < n_mid && go; ++l) {
-                    if (!wait_bar(&sm.a_full, pa, ctl, CTL_ABORT, ctr0, wait_ns)) {
+                for (int l = 0; l < n_gemm && go; ++l) {
+                    // x_h is stored and the accumulator has been read
+                    if (!mbar_try(&sm.a_h, pa) && !wait_bar(&sm.a_h, pa, ctl, CTL_ABORT, ctr0, wait_ns)) {
                         go = false;
                         break;
                     }
-                    pa ^= 1u;
                     if (l == 0 && *vdone) {
                         go = false;
                         break;
                     }
                     tc_fence_after();
-                    for (int part = 0; part < 3 && go; ++part) {  // weight parts low, middle, high
-                        for (int kb = 0; kb < KB; ++kb) {
-                            const int st = (int)(consumed % NST);
-                            const uint32_t par = (uint32_t)((consumed / NST) & 1);
-                            if (!mbar_try(&sm.full[st], par) &&
-                                !wait_bar(&sm.full[st], par, ctl, CTL_ABORT, ctr0, wait_ns)) {
+#pragma unroll
+                    for (int pass = 0; pass < NPASS; ++pass) {
+                        if (pass == 1 && go) {  // from here on x_m and x_l are read too
+                            if (!mbar_try(&sm.a_ml, pa) && !wait_bar(&sm.a_ml, pa, ctl, CTL_ABORT, ctr0, wait_ns))
                                 go = false;
-                                break;
-                            }
-                            const unsigned long long b0 = wd0 + (unsigned long long)st * W_ST;
-                            const unsigned long long a0 = ahd + (unsigned long long)kb * A_KB;
+                            tc_fence_after();
+                        }
+#pragma unroll
+                        for (int kb = 0; kb < G; ++kb) {
+                            // the layer's stages in order; the last pass takes the high part's again
+                            constexpr int S3 = 2 * G;
+                            const int s = (pass == 3 ? S3 : pass * G) + kb, st = s % NST;
+                            if (pass != 3 && go && !mbar_try(&sm.full[st], pf ^ ((s / NST) & 1)) &&
+                                !wait_bar(&sm.full[st], pf ^ ((s / NST) & 1), ctl, CTL_ABORT, ctr0, wait_ns))
+                                go = false;
+                            if (!go) continue;
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
-                                const unsigned long long bd = b0 + (unsigned long long)(2 * k);
+                                const unsigned long long bd = wd0 + (st * W_ST + 2 * k);
                                 const uint32_t acol = (uint32_t)(kb * 32 + k * 8);
-                                if (part == 2) umma_ta(tmem, tmem + AL + acol, bd, IDESC, 1u);  // x_l w_h
-                                if (part >= 1) umma_ta(tmem, tmem + AM + acol, bd, IDESC, 1u);  // x_m w_m, x_m w_h
-                                umma(tmem, a0 + (unsigned long long)(2 * k), bd, IDESC,
-                                     (part | kb | k) != 0);  // x_h w_l (the layer's first op), x_h w_m, x_h w_h
+                                if (pass == 2) umma(tmem, ald + (kb * A_KB + 2 * k), bd, IDESC, 1u);  // x_l w_h
+                                if (pass == 1 || pass == 2)  // x_m w_m, x_m w_h
+                                    umma_ta(tmem, tmem + AM + acol, bd, IDESC, 1u);
+                                if (pass != 2)  // x_h w_l (the layer's first op), x_h w_m, and last x_h w_h
+                                    umma_ta(tmem, tmem + AH + acol, bd, IDESC, (pass | kb | k) != 0);
                             }
-                            umma_commit(&sm.empty[st]);
-                            ++consumed;
+                            if (pass != 2) umma_commit(&sm.empty[st]);
                         }
                     }
+                    pa ^= 1u;
+                    pf ^= (3 * G / NST) & 1;
                     if (go) umma_commit(&sm.acc_full);
                 }
             }
@@ -224,37 +349,120 @@ __global__ void __launch_bounds__(384, 1)
             wait_bar(&sm.drain, 0, ctl, 0, ctr0);
         }
         __syncwarp();
-    } else if (warp >= 4) {
-        // ---- epilogue: two threads per row, column halves hf = 0, 1 --------------
-        const int e = tid - 128, ew = e >> 5, q = ew & 3, hf = ew >> 2;
+    } else {
+        // ---- epilogue: G threads per row, 64 columns each ------------------------
+        const int e = tid - EPI_T0, grp = e >> 7, q = warp & 3;  // a warp reads TMEM lanes 32 (warp % 4) ..
         const int row = 32 * q + lane;
-        const uint32_t tlane = (uint32_t)(32 * q) << 16;
-        const uint32_t arow = su32(&sm.ah[0][0]) + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
+        const uint32_t tlane = tmem + ((uint32_t)(32 * q) << 16);
+        const uint32_t tacc = tlane + 64u * grp, th = tlane + AH + 32u * grp, tm = tlane + AM + 32u * grp;
+        const uint32_t lrow = su32(&sm.al[grp][0]) + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
         const int sw = row & 7;
-        constexpr int HW = W / 2;  // columns (outputs, next-layer inputs) per thread
+        const int c0 = 64 * grp;  // this thread's first column
+        const unsigned lt = (1u << lane) - 1u;
         int cur = 0;
         const Item *it = &items[0];
         uint32_t pacc = 0;
-        for (;;) {
-            // 1. the tile: 128 rows of item cur's list (or point array)
-            if (e == 0) {
-                unsigned long long total = (unsigned long long)npts, base = 0;
-                if (MODE == XMODE_REFINE)
-                    total = (it->s.ctr->flags & STOP_FLAGS) ? 0ull : it->s.ctr->refine;
-                base = total ? atomicAdd(MODE == XMODE_REFINE ? &it->s.ctr->next_tile2 : &it->s.ctr->next_tile,
-                                         (unsigned long long)TM)
-                             : 0ull;
-                sm.base = base;
-                sm.total = total;
+        // hopping state of the row (group 0's thread)
+        uint32_t col = NONE, rank = 0;
+        int k = 0;
+        bool done = false;
+        float hx = 0.f, hy = 0.f;
+        unsigned long long evals = 0;
+        for (long long tile = blockIdx.x;; tile += gridDim.x) {
+            // 1. the rows' work, from item cur: group 0 decides and shares the points
+            unsigned long long idx = 0;
+            uint32_t vslot = 0;
+            bool live = false;
+            const GridP &g = it->g;
+            const Scratch &s = it->s;
+            const int N = g.N;
+            if (grp == 0) {
+                float px = 0.f, py = 0.f, pz = 0.f;
+                if (MODE == XM_HOP) {
+                    const uint32_t ncols = (uint32_t)N * (uint32_t)N;
+                    const bool need = col == NONE && !done;
+                    const unsigned needm = __ballot_sync(FULL, need);
+                    if (needm) {
+                        const int leader = __ffs(needm) - 1;
+                        unsigned long long base = 0;
+                        if (lane == leader) base = atomicAdd(&s.ctr->next_col, (unsigned long long)__popc(needm));
+                        base = __shfl_sync(FULL, base, leader);
+                        if (need) {
+                            const unsigned long long c = base + __popc(needm & lt);
+                            if (c < ncols) {
+                                col = column_of_claim((uint32_t)c, N);
+                                k = 0;
+                                rank = 0;
+                                const int i = (int)(col / (uint32_t)N), j = (int)(col - (uint32_t)i * N);
+                                hx = fmaf((float)i + 0.5f, g.h, g.lo[0]);
+                                hy = fmaf((float)j + 0.5f, g.h, g.lo[1]);
+                            } else {
+                                done = true;
+                            }
+                        }
+                    }
+                    live = col != NONE;
+                    if (live) {
+                        px = hx;
+                        py = hy;
+                        pz = fmaf((float)k + 0.5f, g.h, g.lo[2]);
+                    }
+                } else {
+                    unsigned long long total = (unsigned long long)npts;
+                    if (MODE == XM_LATTICE) total = (unsigned long long)(N + 1) * (N + 1) * (N + 1);
+                    if (MODE == XM_VERTS || MODE == XM_REFINE)
+                        total = (s.ctr->flags & STOP_FLAGS) ? 0ull : (MODE == XM_VERTS ? s.ctr->verts : s.ctr->refine);
+                    unsigned long long base = total;
+                    if (MODE == XM_POINTS || MODE == XM_ADJ) {  // equal tiles dealt out in turn
+                        base = (unsigned long long)tile * TM + 32 * q;
+                    } else {
+                        if (lane == 0 && !done)
+                            base = atomicAdd(MODE == XM_REFINE ? &s.ctr->next_tile2 : &s.ctr->next_tile, 32ull);
+                        base = __shfl_sync(FULL, base, 0);
+                    }
+                    idx = base + lane;
+                    live = idx < total;
+                    if (base >= total) done = true;
+                    if (live) {
+                        if (MODE == XM_POINTS || MODE == XM_ADJ) {
+                            px = pts[3 * idx];
+                            py = pts[3 * idx + 1];
+                            pz = pts[3 * idx + 2];
+                        } else if (MODE == XM_LATTICE) {
+                            const unsigned long long N1 = N + 1;
+                            const unsigned long long a = idx % N1, b = (idx / N1) % N1, c = idx / (N1 * N1);
+                            px = fmaf((float)a, g.h, g.lo[0]);
+                            py = fmaf((float)b, g.h, g.lo[1]);
+                            pz = fmaf((float)c, g.h, g.lo[2]);
+                        } else {
+                            vslot = MODE == XM_REFINE ? s.rlist[idx] : (uint32_t)idx;
+                            const unsigned long long key = s.vkey[vslot];
+                            const int N1 = N + 1;
+                            const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), c = (uint32_t)(key >> 32);
+                            const uint32_t a = line / (uint32_t)N1, b = line - a * (uint32_t)N1;
+                            px = fmaf((float)a, g.h, g.lo[0]);
+                            py = fmaf((float)b, g.h, g.lo[1]);
+                            pz = fmaf((float)c, g.h, g.lo[2]);
+                        }
+                    }
+                }
+                sm.pt[row] = make_float4(px, py, pz, live ? 1.f : 0.f);
             }
+            const bool any = bar_any(BAR_EPI, EPI, live);
             // the abort decision goes through the barrier so that it is uniform
             const bool abort = bar_any(BAR_EPI, EPI, (*ctl & CTL_ABORT) != 0);
-            const unsigned long long base = sm.base, total = sm.total;
-            if (abort || base >= total) {
+            if (abort || !any) {
+                if (MODE == XM_HOP && grp == 0) {
+                    for (int o = 16; o > 0; o >>= 1) evals += __shfl_xor_sync(FULL, evals, o);
+                    if (lane == 0 && evals) atomicAdd(&s.ctr->hop_evals, evals);
+                    evals = 0;
+                }
                 if (!abort && cur + 1 < n_items) {
                     // item cur has no rows left for this CTA: the next item
                     ++cur;
                     it = &items[cur];
+                    col = NONE;
+                    done = false;
                     load_params<W>(sm, it->m, e);
                     bar_sync(BAR_EPI, EPI);
                     continue;
@@ -264,121 +472,217 @@ __global__ void __launch_bounds__(384, 1)
                     __threadfence_block();
                     mbar_arrive(&sm.item_ready);
                 }
-                mbar_arrive(&sm.a_full);  // the final phase: the MMA sees done
+                mbar_arrive(&sm.a_h);  // the final phase: the MMA sees done
                 break;
             }
             if (e == 0) {
                 sm.cur_w = it->m.wx6;
                 mbar_arrive(&sm.item_ready);
+                if (MODE == XM_HOP) atomicAdd(&s.ctr->row_slots, (unsigned long long)TM);
             }
             const MlpDev &m = it->m;
-            const GridP &g = it->g;
-            const unsigned long long idx = base + (unsigned long long)row;
-            const bool live = idx < total;
-            float px = 0.f, py = 0.f, pz = 0.f;
-            uint32_t vslot = 0;
-            if (live) {
-                if (MODE == XMODE_POINTS) {
-                    px = pts[3 * idx];
-                    py = pts[3 * idx + 1];
-                    pz = pts[3 * idx + 2];
-                } else {
-                    vslot = it->s.rlist[idx];
-                    const unsigned long long key = it->s.vkey[vslot];
-                    const int N1 = g.N + 1;
-                    const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), c = (uint32_t)(key >> 32);
-                    const uint32_t a = line / (uint32_t)N1, b = line - a * (uint32_t)N1;
-                    px = fmaf((float)a, g.h, g.lo[0]);
-                    py = fmaf((float)b, g.h, g.lo[1]);
-                    pz = fmaf((float)c, g.h, g.lo[2]);
-                }
-            }
+            const float4 pt = sm.pt[row];
+            const bool rlive = pt.w != 0.f;
+            // adjoint: this thread's piece of row tile * 128 + row of the chunk's arrays
+            const long long arows = (npts + TM - 1) / TM * TM, arow_i = tile * TM + row;
+            const size_t aoff = MODE == XM_ADJ ? (size_t)arow_i * W + c0 : 0;
+            const size_t moff = MODE == XM_ADJ ? (size_t)arow_i * G + grp : 0;
+            constexpr bool RELU_CVT = MODE != XM_ADJ;  // x holds z; the adjoint keeps relu(z), which it also stores
+            float x[64];
             // 2. layer 0 in FP32 (the FP32 engine's operation order), split -> A operands
-            __syncwarp();  // tcgen05.st below needs the whole warp converged
             {
-                const unsigned long long ppx = pack2(px, px), ppy = pack2(py, py), ppz = pack2(pz, pz);
-#pragma unroll 1
-                for (int j = 0; j < HW / 32; ++j) {
-                    const int c0 = hf * HW + 32 * j;  // first output of this 32-output chunk
-                    uint32_t mh[16], ml[16], hh[16];
+                const unsigned long long ppx = pack2(pt.x, pt.x), ppy = pack2(pt.y, pt.y), ppz = pack2(pt.z, pt.z);
 #pragma unroll
-                    for (int p = 0; p < 16; ++p) {
-                        const float4 wa = sm.w0b[c0 + 2 * p], wb = sm.w0b[c0 + 2 * p + 1];
-                        const unsigned long long z = ffma2(pack2(wa.x, wa.y), ppx,
-                                                           ffma2(pack2(wa.z, wa.w), ppy,
-                                                                 ffma2(pack2(wb.x, wb.y), ppz, pack2(wb.z, wb.w))));
-                        split3(fmaxf(lo2(z), 0.f), fmaxf(hi2(z), 0.f), hh[p], mh[p], ml[p]);
-                    }
-                    const int kb = c0 >> 6, cc = (c0 & 63) >> 3;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        sts128(arow + kb * (TM * 128) + (((cc + u) ^ sw) << 4), hh[4 * u], hh[4 * u + 1],
-                               hh[4 * u + 2], hh[4 * u + 3]);
-                    tmem_st16(tmem + tlane + AM + (uint32_t)(c0 / 2), mh);
-                    tmem_st16(tmem + tlane + AL + (uint32_t)(c0 / 2), ml);
+                for (int p = 0; p < 32; ++p) {
+                    const float4 wa = sm.w0b[c0 + 2 * p], wb = sm.w0b[c0 + 2 * p + 1];
+                    const unsigned long long z = ffma2(pack2(wa.x, wa.y), ppx,
+                                                       ffma2(pack2(wa.z, wa.w), ppy,
+                                                             ffma2(pack2(wb.x, wb.y), ppz, pack2(wb.z, wb.w))));
+                    x[2 * p] = RELU_CVT ? lo2(z) : fmaxf(lo2(z), 0.f);
+                    x[2 * p + 1] = RELU_CVT ? hi2(z) : fmaxf(hi2(z), 0.f);
                 }
-                tmem_wait_st();
-                tc_fence_before();
-                fence_async_smem();
-                mbar_arrive(&sm.a_full);
             }
-            // 3. hidden layers: accumulator -> bias, ReLU -> split -> next A operands,
-            //    and after the last one the output dot product
-            float gs = 0.f;
-            for (int l = 0; l < n_mid; ++l) {
+            __syncwarp();  // tcgen05.st below needs the whole warp converged
+            if (MODE == XM_ADJ) {
+                if (rlive) store_row(adj.A + aoff, x);
+                adj.mask[moff] = relu_bits(x);
+            }
+            put_h<RELU_CVT>(x, th);
+            tc_fence_before();
+            mbar_arrive(&sm.a_h);
+            put_ml<RELU_CVT>(x, tm, lrow, sw);
+            tc_fence_before();
+            fence_async_smem();
+            mbar_arrive(&sm.a_ml);
+            // 3. the products' results, layer by layer -> the next A operands, and at
+            //    the end the output dot product (adjoint: grad_x g)
+            constexpr float KAPPA = kappa_of<W>();
+            const unsigned long long KK = pack2(KAPPA, KAPPA);
+            float gs[3] = {0.f, 0.f, 0.f};
+            for (int l = 0; l < n_gemm; ++l) {
+                const bool back = MODE == XM_ADJ && l >= n_mid;
+                uint2 mk = make_uint2(0u, 0u);
+                if (back) mk = adj.mask[(size_t)(2 * n_mid - 1 - l) * arows * G + moff];
                 wait_bar(&sm.acc_full, pacc, ctl, CTL_ABORT, ctr0, wait_ns);
                 pacc ^= 1u;
                 __syncwarp();  // tcgen05.ld below needs the whole warp converged
                 tc_fence_after();
-                const float *bl = sm.bmid + l * W;
-                const bool last = l + 1 == n_mid;
-#pragma unroll 1
-                for (int j = 0; j < HW / 32; ++j) {
-                    const int c0 = hf * HW + 32 * j;
-                    uint32_t acc[32];
-                    tmem_ld32_async(tmem + tlane + (uint32_t)c0, acc);
+                {
+                    uint32_t lo[32], hi[32];
+                    tmem_ld32_async(tacc, lo);
+                    tmem_ld32_async(tacc + 32, hi);
                     tmem_wait_ld();
-                    if (!last) {
-                        uint32_t mh[16], ml[16], hh[16];
 #pragma unroll
-                        for (int p = 0; p < 16; ++p) {
-                            const float2 b = *reinterpret_cast<const float2 *>(bl + c0 + 2 * p);
-                            split3(fmaxf(__uint_as_float(acc[2 * p]) + b.x, 0.f),
-                                   fmaxf(__uint_as_float(acc[2 * p + 1]) + b.y, 0.f), hh[p], mh[p], ml[p]);
-                        }
-                        const int kb = c0 >> 6, cc = (c0 & 63) >> 3;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            sts128(arow + kb * (TM * 128) + (((cc + u) ^ sw) << 4), hh[4 * u], hh[4 * u + 1],
-                                   hh[4 * u + 2], hh[4 * u + 3]);
-                        tmem_st16(tmem + tlane + AM + (uint32_t)(c0 / 2), mh);
-                        tmem_st16(tmem + tlane + AL + (uint32_t)(c0 / 2), ml);
-                    } else {
-#pragma unroll
-                        for (int p = 0; p < 32; ++p)
-                            gs = fmaf(sm.wout[c0 + p], fmaxf(__uint_as_float(acc[p]) + bl[c0 + p], 0.f), gs);
+                    for (int c = 0; c < 32; ++c) {
+                        x[c] = __uint_as_float(lo[c]);
+                        x[32 + c] = __uint_as_float(hi[c]);
                     }
                 }
-                if (!last) {
-                    tmem_wait_st();
+                if (!back) {
+                    const float4 *bl = reinterpret_cast<const float4 *>(sm.bmid + l * W + c0);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const float4 b = bl[c];
+                        // z = acc + (b + KAPPA 2^e(acc)): one rounding at the size of z
+                        const unsigned long long z0 =
+                            fadd2(pack2(x[4 * c], x[4 * c + 1]),
+                                  ffma2(pack2(pow2_of(x[4 * c]), pow2_of(x[4 * c + 1])), KK, pack2(b.x, b.y)));
+                        const unsigned long long z1 =
+                            fadd2(pack2(x[4 * c + 2], x[4 * c + 3]),
+                                  ffma2(pack2(pow2_of(x[4 * c + 2]), pow2_of(x[4 * c + 3])), KK, pack2(b.z, b.w)));
+                        x[4 * c] = RELU_CVT ? lo2(z0) : fmaxf(lo2(z0), 0.f);
+                        x[4 * c + 1] = RELU_CVT ? hi2(z0) : fmaxf(hi2(z0), 0.f);
+                        x[4 * c + 2] = RELU_CVT ? lo2(z1) : fmaxf(lo2(z1), 0.f);
+                        x[4 * c + 3] = RELU_CVT ? hi2(z1) : fmaxf(hi2(z1), 0.f);
+                    }
+                    if (MODE == XM_ADJ) {
+                        if (rlive) store_row(adj.A + (size_t)(l + 1) * adj.ldl + aoff, x);
+                        const uint2 bits = relu_bits(x);
+                        if (l + 1 < n_mid) {
+                            adj.mask[(size_t)(l + 1) * arows * G + moff] = bits;
+                        } else {  // the top: delta_L = w_out [z_L > 0]
+#pragma unroll
+                            for (int c = 0; c < 64; ++c)
+                                x[c] = ((c < 32 ? bits.x : bits.y) >> (c & 31)) & 1u ? sm.wout[c0 + c] : 0.f;
+                            if (rlive) store_row(adj.D + (size_t)n_mid * adj.ldl + aoff, x);
+                        }
+                    }
+                } else {  // delta_{l'} = (W^T delta) [z_{l'} > 0], l' = 2 n_mid - 1 - l
+#pragma unroll
+                    for (int c = 0; c < 64; ++c)
+                        x[c] = ((c < 32 ? mk.x : mk.y) >> (c & 31)) & 1u ? fmaf(pow2_of(x[c]), KAPPA, x[c]) : 0.f;
+                    if (rlive) store_row(adj.D + (size_t)(2 * n_mid - 1 - l) * adj.ldl + aoff, x);
+                }
+                if (l + 1 < n_gemm) {
+                    put_h<RELU_CVT>(x, th);
+                    tc_fence_before();
+                    mbar_arrive(&sm.a_h);
+                    put_ml<RELU_CVT>(x, tm, lrow, sw);
                     tc_fence_before();
                     fence_async_smem();
-                    mbar_arrive(&sm.a_full);
+                    mbar_arrive(&sm.a_ml);
                 } else {
                     tc_fence_before();
+                    if (MODE == XM_ADJ) {
+#pragma unroll
+                        for (int p = 0; p < 32; ++p) {
+                            const float4 wa = sm.w0b[c0 + 2 * p], wb = sm.w0b[c0 + 2 * p + 1];
+                            gs[0] = fmaf(wa.y, x[2 * p + 1], fmaf(wa.x, x[2 * p], gs[0]));
+                            gs[1] = fmaf(wa.w, x[2 * p + 1], fmaf(wa.z, x[2 * p], gs[1]));
+                            gs[2] = fmaf(wb.y, x[2 * p + 1], fmaf(wb.x, x[2 * p], gs[2]));
+                        }
+                    } else {
+                        // eight sums of every eighth column: the roundings of one long
+                        // chain would be the largest error of a narrow network
+                        const float4 *wp = reinterpret_cast<const float4 *>(sm.wout + c0);
+                        float d[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            const float4 w = wp[c];
+                            d[4 * (c & 1)] = fmaf(w.x, relu_nan(x[4 * c]), d[4 * (c & 1)]);
+                            d[4 * (c & 1) + 1] = fmaf(w.y, relu_nan(x[4 * c + 1]), d[4 * (c & 1) + 1]);
+                            d[4 * (c & 1) + 2] = fmaf(w.z, relu_nan(x[4 * c + 2]), d[4 * (c & 1) + 2]);
+                            d[4 * (c & 1) + 3] = fmaf(w.w, relu_nan(x[4 * c + 3]), d[4 * (c & 1) + 3]);
+                        }
+                        gs[0] = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7]));
+                    }
                 }
             }
-            // 4. f = outer(g): the two halves' sums as the FP32 engine adds them
-            sm.red[hf][row] = gs;
+            // 4. the groups' sums in order, then f and the hop step or the store
+            for (int a = 0; a < (MODE == XM_ADJ ? 3 : 1); ++a) sm.red[a][grp][row] = gs[a];
             bar_sync(BAR_EPI, EPI);
-            if (hf == 0 && live) {
-                const float g = sm.red[0][row] + sm.red[1][row] + m.bout;
-                const float f = outer_f(m, px, py, pz, g);
-                if (MODE == XMODE_REFINE) {
-                    if (!isfinite(f)) atomicOr(&it->s.ctr->flags, FLAG_NONFINITE);
-                    it->s.vval[vslot] = f;
-                } else {
+            if (grp != 0) continue;
+            float tot[3] = {0.f, 0.f, 0.f};
+            for (int a = 0; a < (MODE == XM_ADJ ? 3 : 1); ++a) {
+                tot[a] = sm.red[a][0][row];
+                for (int u = 1; u < G; ++u) tot[a] += sm.red[a][u][row];
+            }
+            if (MODE == XM_ADJ) {
+                if (rlive) {
+                    // s_v = -(dL/dv . grad_x f) / |grad_x f|^2
+                    const float r = sqrtf(pt.x * pt.x + pt.y * pt.y + pt.z * pt.z);
+                    const float ir = r > 0.f ? m.radial / r : 0.f, ibl = 1.f / m.beta * m.inv_lam;
+                    const float fx = (pt.x * ir + m.alpha * tot[0]) * ibl;
+                    const float fy = (pt.y * ir + m.alpha * tot[1]) * ibl;
+                    const float fz = (pt.z * ir + m.alpha * tot[2]) * ibl;
+                    const float n2 = fx * fx + fy * fy + fz * fz;
+                    const float dot = adj.dL[3 * arow_i] * fx + adj.dL[3 * arow_i + 1] * fy + adj.dL[3 * arow_i + 2] * fz;
+                    adj.s[arow_i] = n2 > 0.f ? -dot / n2 : 0.f;
+                }
+                continue;
+            }
+            const float f = outer_f(m, pt.x, pt.y, pt.z, tot[0] + m.bout);
+            if (MODE == XM_HOP) {
+                bool mark = false, empty = false;
+                int step = 1;
+                if (live) {
+                    ++evals;
+                    float d = fabsf(f) - g.eps;
+                    if (!isfinite(f)) {
+                        atomicOr(&s.ctr->flags, FLAG_NONFINITE);
+                        d = 0.f;
+                    }
+                    if (d <= g.tau) {
+                        mark = true;
+                        empty = cell_is_empty(g, d, pt.x, pt.y, pt.z);
+                    } else {
+                        const float stp = floorf(d * g.inv_h);
+                        step = stp < 1.f ? 1 : (stp > (float)N ? N : (int)stp);
+                    }
+                }
+                const unsigned mm = __ballot_sync(FULL, mark);
+                if (mm) {
+                    const int leader = __ffs(mm) - 1;
+                    unsigned long long base = 0;
+                    if (lane == leader) base = atomicAdd(&s.ctr->marks, (unsigned long long)__popc(mm));
+                    base = __shfl_sync(FULL, base, leader);
+                    if (mark) {
+                        const unsigned long long mi = base + __popc(mm & lt);
+                        if (mi < (unsigned long long)s.cap_marks)
+                            s.marks_raw[mi] = pack_mark(col, (uint32_t)k, rank, empty);
+                        else
+                            atomicOr(&s.ctr->flags, FLAG_MARK_OVERFLOW);
+                    }
+                }
+                if (live) {
+                    if (mark) {
+                        ++rank;
+                        ++k;
+                    } else {
+                        k += step;
+                    }
+                    if (k >= N) {
+                        s.colcount[col] = rank;
+                        col = NONE;
+                    }
+                }
+            } else if (live) {
+                if (MODE == XM_POINTS) {
                     outv[idx] = f;
+                } else {
+                    if (!isfinite(f)) atomicOr(&s.ctr->flags, FLAG_NONFINITE);
+                    if (MODE == XM_LATTICE) s.lat[idx] = f;
+                    else s.vval[vslot] = f;
                 }
             }
         }
@@ -392,15 +696,16 @@ __global__ void __launch_bounds__(384, 1)
 }
 
 template <int W, int MODE>
-void launch_x6(const Item *items, int n_items, const float *p, long long n, float *out, int nsm, cudaStream_t st) {
+void launch_x6(const Item *items, int n_items, const Item &single, const float *p, long long n, float *out,
+               const AdjOut &adj, int nsm, cudaStream_t st) {
     const size_t smem = sizeof(SmemX<W>) + 1024;
     cudaFuncSetAttribute(k_mlp_x6<W, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int grid = nsm;
-    if (MODE == XMODE_POINTS) {
+    int grid = nsm * ctas_of<W>();
+    if (MODE == XM_POINTS || MODE == XM_ADJ) {
         const long long tiles = (n + TM - 1) / TM;
         if (grid > tiles) grid = (int)(tiles < 1 ? 1 : tiles);
     }
-    k_mlp_x6<W, MODE><<<grid, 384, smem, st>>>(items, n_items, p, n, out, wait_limit_ns());
+    k_mlp_x6<W, MODE><<<grid, EPI_T0 + 2 * W, smem, st>>>(items, n_items, single, p, n, out, adj, wait_limit_ns());
 }
 
 }  // namespace
@@ -414,23 +719,45 @@ void launch_x6(const Item *items, int n_items, const float *p, long long n, floa
 
 int x6_max_mid() { return MAXMID; }
 
-void launch_refine_mlp_x6(const Item *items, int n_items, int width, int nsm, cudaStream_t st) {
-    GH_X6_W(width, (launch_x6<WW, XMODE_REFINE>(items, n_items, nullptr, 0, nullptr, nsm, st)))
+void launch_hop_mlp_x6(const Item *items, int n_items, int width, int nsm, cudaStream_t st) {
+    GH_X6_W(width, (launch_x6<WW, XM_HOP>(items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
 }
 
-void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, float *out, int nsm, cudaStream_t st) {
-    // one item whose counters live in a small private buffer
+void launch_eval_vertices_mlp_x6(const Item *items, int n_items, int width, int nsm, bool refine_list,
+                                 cudaStream_t st) {
+    if (refine_list) {
+        GH_X6_W(width, (launch_x6<WW, XM_REFINE>(items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+    } else {
+        GH_X6_W(width, (launch_x6<WW, XM_VERTS>(items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+    }
+}
+
+void launch_lattice_mlp_x6(const Item *items, int width, int nsm, cudaStream_t st) {
+    GH_X6_W(width, (launch_x6<WW, XM_LATTICE>(items, 1, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+}
+
+// A network's descriptor for the kernels that take points instead of an item
+// (its counters only carry the error flag of a timeout, which nothing reads).
+static Item points_item(const MlpDev &m) {
     static thread_local Counters *ctr = nullptr;
-    static thread_local Item *ditem = nullptr;
     if (!ctr) cudaMalloc(&ctr, sizeof(Counters));
-    if (!ditem) cudaMalloc(&ditem, sizeof(Item));
     Item h{};
     h.m = m;
     h.s.ctr = ctr;
     h.kind = 1;
-    cudaMemsetAsync(ctr, 0, sizeof(Counters), st);
-    cudaMemcpyAsync(ditem, &h, sizeof(Item), cudaMemcpyHostToDevice, st);
-    GH_X6_W(m.width, (launch_x6<WW, XMODE_POINTS>(ditem, 1, p, n, out, nsm, st)))
+    return h;
+}
+
+void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, float *out, int nsm, cudaStream_t st) {
+    const Item it = points_item(m);
+    GH_X6_W(m.width, (launch_x6<WW, XM_POINTS>(nullptr, 1, it, p, n, out, AdjOut{}, nsm, st)))
+}
+
+void launch_adj_mlp_x6(const MlpDev &m, const float *P, const float *dL, long long V, float *A, float *D, float *s,
+                       uint32_t *mask, long long ldl, int nsm, cudaStream_t st) {
+    const Item it = points_item(m);
+    const AdjOut a{dL, A, D, s, reinterpret_cast<uint2 *>(mask), ldl, m.wx6t};
+    GH_X6_W(m.width, (launch_x6<WW, XM_ADJ>(nullptr, 1, it, P, V, nullptr, a, nsm, st)))
 }
 
 }  // namespace gh

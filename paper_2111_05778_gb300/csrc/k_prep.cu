@@ -15,6 +15,8 @@
 //       w = w_h + w_m + w_l exactly (w_h = bf16(w), w_m = bf16(w - w_h),
 //       w_l = bf16(w - w_h - w_m)), stored part by part (low, middle, high),
 //       each part in wbf's layout;
+//   wx6t the same of the transposed weights (rows = inputs of the layer, K =
+//       its outputs), layer n_mid first (the adjoint walks down);
 //   bm  hidden biases, n_mid x [W].
 #include "gh_internal.cuh"
 
@@ -37,7 +39,7 @@ __device__ __forceinline__ float bf16_val(uint16_t b) { return __uint_as_float((
 __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ params, int W, int n_mid,
                                                   float *__restrict__ wt, float *__restrict__ wtb,
                                                   uint16_t *__restrict__ wbf, uint16_t *__restrict__ wx6,
-                                                  float *__restrict__ bm) {
+                                                  uint16_t *__restrict__ wx6t, float *__restrict__ bm) {
     const long long WW = (long long)W * W, total = (long long)n_mid * WW;
     const long long mid0 = 4LL * W;  // W0 and b0 come first
     const int KB = W / 64;
@@ -57,8 +59,12 @@ __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ para
         const uint16_t mid = bf16_rne(rem);
         const uint16_t low = bf16_rne(rem - bf16_val(mid));
         const uint16_t parts[3] = {low, mid, hi};
-        for (int p = 0; p < 3; ++p)
+        const int kt = o >> 6, ko = o & 63;
+        const int bytet = (i >> 3) * 1024 + (i & 7) * 128 + (((ko >> 3) ^ (i & 7)) << 4) + (ko & 7) * 2;
+        for (int p = 0; p < 3; ++p) {
             wx6[(((long long)l * 3 + p) * KB + kb) * W * 64 + byte / 2] = parts[p];
+            wx6t[(((long long)(n_mid - 1 - l) * 3 + p) * KB + kt) * W * 64 + bytet / 2] = parts[p];
+        }
     }
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)n_mid * W;
          e += (long long)gridDim.x * blockDim.x) {
@@ -70,8 +76,8 @@ __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ para
 }  // namespace
 
 void launch_prep_mlp(const float *params, int W, int n_mid, float *wt, float *wtb, uint16_t *wbf, uint16_t *wx6,
-                     float *bm, cudaStream_t st) {
-    k_prep_mlp<<<1024, 256, 0, st>>>(params, W, n_mid, wt, wtb, wbf, wx6, bm);
+                     uint16_t *wx6t, float *bm, cudaStream_t st) {
+    k_prep_mlp<<<1024, 256, 0, st>>>(params, W, n_mid, wt, wtb, wbf, wx6, wx6t, bm);
 }
 
 }  // namespace gh
