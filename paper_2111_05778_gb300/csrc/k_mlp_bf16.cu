@@ -12,19 +12,25 @@
 // every hidden activation.  The output layer (W -> 1) runs on CUDA cores in
 // FP32.
 //
-// One persistent CTA per SM, 384 threads:
+// One persistent CTA per SM, 64 threads + 128 or 256 per tile:
 //   warp 0       TMA producer: 1-D bulk copies (cp.async.bulk) of BF16 weight
 //                K-blocks, stored pre-swizzled in global memory, into a
-//                2-stage shared-memory ring (mbarrier complete_tx).
+//                shared-memory ring (mbarrier complete_tx).
 //   warp 1       allocates TMEM; one lane issues tcgen05.mma for two 128-row
 //                tiles per weight K-block (M = 128, N = W, K = 16 per op) and
 //                tcgen05.commit's to the ring's "empty" barriers and to the
 //                accumulator barrier.
-//   warps 4..11  epilogue, one row (one ray or one point) per thread: layer 0,
-//                TMEM -> registers (tcgen05.ld) -> bias, ReLU, BF16 -> the next
-//                layer's A operand in 128B-swizzled K-major shared memory,
-//                the FP32 output dot product, and the grid-hopping step of
-//                Algorithm 1 (with the eps shrink) or the store of f.
+//   warps 2..    epilogue, one or two threads per row with all or half of the
+//                columns each: TMEM -> registers (tcgen05.ld) -> bias, ReLU,
+//                BF16 -> the next layer's A operand in 128B-swizzled K-major
+//                shared memory, and the FP32 output dot product.  The first
+//                thread owns the row (one ray or one point): the layer-0
+//                operand, the grid-hopping step of Algorithm 1 (with the eps
+//                shrink) or the store of f.
+// What bounds it at width 256 is the SM's shared-memory port: per tile and
+// layer 192 KB of operand reads, 64 or 128 KB of weights and 64 KB of
+// activations written and 32 KB of biases read are about 3,000 cycles at 128
+// bytes a cycle, against 2,048 of the products; a phase takes 3,200.
 // Every wait is bounded (2 s of %globaltimer); a timeout sets an error flag,
 // makes all roles leave their loops, drains the copies in flight, and frees
 // TMEM before the kernel returns.
@@ -39,9 +45,8 @@ namespace {
 
 using namespace tc;
 
-constexpr int EPI_T0 = 128;  // first epilogue thread (warp 4)
+constexpr int EPI_T0 = 64;   // first epilogue thread (warp 2)
 constexpr int TM = 128;      // rows per tile
-constexpr int NSTAGE = 2;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
@@ -55,36 +60,46 @@ constexpr int maxmid_of() {
     return W == 256 ? 7 : 8;
 }
 
+// Threads per row of a tile.  At width 256 one thread would convert 256
+// columns per layer, longer than the other tile's products take; at width 64
+// a second thread only adds barrier arrivals (2^20 points 191 us with one, 194
+// with two).
+template <int W>
+constexpr int halves_of() {
+    return W == 64 ? 1 : 2;
+}
+
+// Weight ring: stages of KS inputs x W outputs.  Width 256 has room for 64 KB
+// beside the two A operands: four stages of 32 inputs, each refilled after its
+// two products (256 cycles); with two stages of 64 inputs the products waited
+// about 1,100 of 3,300 cycles per layer for the refill (hop at N = 1024 10.6
+// -> 10.2 ms).  The narrower widths hold two whole layers in stages of 64.
+template <int W>
+constexpr int ks_of() {
+    return W == 256 ? 32 : 64;
+}
+template <int W>
+constexpr int nslot_of() {
+    return W == 256 ? 4 : W / 32;
+}
+
 template <int W>
 struct SmemB {
+    static constexpr int NSLOT = nslot_of<W>();
     uint8_t a[2][W / 64][TM * 128];  // A operands: one per tile, K-blocks of 128 rows x 128 B (1024-aligned)
-    uint8_t w[NSTAGE][W * 128];      // weight ring: one K-block of W rows x 128 B per stage
+    uint8_t w[NSLOT][W * 2 * ks_of<W>()];  // weight ring: one K-block of W rows x KS inputs per stage
     uint8_t b0[2][W * 32];           // per tile: layer-0 operand B0 of its current item, W rows x 16 inputs
                                      // (32-byte swizzle: row n, 16-byte chunk c at (n/8)*256 + (n%8)*32 +
                                      // ((c ^ (n/4)%2) * 16))
     float bmid[2][maxmid_of<W>() * W];  // per tile: hidden-layer biases
-    float zb[W];                        // zeros: the layer-0 phase adds no bias (B0 holds it)
+    float red[2][TM];                // per tile: the second halves' output dot products
     float wout[2][W];                // per tile: output-layer weights
-    unsigned long long full[NSTAGE], empty[NSTAGE], acc_full[2], a_full[2], item_ready[2], drain;
+    unsigned long long full[NSLOT], empty[NSLOT], acc_full[2], a_full[2], item_ready[2], drain;
     const uint16_t *cur_wbf[2];      // per tile: weights of its current item
     int done[2];                     // per tile: no more work
     uint32_t tmem_base;
     int ctl;
 };
-
-// OR-reduction over the 128 epilogue threads of one tile (named barrier id).
-__device__ __forceinline__ bool epi_any(int id, bool v) {
-    uint32_t out;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, 128, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(out)
-        : "r"((uint32_t)v), "r"(id)
-        : "memory");
-    return out != 0;
-}
 
 __device__ __forceinline__ float outer_f(const MlpDev &m, float x, float y, float z, float g) {
     const float r = sqrtf(fmaf(x, x, fmaf(y, y, z * z)));
@@ -115,8 +130,8 @@ __device__ __forceinline__ void put_b0(SmemB<W> &sm, int t, int o, float wx, flo
     sts128(base + ((1u ^ sw) << 4), zl | (bh << 16), bl, 0u, 0u);
 }
 
-// Item parameters of tile t (its 128 epilogue threads, or all threads at
-// set-up with e and the stride given): B0, hidden biases, output weights.
+// Item parameters of tile t (its epilogue threads, or all threads at set-up
+// with e and the stride given): B0, hidden biases, output weights.
 template <int W>
 __device__ __forceinline__ void load_item(SmemB<W> &sm, int t, const MlpDev &mm, int e, int stride) {
     for (int o = e; o < W; o += stride) {
@@ -137,13 +152,15 @@ __device__ __forceinline__ void load_item(SmemB<W> &sm, int t, const MlpDev &mm,
 // biases and output weights; the producer streams the weights of whichever
 // item the phase's tile is on.
 template <int W, int MODE, int TILES>
-__global__ void __launch_bounds__(128 + 128 * TILES, 1)
+__global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W>() * TILES, 1)
     k_mlp_bf16(const Item *__restrict__ items, int n_items, const float *__restrict__ pts, long long npts,
                float *__restrict__ outv, unsigned long long wait_ns) {
     extern __shared__ uint8_t smem_raw[];
-    constexpr int KB = W / 64;
-    constexpr int RS = KB < NSTAGE ? KB : NSTAGE;  // K-blocks a phase can take over from the one before
-    constexpr uint32_t STAGE_BYTES = W * 128;
+    constexpr int HALVES = halves_of<W>(), ET = TM * HALVES;  // epilogue threads per row, per tile
+    constexpr int KS = ks_of<W>(), KB = W / KS;  // K-blocks per hidden layer
+    constexpr int NSLOT = nslot_of<W>();
+    constexpr int RS = KB < NSLOT ? KB : NSLOT;  // K-blocks a phase can take over from the one before
+    constexpr uint32_t STAGE_BYTES = W * 2 * KS;
     constexpr uint32_t TMEM_COLS = TILES * W < 32 ? 32 : TILES * W;
     constexpr uint32_t IDESC = idesc_bf16(TM, W);
     SmemB<W> &sm = *reinterpret_cast<SmemB<W> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
@@ -154,15 +171,14 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
 
     // ---- set-up ----------------------------------------------------------
     for (int t = 0; t < TILES; ++t) load_item<W>(sm, t, items[0].m, tid, blockDim.x);
-    for (int i = tid; i < W; i += blockDim.x) sm.zb[i] = 0.f;
     if (tid == 0) {
-        for (int i = 0; i < NSTAGE; ++i) {
+        for (int i = 0; i < NSLOT; ++i) {
             mbar_init(&sm.full[i], 1);
             mbar_init(&sm.empty[i], 1);
         }
         for (int t = 0; t < 2; ++t) {
             mbar_init(&sm.acc_full[t], 1);
-            mbar_init(&sm.a_full[t], 128);
+            mbar_init(&sm.a_full[t], ET);
             mbar_init(&sm.item_ready[t], 1);
             sm.cur_wbf[t] = items[0].m.wbf;
             sm.done[t] = t < TILES ? 0 : 1;
@@ -186,7 +202,7 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
     if (warp == 0) {
         // ---- TMA producer: the phases in the MMA's order ----------------------
         if (lane == 0) {
-            long long issued = 0;
+            uint32_t issued = 0;
             int t = 0, lt[2] = {0, 0};
             bool fin[2] = {false, TILES < 2};
             uint32_t pir[2] = {0u, 0u};
@@ -219,9 +235,9 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                 keep = !reuse && !fin[t ^ 1] && lt[t ^ 1] == lt[t] && src[t ^ 1] == src[t];
                 for (int i = reuse ? RS : 0; i < KB; ++i) {
                     const int kb = reuse ? i - RS : i;
-                    const int st = (int)(issued % NSTAGE);
-                    const uint32_t par = (uint32_t)(((issued / NSTAGE) & 1) ^ 1);
-                    if (!wait_bar(&sm.empty[st], par, ctl, CTL_ABORT, ctr0, wait_ns)) {
+                    const uint32_t st = issued % NSLOT, par = ((issued / NSLOT) & 1) ^ 1;
+                    if (!mbar_try(&sm.empty[st], par) &&
+                        !wait_bar(&sm.empty[st], par, ctl, CTL_ABORT, ctr0, wait_ns)) {
                         go = false;
                         break;
                     }
@@ -234,10 +250,8 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                 if (!fin[t ^ 1]) t ^= 1;
             }
             // the copies still in flight land before the CTA may exit
-            for (long long i = issued - NSTAGE; i < issued; ++i) {
-                if (i < 0) continue;
-                wait_bar(&sm.full[i % NSTAGE], (uint32_t)((i / NSTAGE) & 1), ctl, 0, ctr0);
-            }
+            for (uint32_t i = issued < NSLOT ? 0 : issued - NSLOT; i < issued; ++i)
+                wait_bar(&sm.full[i % NSLOT], (i / NSLOT) & 1, ctl, 0, ctr0);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -249,13 +263,14 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
         // units apart, K = 16 is 2 units), a stage that has landed is taken
         // without a call, and the per-tile state lives in scalars.
         if (lane == 0) {
-            long long consumed = 0;
             int t = 0, lt0 = 0, lt1 = 0;
             bool fin0 = false, fin1 = TILES < 2;
             uint32_t pa0 = 0u, pa1 = 0u;
+            uint32_t pf = 0u;  // ring: phase of the next stage to land
+            int sb = 0;        // and, where the ring holds two layers, its index
             constexpr unsigned long long A_KB = (TM * 128) >> 4, W_ST = STAGE_BYTES >> 4;
             const unsigned long long ad0 = sdesc(su32(&sm.a[0][0][0])), ad1 = sdesc(su32(&sm.a[1][0][0]));
-            const unsigned long long wd0 = sdesc(su32(sm.w[0]));
+            const unsigned long long wd0 = KS == 32 ? sdesc64(su32(sm.w[0])) : sdesc(su32(sm.w[0]));
             const unsigned long long bd0 = sdesc32(su32(sm.b0[0])), bd1 = sdesc32(su32(sm.b0[1]));
             const uint16_t *w0 = nullptr, *w1 = nullptr;  // per tile: weights of its current item
             bool go = true, keep = false;
@@ -293,30 +308,43 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                     // the ring) come first, then the K-blocks streamed for this phase
                     const bool reuse = keep;
                     keep = !reuse && !(t ? fin0 : fin1) && (t ? lt0 : lt1) == L && (t ? w0 : w1) == (t ? w1 : w0);
-                    for (int i = 0; i < KB; ++i) {
-                        int kb, st;
-                        if (reuse && i < RS) {
-                            kb = KB - RS + i;
-                            st = (int)((consumed - RS + i) % NSTAGE);
-                        } else {
-                            kb = reuse ? i - RS : i;
-                            st = (int)(consumed % NSTAGE);
-                            const uint32_t par = (uint32_t)((consumed / NSTAGE) & 1);
-                            if (!mbar_try(&sm.full[st], par) &&
-                                !wait_bar(&sm.full[st], par, ctl, CTL_ABORT, ctr0, wait_ns)) {
-                                go = false;
-                                break;
-                            }
-                            ++consumed;
-                        }
-                        const unsigned long long a = ad + (unsigned long long)kb * A_KB;
+                    // Every phase streams a multiple of the ring's stages (width 256: 8
+                    // or 4 of 4) or half of them (one layer, or nothing), so K-blocks
+                    // fall on fixed stages and the code is straight-line.  Working the
+                    // stage and its phase out per K-block cost this thread about 400
+                    // cycles of the 512 that four products take.
+                    auto group = [&](int st, int kb, bool first, bool landed, bool release) {
+                        if (!landed && go && !mbar_try(&sm.full[st], pf) &&
+                            !wait_bar(&sm.full[st], pf, ctl, CTL_ABORT, ctr0, wait_ns))
+                            go = false;
+                        if (!go) return;
+                        const unsigned long long a =
+                            ad + (KS == 32 ? (unsigned long long)(kb >> 1) * A_KB + 4 * (kb & 1) : kb * A_KB);
                         const unsigned long long b = wd0 + (unsigned long long)st * W_ST;
-                        umma(d, a, b, IDESC, i != 0);
-                        umma(d, a + 2, b + 2, IDESC, 1u);
-                        umma(d, a + 4, b + 4, IDESC, 1u);
-                        umma(d, a + 6, b + 6, IDESC, 1u);
-                        // a kept stage is released by the next phase, after its own use
-                        if (!(keep && i >= KB - RS)) umma_commit(&sm.empty[st]);
+#pragma unroll
+                        for (int q = 0; q < KS / 16; ++q) umma(d, a + 2 * q, b + 2 * q, IDESC, q || !first ? 1u : 0u);
+                        if (release) umma_commit(&sm.empty[st]);
+                    };
+                    if (KB > NSLOT) {
+                        if (reuse) {
+#pragma unroll
+                            for (int i = 0; i < RS; ++i) group(i, KB - RS + i, i == 0, true, true);
+                        }
+#pragma unroll
+                        for (int i = 0; i < KB; ++i) {
+                            if (i >= KB - RS && reuse) break;  // (these came first)
+                            // a kept stage is released by the next phase, after its own use
+                            group(i % NSLOT, i, i == 0 && !reuse, false, !(keep && i >= KB - RS));
+                            if (i % NSLOT == NSLOT - 1) pf ^= 1u;
+                        }
+                    } else if (reuse) {
+#pragma unroll
+                        for (int i = 0; i < KB; ++i) group((sb ^ KB) + i, i, i == 0, true, true);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < KB; ++i) group(sb + i, i, i == 0, false, !keep);
+                        if (sb) pf ^= 1u;
+                        sb ^= KB;
                     }
                 }
                 if (!go) break;
@@ -331,98 +359,112 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
             wait_bar(&sm.drain, 0, ctl, 0, ctr0);
         }
         __syncwarp();
-    } else if (warp >= 4) {
-        // ---- epilogue: one row per thread, 128 rows per tile -------------------
-        const int t = (warp - 4) >> 2, row = tid - EPI_T0 - 128 * t, q = (warp - 4) & 3;
+    } else {
+        // ---- epilogue: HALVES threads per row, 128 rows per tile ----------------
+        const int e = tid - EPI_T0, t = e / ET, half = HALVES == 2 ? (e >> 7) & 1 : 0, q = warp & 3;
+        const int row = 32 * q + lane;  // a warp reads TMEM lanes 32 (warp % 4) ..
+        const bool own = half == 0;     // this thread owns its row
         const int bar = 1 + t;
-        const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(t * W);
+        constexpr int HC = W / HALVES;  // columns per thread, from c0
+        const int c0 = half * HC;
+        const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(t * W + c0);
         const uint32_t arow = su32(&sm.a[t][0][0]) + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
         const int sw = row & 7;
         const unsigned lt = (1u << lane) - 1u;
         int cur = 0;
         const Item *it = &items[0];
-        GridP g = it->g;  // the current item's grid and scratch, kept in registers
-        Counters *ctr = it->s.ctr;
-        unsigned long long *marks_raw = it->s.marks_raw;
-        uint32_t *colcount = it->s.colcount;
-        unsigned long long cap_marks = (unsigned long long)it->s.cap_marks;
+        GridP g = it->g;  // the current item's grid, kept in registers
         uint32_t col = NONE, rank = 0;
         int k = 0;
         bool done = false;
         float x = 0.f, y = 0.f;
-        unsigned long long evals = 0, idx = 0;
+        unsigned long long idx = 0;
+        uint32_t evals = 0;  // flushed per item: a row makes fewer than 2^32 evaluations
         uint32_t pacc = 0;
-        float *bmid = sm.bmid[t];
-        float *wout = sm.wout[t];
+        const float *bmid = sm.bmid[t] + c0;
+        const float *wout = sm.wout[t] + c0;
         // a mark found in the previous step, written once its slot is known
-        bool pend_mark = false;
         unsigned long long pend_base = 0, pend_rec = 0;
         unsigned pend_mask = 0;
+        auto write_pending = [&]() {
+            if (!pend_mask) return;
+            const Scratch &s = it->s;
+            const unsigned long long b0 = __shfl_sync(FULL, pend_base, __ffs(pend_mask) - 1);
+            if (pend_mask & (1u << lane)) {
+                const unsigned long long mi = b0 + __popc(pend_mask & lt);
+                if (mi < (unsigned long long)s.cap_marks) s.marks_raw[mi] = pend_rec;
+                else atomicOr(&s.ctr->flags, FLAG_MARK_OVERFLOW);
+            }
+            pend_mask = 0;
+        };
         for (;;) {
             // 1. the work of this row, from item cur
             const int N = g.N;
+            Counters *ctr = it->s.ctr;
             bool live = false;
             float px = 0.f, py = 0.f, pz = 0.f;
-            if (MODE == MODE_HOP) {
-                const uint32_t ncols = (uint32_t)N * (uint32_t)N;
-                const bool need = col == NONE && !done;
-                const unsigned needm = __ballot_sync(FULL, need);
-                if (needm) {
-                    const int leader = __ffs(needm) - 1;
+            if (own) {
+                if (MODE == MODE_HOP) {
+                    const uint32_t ncols = (uint32_t)N * (uint32_t)N;
+                    const bool need = col == NONE && !done;
+                    const unsigned needm = __ballot_sync(FULL, need);
+                    if (needm) {
+                        const int leader = __ffs(needm) - 1;
+                        unsigned long long base = 0;
+                        if (lane == leader) base = atomicAdd(&ctr->next_col, (unsigned long long)__popc(needm));
+                        base = __shfl_sync(FULL, base, leader);
+                        if (need) {
+                            const unsigned long long c = base + __popc(needm & lt);
+                            if (c < ncols) {
+                                col = column_of_claim((uint32_t)c, N);
+                                k = 0;
+                                rank = 0;
+                                const int i = (int)(col / (uint32_t)N), j = (int)(col - (uint32_t)i * N);
+                                x = fmaf((float)i + 0.5f, g.h, g.lo[0]);
+                                y = fmaf((float)j + 0.5f, g.h, g.lo[1]);
+                            } else {
+                                done = true;
+                            }
+                        }
+                    }
+                    live = col != NONE;
+                    if (live) {
+                        px = x;
+                        py = y;
+                        pz = fmaf((float)k + 0.5f, g.h, g.lo[2]);
+                    }
+                } else {
+                    unsigned long long total = (unsigned long long)npts;
+                    if (MODE == MODE_VERTS)
+                        total = (ctr->flags & STOP_FLAGS) ? 0ull : ctr->verts;
                     unsigned long long base = 0;
-                    if (lane == leader) base = atomicAdd(&ctr->next_col, (unsigned long long)__popc(needm));
-                    base = __shfl_sync(FULL, base, leader);
-                    if (need) {
-                        const unsigned long long c = base + __popc(needm & lt);
-                        if (c < ncols) {
-                            col = column_of_claim((uint32_t)c, N);
-                            k = 0;
-                            rank = 0;
-                            const int i = (int)(col / (uint32_t)N), j = (int)(col - (uint32_t)i * N);
-                            x = fmaf((float)i + 0.5f, g.h, g.lo[0]);
-                            y = fmaf((float)j + 0.5f, g.h, g.lo[1]);
+                    if (lane == 0) base = done ? total : atomicAdd(&ctr->next_tile, 32ull);
+                    base = __shfl_sync(FULL, base, 0);
+                    idx = base + lane;
+                    live = idx < total;
+                    if (base >= total) done = true;
+                    if (live) {
+                        if (MODE == MODE_POINTS) {
+                            px = pts[3 * idx];
+                            py = pts[3 * idx + 1];
+                            pz = pts[3 * idx + 2];
                         } else {
-                            done = true;
+                            const unsigned long long key = it->s.vkey[idx];
+                            const int N1 = N + 1;
+                            const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), c = (uint32_t)(key >> 32);
+                            const uint32_t a = line / (uint32_t)N1, b = line - a * (uint32_t)N1;
+                            px = fmaf((float)a, g.h, g.lo[0]);
+                            py = fmaf((float)b, g.h, g.lo[1]);
+                            pz = fmaf((float)c, g.h, g.lo[2]);
                         }
                     }
                 }
-                live = col != NONE;
-                if (live) {
-                    px = x;
-                    py = y;
-                    pz = fmaf((float)k + 0.5f, g.h, g.lo[2]);
-                }
-            } else {
-                unsigned long long total = (unsigned long long)npts;
-                if (MODE == MODE_VERTS)
-                    total = (ctr->flags & STOP_FLAGS) ? 0ull : ctr->verts;
-                unsigned long long base = 0;
-                if (lane == 0) base = done ? total : atomicAdd(&ctr->next_tile, 32ull);
-                base = __shfl_sync(FULL, base, 0);
-                idx = base + lane;
-                live = idx < total;
-                if (base >= total) done = true;
-                if (live) {
-                    if (MODE == MODE_POINTS) {
-                        px = pts[3 * idx];
-                        py = pts[3 * idx + 1];
-                        pz = pts[3 * idx + 2];
-                    } else {
-                        const unsigned long long key = it->s.vkey[idx];
-                        const int N1 = N + 1;
-                        const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), c = (uint32_t)(key >> 32);
-                        const uint32_t a = line / (uint32_t)N1, b = line - a * (uint32_t)N1;
-                        px = fmaf((float)a, g.h, g.lo[0]);
-                        py = fmaf((float)b, g.h, g.lo[1]);
-                        pz = fmaf((float)c, g.h, g.lo[2]);
-                    }
-                }
+                __syncwarp();
             }
-            __syncwarp();
-            const bool any = epi_any(bar, live);
+            const bool any = bar_any(bar, ET, live);
             // the abort decision goes through the barrier so that it is uniform
-            if (epi_any(bar, (*ctl & CTL_ABORT) != 0)) {
-                if (row == 0) {
+            if (bar_any(bar, ET, (*ctl & CTL_ABORT) != 0)) {
+                if (own && row == 0) {
                     vdone[t] = 1;
                     __threadfence_block();
                     mbar_arrive(&sm.item_ready[t]);
@@ -432,24 +474,16 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
             }
             if (!any) {
                 // item cur has no work left for this tile: next item, or done
-                if (MODE == MODE_HOP) {
-                    if (pend_mark) {
-                        const unsigned long long b0 = __shfl_sync(FULL, pend_base, __ffs(pend_mask) - 1);
-                        if (pend_mask & (1u << lane)) {
-                            const unsigned long long mi = b0 + __popc(pend_mask & lt);
-                            if (mi < cap_marks) marks_raw[mi] = pend_rec;
-                            else atomicOr(&ctr->flags, FLAG_MARK_OVERFLOW);
-                        }
-                    }
-                    pend_mark = false;
-                    pend_mask = 0;
-                    for (int o = 16; o > 0; o >>= 1) evals += __shfl_xor_sync(FULL, evals, o);
-                    if (lane == 0 && evals) atomicAdd(&ctr->hop_evals, evals);
+                if (MODE == MODE_HOP && own) {
+                    write_pending();
+                    unsigned long long ev = evals;
+                    for (int o = 16; o > 0; o >>= 1) ev += __shfl_xor_sync(FULL, ev, o);
+                    if (lane == 0 && ev) atomicAdd(&ctr->hop_evals, ev);
                     evals = 0;
                 }
                 ++cur;
                 if (cur >= n_items) {
-                    if (row == 0) {
+                    if (own && row == 0) {
                         vdone[t] = 1;
                         __threadfence_block();
                         mbar_arrive(&sm.item_ready[t]);
@@ -459,25 +493,20 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                 }
                 it = &items[cur];
                 g = it->g;
-                ctr = it->s.ctr;
-                marks_raw = it->s.marks_raw;
-                colcount = it->s.colcount;
-                cap_marks = (unsigned long long)it->s.cap_marks;
                 col = NONE;
                 done = false;
-                load_item<W>(sm, t, it->m, row, 128);
-                epi_any(bar, false);  // the new item's parameters are in place
+                load_item<W>(sm, t, it->m, row + TM * half, ET);
+                bar_sync(bar, ET);  // the new item's parameters are in place
                 continue;
             }
-            if (row == 0) {
-                sm.cur_wbf[t] = it->m.wbf;
-                mbar_arrive(&sm.item_ready[t]);
-                if (MODE == MODE_HOP) atomicAdd(&ctr->row_slots, 128ull);
-            }
-            const MlpDev &m = it->m;
-            // 2. the layer-0 operand A0 (BF16 high and low parts of the point, two
-            // unit inputs for the bias) in the first 16 inputs of K-block 0
-            {
+            if (own) {
+                if (row == 0) {
+                    sm.cur_wbf[t] = it->m.wbf;
+                    mbar_arrive(&sm.item_ready[t]);
+                    if (MODE == MODE_HOP) atomicAdd(&ctr->row_slots, 128ull);
+                }
+                // 2. the layer-0 operand A0 (BF16 high and low parts of the point, two
+                // unit inputs for the bias) in the first 16 inputs of K-block 0
                 uint32_t xh, xl, yh, yl, zh, zl;
                 split2(px, xh, xl);
                 split2(py, yh, yl);
@@ -485,20 +514,10 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                 constexpr uint32_t ONE = 0x3F80u;  // 1.0 in BF16
                 sts128(arow + ((0 ^ sw) << 4), xh | (xl << 16), xh | (yh << 16), yl | (yh << 16), zh | (zl << 16));
                 sts128(arow + ((1 ^ sw) << 4), zh | (ONE << 16), ONE, 0u, 0u);
+                fence_async_smem();
             }
-            fence_async_smem();
             mbar_arrive(&sm.a_full[t]);
-            if (MODE == MODE_HOP && pend_mark) {
-                // the previous step's marks: their slots came back meanwhile
-                const unsigned long long b0 = __shfl_sync(FULL, pend_base, __ffs(pend_mask) - 1);
-                if (pend_mask & (1u << lane)) {
-                    const unsigned long long mi = b0 + __popc(pend_mask & lt);
-                    if (mi < cap_marks) marks_raw[mi] = pend_rec;
-                    else atomicOr(&ctr->flags, FLAG_MARK_OVERFLOW);
-                }
-                pend_mark = false;
-                pend_mask = 0;
-            }
+            if (MODE == MODE_HOP && own) write_pending();  // the previous step's marks: their slots came back meanwhile
             // 3. phases 0 (layer 0, its bias in B0) .. n_mid (hidden layers)
             float gsum = 0.f;
             for (int l = 0; l <= n_mid; ++l) {
@@ -506,60 +525,70 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                 pacc ^= 1u;
                 __syncwarp();  // tcgen05.ld below needs the whole warp converged
                 tc_fence_after();
-                const float *bl = l ? bmid + (l - 1) * W : sm.zb;
-                uint32_t ra[32], rb[32];
-                tmem_ld32_async(taddr, ra);
-                tmem_wait_ld();
+                const float *bl = bmid + (l - 1) * W;
                 if (l < n_mid) {
 #pragma unroll
-                    for (int j = 0; j < W / 32; ++j) {
-                        // the next chunk's load runs while this one is converted
-                        uint32_t(&cu)[32] = (j & 1) ? rb : ra;
-                        uint32_t(&nx)[32] = (j & 1) ? ra : rb;
-                        if (j + 1 < W / 32) tmem_ld32_async(taddr + 32 * (j + 1), nx);
-                        const float4 *bp = reinterpret_cast<const float4 *>(bl + 32 * j);
-                        const int kb = j >> 1, c0 = (j & 1) * 4;
+                    for (int j = 0; j < HC / 32; ++j) {
+                        uint32_t cu[32];
+                        tmem_ld32_async(taddr + 32 * j, cu);
+                        tmem_wait_ld();
+                        const int cc = c0 + 32 * j;  // first column of the chunk
+                        const uint32_t ab = arow + (uint32_t)((cc >> 6) * (TM * 128));
+                        const int ch = (cc & 63) >> 3;
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            const float4 b0 = bp[2 * c], b1 = bp[2 * c + 1];
-                            const uint32_t p0 = pack_relu_bf16(__uint_as_float(cu[8 * c + 0]) + b0.x,
-                                                               __uint_as_float(cu[8 * c + 1]) + b0.y);
-                            const uint32_t p1 = pack_relu_bf16(__uint_as_float(cu[8 * c + 2]) + b0.z,
-                                                               __uint_as_float(cu[8 * c + 3]) + b0.w);
-                            const uint32_t p2 = pack_relu_bf16(__uint_as_float(cu[8 * c + 4]) + b1.x,
-                                                               __uint_as_float(cu[8 * c + 5]) + b1.y);
-                            const uint32_t p3 = pack_relu_bf16(__uint_as_float(cu[8 * c + 6]) + b1.z,
-                                                               __uint_as_float(cu[8 * c + 7]) + b1.w);
-                            sts128(arow + kb * (TM * 128) + (((c0 + c) ^ sw) << 4), p0, p1, p2, p3);
+                            unsigned long long z[4];
+#pragma unroll
+                            for (int p = 0; p < 4; ++p)
+                                z[p] = pack2(__uint_as_float(cu[8 * c + 2 * p]), __uint_as_float(cu[8 * c + 2 * p + 1]));
+                            if (l) {
+                                const float4 b0 = reinterpret_cast<const float4 *>(bl + 32 * j)[2 * c];
+                                const float4 b1 = reinterpret_cast<const float4 *>(bl + 32 * j)[2 * c + 1];
+                                z[0] = fadd2(z[0], pack2(b0.x, b0.y));
+                                z[1] = fadd2(z[1], pack2(b0.z, b0.w));
+                                z[2] = fadd2(z[2], pack2(b1.x, b1.y));
+                                z[3] = fadd2(z[3], pack2(b1.z, b1.w));
+                            }
+                            sts128(ab + (uint32_t)(((ch + c) ^ sw) << 4), pack_relu_bf16(lo2(z[0]), hi2(z[0])),
+                                   pack_relu_bf16(lo2(z[1]), hi2(z[1])), pack_relu_bf16(lo2(z[2]), hi2(z[2])),
+                                   pack_relu_bf16(lo2(z[3]), hi2(z[3])));
                         }
-                        tmem_wait_ld();
                     }
                     tc_fence_before();
                     fence_async_smem();
                     mbar_arrive(&sm.a_full[t]);
                 } else {
                     // output layer in FP32 from the accumulators
+                    float d0 = 0.f, d1 = 0.f;
 #pragma unroll
-                    for (int j = 0; j < W / 32; ++j) {
-                        uint32_t(&cu)[32] = (j & 1) ? rb : ra;
-                        uint32_t(&nx)[32] = (j & 1) ? ra : rb;
-                        if (j + 1 < W / 32) tmem_ld32_async(taddr + 32 * (j + 1), nx);
+                    for (int j = 0; j < HC / 32; ++j) {
+                        uint32_t cu[32];
+                        tmem_ld32_async(taddr + 32 * j, cu);
+                        tmem_wait_ld();
                         const float4 *bp = reinterpret_cast<const float4 *>(bl + 32 * j);
                         const float4 *wp = reinterpret_cast<const float4 *>(wout + 32 * j);
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
                             const float4 b = bp[c], w = wp[c];
-                            gsum = fmaf(w.x, fmaxf(__uint_as_float(cu[4 * c + 0]) + b.x, 0.f), gsum);
-                            gsum = fmaf(w.y, fmaxf(__uint_as_float(cu[4 * c + 1]) + b.y, 0.f), gsum);
-                            gsum = fmaf(w.z, fmaxf(__uint_as_float(cu[4 * c + 2]) + b.z, 0.f), gsum);
-                            gsum = fmaf(w.w, fmaxf(__uint_as_float(cu[4 * c + 3]) + b.w, 0.f), gsum);
+                            d0 = fmaf(w.x, fmaxf(__uint_as_float(cu[4 * c + 0]) + b.x, 0.f), d0);
+                            d1 = fmaf(w.y, fmaxf(__uint_as_float(cu[4 * c + 1]) + b.y, 0.f), d1);
+                            d0 = fmaf(w.z, fmaxf(__uint_as_float(cu[4 * c + 2]) + b.z, 0.f), d0);
+                            d1 = fmaf(w.w, fmaxf(__uint_as_float(cu[4 * c + 3]) + b.w, 0.f), d1);
                         }
-                        tmem_wait_ld();
                     }
                     tc_fence_before();
+                    gsum = d0 + d1;
                 }
             }
-            // 4. f, then the hop step or the store
+            if (HALVES == 2) {
+                if (!own) sm.red[t][row] = gsum;
+                bar_sync(bar, ET);
+                if (!own) continue;
+                gsum += sm.red[t][row];
+            }
+            // 4. f, then the hop step or the store (red is rewritten only after
+            // the barriers at the top of the next step)
+            const MlpDev &m = it->m;
             const float f = outer_f(m, px, py, pz, gsum + m.bout);
             if (MODE == MODE_HOP) {
                 bool mark = false, empty = false;
@@ -580,10 +609,9 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                 }
                 const unsigned mm = __ballot_sync(FULL, mark);
                 if (mm) {
-                    // claim the slots now; the records are written after the next layer 0
+                    // claim the slots now; the records are written in the next step
                     const int leader = __ffs(mm) - 1;
                     if (lane == leader) pend_base = atomicAdd(&ctr->marks, (unsigned long long)__popc(mm));
-                    pend_mark = true;
                     pend_mask = mm;
                     if (mark) pend_rec = pack_mark(col, (uint32_t)k, rank, empty);
                 }
@@ -595,21 +623,20 @@ __global__ void __launch_bounds__(128 + 128 * TILES, 1)
                         k += step;
                     }
                     if (k >= N) {
-                        colcount[col] = rank;
+                        it->s.colcount[col] = rank;
                         col = NONE;
                     }
+                    ++evals;
                 }
-                if (live) ++evals;
             } else if (live) {
                 if (MODE == MODE_VERTS) {
-                    if (!isfinite(f)) atomicOr(&it->s.ctr->flags, FLAG_NONFINITE);
+                    if (!isfinite(f)) atomicOr(&ctr->flags, FLAG_NONFINITE);
                     it->s.vval[idx] = f;
                 } else {
                     outv[idx] = f;
                 }
             }
         }
-        (void)evals;
     }
     // ---- tear-down ---------------------------------------------------------
     tc_fence_before();
@@ -628,7 +655,7 @@ void launch_bf16(const Item *items, int n_items, const float *p, long long n, fl
         const long long tiles = (n + 128 * TILES - 1) / (128 * TILES);
         if (grid > tiles) grid = (int)(tiles < 1 ? 1 : tiles);
     }
-    k_mlp_bf16<W, MODE, TILES><<<grid, 128 + 128 * TILES, smem, st>>>(items, n_items, p, n, out, wait_limit_ns());
+    k_mlp_bf16<W, MODE, TILES><<<grid, EPI_T0 + TM * halves_of<W>() * TILES, smem, st>>>(items, n_items, p, n, out, wait_limit_ns());
 }
 
 }  // namespace

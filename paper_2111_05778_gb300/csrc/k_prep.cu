@@ -10,11 +10,12 @@
 //       the 128-byte swizzled K-major layout the MMA reads from shared memory
 //       (row n, 16-byte chunk c of inputs [8c, 8c+8) at
 //       (n/8)*1024 + (n%8)*128 + ((c ^ n%8) * 16)), BF16 rounded to nearest
-//       even;
+//       even; at width 256 K-blocks of 32 inputs with the 64-byte swizzle
+//       ((n/8)*512 + (n%8)*64 + ((c ^ (n/2)%4) * 16));
 //   wx6 (split-BF16 engine): per layer three BF16 parts of every weight,
 //       w = w_h + w_m + w_l exactly (w_h = bf16(w), w_m = bf16(w - w_h),
 //       w_l = bf16(w - w_h - w_m)), stored part by part (low, middle, high),
-//       each part in wbf's layout;
+//       each part in K-blocks of 64 inputs with the 128-byte swizzle;
 //   wx6t the same of the transposed weights (rows = inputs of the layer, K =
 //       its outputs), layer n_mid first (the adjoint walks down);
 //   bm  hidden biases, n_mid x [W].
@@ -54,7 +55,13 @@ __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ para
         const int kb = i >> 6, kk = i & 63;
         const int byte = (o >> 3) * 1024 + (o & 7) * 128 + (((kk >> 3) ^ (o & 7)) << 4) + (kk & 7) * 2;
         const uint16_t hi = bf16_rne(v);
-        wbf[((long long)l * KB + kb) * W * 64 + byte / 2] = hi;
+        if (W == 256) {
+            const int kc = (i >> 3) & 3;
+            wbf[((long long)l * 2 * KB + (i >> 5)) * W * 32 +
+                ((o >> 3) * 512 + (o & 7) * 64 + ((kc ^ ((o >> 1) & 3)) << 4) + (i & 7) * 2) / 2] = hi;
+        } else {
+            wbf[((long long)l * KB + kb) * W * 64 + byte / 2] = hi;
+        }
         const float rem = v - bf16_val(hi);  // exact
         const uint16_t mid = bf16_rne(rem);
         const uint16_t low = bf16_rne(rem - bf16_val(mid));

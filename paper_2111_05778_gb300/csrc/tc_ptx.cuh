@@ -102,6 +102,13 @@ __device__ __forceinline__ unsigned long long sdesc(uint32_t saddr) {
            (1ull << 46) | (2ull << 61);
 }
 
+// K-major operand of 32 BF16 inputs per row, 64-byte swizzle, 8-row groups
+// 512 B apart.
+__device__ __forceinline__ unsigned long long sdesc64(uint32_t saddr) {
+    return (unsigned long long)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((unsigned long long)(512 >> 4) << 32) |
+           (1ull << 46) | (4ull << 61);
+}
+
 // K-major operand of 16 BF16 inputs per row, 32-byte swizzle, 8-row groups
 // 256 B apart.
 __device__ __forceinline__ unsigned long long sdesc32(uint32_t saddr) {
