@@ -287,10 +287,15 @@ void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, floa
     // forward: pre-activations of every layer; backward chain of g (both on the
     // FP32 tile engine of the network's evaluation)
     const long long ldl = (long long)b.VC * W;
-    launch_adj_fwd_fp32(m, P, V, b.Z, ldl, b.mbits, b.nsm, st);
-    k_adj_top<<<eb, 256, 0, st>>>(Zl[L], V, m.wout, W, Dl[L]);
-    launch_adj_bwd_fp32(m, V, b.mbits, b.D, ldl, b.nsm, st);
-    k_adj_s<<<(V + 7) / 8, 256, 0, st>>>(P, dL, V, Dl[0], m.w0, W, m.alpha, 1.f / m.beta * m.inv_lam, m.radial, b.s);
+    if (L <= x6_max_mid()) {
+        // on the tensor cores, both ways per tile in one launch; Z holds relu(z)
+        launch_adj_mlp_x6(m, P, dL, V, b.Z, b.D, b.s, b.mbits, ldl, b.nsm, st);
+    } else {
+        launch_adj_fwd_fp32(m, P, V, b.Z, ldl, b.mbits, b.nsm, st);
+        k_adj_top<<<eb, 256, 0, st>>>(Zl[L], V, m.wout, W, Dl[L]);
+        launch_adj_bwd_fp32(m, V, b.mbits, b.D, ldl, b.nsm, st);
+        k_adj_s<<<(V + 7) / 8, 256, 0, st>>>(P, dL, V, Dl[0], m.w0, W, m.alpha, 1.f / m.beta * m.inv_lam, m.radial, b.s);
+    }
     // parameter gradients: sums over the vertices of the chunk
     const size_t oW0 = 0, ob0 = (size_t)3 * W, omid = ob0 + W;
     const size_t ow = omid + (size_t)L * ((size_t)W * W + W);
