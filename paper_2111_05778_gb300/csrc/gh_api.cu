@@ -1277,7 +1277,7 @@ extern "C" int gh_backward(const gh_sdb *cs, const float *verts, const float *dL
     // vertices per chunk: the stored activations and deltas of a chunk take
     // 2 (L + 1) W floats per vertex (1.6 GB at W = 256, L = 5)
     constexpr int VCHUNK = GH_ADJOINT_CHUNK;
-    const size_t need = adjoint_buffer_floats(W, L, VCHUNK, S);
+    const size_t need = adjoint_buffer_floats(W, L, VCHUNK, S, nsm);
     if (s->adj_floats < need) {
         if (s->adj) cudaFree(s->adj);
         s->adj = nullptr;
@@ -1293,7 +1293,7 @@ extern "C" int gh_backward(const gh_sdb *cs, const float *verts, const float *dL
     b.D = b.Z + (size_t)(L + 1) * b.VC * W;
     b.s = b.D + (size_t)(L + 1) * b.VC * W;
     b.part = b.s + b.VC;
-    b.ones = b.part + (size_t)S * W * W;
+    b.ones = b.part + adjoint_part_floats(W, L, S, nsm);
     b.mbits = reinterpret_cast<uint32_t *>(b.ones + b.VC);
     adjoint_fill_ones(b.ones, b.VC, st);
     for (long long v0 = 0; v0 < V; v0 += b.VC) {

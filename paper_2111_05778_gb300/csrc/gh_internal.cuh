@@ -291,7 +291,14 @@ void launch_adj_fwd_fp32(const MlpDev &m, const float *P, long long V, float *Z,
                          int nsm, cudaStream_t st);
 void launch_adj_bwd_fp32(const MlpDev &m, long long V, const uint32_t *mbits, float *D, long long ldl, int nsm,
                          cudaStream_t st);
-size_t adjoint_buffer_floats(int W, int n_mid, int VC, int splits);
+// weight and bias gradients of the hidden layers (k_adj_wgrad.cu): dst packs
+// { W_l b_l } per layer, (+)= c * the sums; part: work space of
+// adj_wgrad_floats
+size_t adj_wgrad_floats(int W, int n_mid, int nsm);
+void launch_adj_wgrad(const MlpDev &m, const float *A, const float *D, const float *s, long long V, long long ldl,
+                      float *part, float c, float *dst, bool accumulate, int nsm, cudaStream_t st);
+size_t adjoint_part_floats(int W, int n_mid, int splits, int nsm);
+size_t adjoint_buffer_floats(int W, int n_mid, int VC, int splits, int nsm);
 void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, float *grad, bool accumulate,
                    const AdjBuffers &b, cudaStream_t st);
 void adjoint_fill_ones(float *p, long long n, cudaStream_t st);

@@ -267,10 +267,16 @@ __global__ void k_fill(float *p, long long n, float v) {
 
 }  // namespace
 
-size_t adjoint_buffer_floats(int W, int n_mid, int VC, int splits) {
+// floats of the partial sums: the FFMA path's splits or the tensor path's ranges
+size_t adjoint_part_floats(int W, int n_mid, int splits, int nsm) {
+    const size_t a = (size_t)splits * W * W, b = adj_wgrad_floats(W, n_mid, nsm);
+    return a > b ? a : b;
+}
+
+size_t adjoint_buffer_floats(int W, int n_mid, int VC, int splits, int nsm) {
     const size_t L1 = (size_t)n_mid + 1;
     const size_t mask_words = (size_t)n_mid * ((VC + 127) / 128) * 256 * (W / 64);
-    return L1 * VC * W * 2 + VC + (size_t)splits * W * W + VC + mask_words;
+    return L1 * VC * W * 2 + VC + adjoint_part_floats(W, n_mid, splits, nsm) + VC + mask_words;
 }
 
 // One chunk of vertices; accumulates into grad (packed like the parameters).
@@ -305,7 +311,9 @@ void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, floa
     k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W * 3, c, grad + oW0, accumulate);
     colsum<1, false>(Dl[0], V, W, b.s, nullptr, S, b.part, st);
     k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W, c, grad + ob0, accumulate);
-    for (int l = 1; l <= L; ++l) {
+    const bool tensor = L <= x6_max_mid();
+    if (tensor) launch_adj_wgrad(m, b.Z, b.D, b.s, V, ldl, b.part, c, grad + omid, accumulate, b.nsm, st);
+    for (int l = 1; l <= (tensor ? 0 : L); ++l) {
         const size_t oW = omid + (size_t)(l - 1) * ((size_t)W * W + W), ob = oW + (size_t)W * W;
         gemm<true, false, false, true>(W, W, V, Dl[l], W, Zl[l - 1], W, b.part, W, nullptr, nullptr, b.s, S, st);
         k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W * W, c, grad + oW, accumulate);
