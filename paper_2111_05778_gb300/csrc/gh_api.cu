@@ -390,7 +390,7 @@ extern "C" int gh_release_cache(void) {
         cudaSetDevice(e.device);
         Scratch &c = e.scr;
         void *ptrs[] = {c.ctr, c.marks_raw, c.marks_csr, c.colcount, c.coloff, c.linecount, c.lineoff,
-                        c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis};
+                        c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.cull};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     }
@@ -428,7 +428,7 @@ extern "C" int gh_create_sdb(const gh_sdb_desc *desc, gh_sdb **out) {
 static void free_scratch(gh_sdb *s) {
     Scratch &c = s->scr;
     void *ptrs[] = {c.ctr, c.marks_raw, c.marks_csr, c.colcount, c.coloff, c.linecount, c.lineoff,
-                    c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis};
+                    c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.cull};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     s->scr = Scratch{};
@@ -480,13 +480,18 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
     const long long keep_cap = c.cap_lat;
     uint32_t *keep_vis = c.vis;
     const long long keep_vcap = c.cap_vis;
+    uint32_t *keep_cull = c.cull;
+    const long long keep_ccap = c.cap_cull;
     c.lat = nullptr;
     c.vis = nullptr;
+    c.cull = nullptr;
     free_scratch(s);
     c.lat = keep_lat;
     c.cap_lat = keep_cap;
     c.vis = keep_vis;
     c.cap_vis = keep_vcap;
+    c.cull = keep_cull;
+    c.cap_cull = keep_ccap;
     s->item_valid = false;
     const long long ncols = (long long)NN * NN, nlines = (long long)(NN + 1) * (NN + 1);
     GH_CUDA(cudaMalloc((void **)&c.ctr, sizeof(Counters)));
@@ -504,6 +509,19 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
     c.cap_marks = cm;
     c.cap_verts = cv;
     s->scr_N = NN;
+    return GH_OK;
+}
+
+// The culling masks of an analytic SDB on an N-grid.
+static int ensure_cull(gh_sdb *s, int N) {
+    const long long need = s->kind == GH_SDB_CSG ? cull_words(N, s->nprim) : 0;
+    if (s->scr.cap_cull >= need) return GH_OK;
+    if (s->scr.cull) cudaFree(s->scr.cull);
+    s->scr.cull = nullptr;
+    s->scr.cap_cull = 0;
+    GH_CUDA(cudaMalloc((void **)&s->scr.cull, sizeof(uint32_t) * need));
+    s->scr.cap_cull = need;
+    s->item_valid = false;
     return GH_OK;
 }
 
@@ -637,7 +655,7 @@ static inline void mark_phase(int i, cudaStream_t st) {
 }
 
 // Kernel launches per phase (fixed by the launch sequence below).
-static constexpr int LAUNCHES_HOP = 2, LAUNCHES_LISTS = 8, LAUNCHES_VERTS = 1, LAUNCHES_REFINE = 4,
+static constexpr int LAUNCHES_HOP = 2, LAUNCHES_LISTS = 7, LAUNCHES_VERTS = 1, LAUNCHES_REFINE = 4,
                      LAUNCHES_MC = 2;
 
 // FP32 evaluation of a neural SDB: on the tensor cores with split-BF16
@@ -681,6 +699,10 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         return GH_OK;
     }
     if (s->kind == GH_SDB_CSG) {
+        if (cull_words(g.N, s->nprim) > 0) {
+            launch_cull(s->d_item, 1, g.N, s->nprim, st);
+            ++launches;
+        }
         launch_hop_csg(s->d_item, 1, s->nprim, nsm, o.ray_block, st);
         mark_phase(1, st);
         launch_build_lists(g, c, st);
@@ -758,7 +780,7 @@ extern "C" int gh_polygonize(const gh_grid *grid, const gh_sdb *csdb, const gh_o
     long long want_m = 8 * N2 > (1 << 16) ? 8 * N2 : (1 << 16);
     long long want_v = 2 * want_m;
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((rc = ensure_scratch(s, g.N, want_m, want_v))) return rc;
+        if ((rc = ensure_scratch(s, g.N, want_m, want_v)) || (rc = ensure_cull(s, g.N))) return rc;
         if (o.method == GH_METHOD_ENUM && (rc = ensure_lattice(s, g.N))) return rc;
         if (wants_index(*out) && (rc = ensure_index(s))) return rc;
         if ((rc = enqueue_once(s, g, o, *out, nsm, st))) return rc;
@@ -1007,7 +1029,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             any_mlp = true;
         }
     }
-    long long launches = 1 + 8 + 1 + 1;  // counters, lists, Marching Cubes, status words
+    long long launches = 1 + 7 + 1 + 1;  // counters, lists, Marching Cubes, status words
     launch_init_b(P.d_items, B, st);
     for (auto &gr : P.groups) {
         ++launches;
@@ -1016,7 +1038,13 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         const int n = gr.second - gr.first;
         if (first->kind == GH_SDB_CSG) {
             int mx = 1;
-            for (int q = gr.first; q < gr.second; ++q) mx = sd[P.order[q]]->nprim > mx ? sd[P.order[q]]->nprim : mx;
+            int mN = 2;
+            for (int q = gr.first; q < gr.second; ++q) {
+                mx = sd[P.order[q]]->nprim > mx ? sd[P.order[q]]->nprim : mx;
+                mN = P.g[P.order[q]].N > mN ? P.g[P.order[q]].N : mN;
+            }
+            launch_cull(di, n, mN, mx, st);
+            ++launches;
             launch_hop_csg(di, n, mx, nsm, o.ray_block, st);
         } else if (o.precision == GH_FP32) {
             hop_mlp_fp32(first, di, n, nsm, st);
@@ -1128,6 +1156,7 @@ extern "C" int gh_polygonize_batch(int B, const gh_grid *grids, const gh_sdb *co
     for (int attempt = 0; attempt < 4; ++attempt) {
         for (int b = 0; b < B; ++b)
             if ((rc = ensure_scratch(sd[b], P.g[b].N, want_m[b], want_v[b])) ||
+                (rc = ensure_cull(sd[b], P.g[b].N)) ||
                 (wants_index(outs[b]) && (rc = ensure_index(sd[b])))) {
                 cudaFree(d_items);
                 return rc;

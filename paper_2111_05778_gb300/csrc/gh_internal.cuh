@@ -172,6 +172,8 @@ struct Scratch {
     long long cap_index;            // entries ebase was sized for (0: none)
     uint32_t *vis;                  // continuation: visited bit per cell [N^3 / 32 words]
     long long cap_vis;              // words of vis
+    uint32_t *cull;                 // analytic SDBs: primitive masks per block of cells (NULL: fold every primitive)
+    long long cap_cull;             // words of cull
 };
 
 // One polygonization of a batch: grid, scratch and SDB.  Kernels that serve
@@ -215,6 +217,8 @@ unsigned long long wait_limit_ns();
 cudaError_t upload_mc_table(const int32_t *ntri, const int32_t *edges);  // k_pipeline.cu
 void launch_init(Scratch &s, cudaStream_t st);
 void launch_stage_prims(const Prim *src, Prim *dst, int nprim, cudaStream_t st);  // records + bounding radii
+long long cull_words(int N, int nprim);  // words of Scratch::cull (0: no masks)
+void launch_cull(const Item *items, int n, int max_N, int max_prims, cudaStream_t st);
 void launch_hop_csg(const Item *items, int n_items, int max_prims, int nsm, int block, cudaStream_t st);
 void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st);
 void launch_eval_vertices_csg(const Prim *prims, int nprim, const GridP &g, Scratch &s, int nsm,
