@@ -541,8 +541,6 @@ static int ensure_index(gh_sdb *s) {
     return GH_OK;
 }
 
-static bool wants_index(const gh_mesh &m) { return m.vert_xyz != nullptr || m.tri_idx != nullptr; }
-
 // The dense lattice array of the enumeration method.
 static int ensure_lattice(gh_sdb *s, int N) {
     const long long need = (long long)(N + 1) * (N + 1) * (N + 1);
@@ -733,8 +731,8 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(5, st);
         launches += LAUNCHES_REFINE;
     }
-    launch_mc(g, c, out, nsm, st);
     if (wants_index(out)) launch_index_mesh(g, c, out, nsm, st);
+    launch_mc(g, c, out, nsm, st);
     launch_finalize(c, out, (long long)g.N * g.N, st);
     mark_phase(6, st);
     g_prof.recorded = g_prof.enabled;
@@ -803,7 +801,6 @@ extern "C" int gh_polygonize(const gh_grid *grid, const gh_sdb *csdb, const gh_o
         if (out->cell_ids && c.cells > (unsigned long long)out->capacity_cells)
             return fail(GH_ERR_CAPACITY, "cell buffer holds %lld, %llu needed", (long long)out->capacity_cells,
                         c.cells);
-        if (c.flags & FLAG_INDEX_MISS) return fail(GH_ERR_CUDA, "indexed output: a triangle edge was not listed");
         if (out->vert_xyz && c.mesh_verts > (unsigned long long)out->capacity_verts)
             return fail(GH_ERR_CAPACITY, "vertex buffer holds %lld, %llu needed", (long long)out->capacity_verts,
                         c.mesh_verts);
@@ -1014,7 +1011,7 @@ static std::vector<std::pair<void *, Item *>> g_graph_items;
 // line lists, the vertex values (one launch for the analytic items, one per
 // neural family), the refinement selection and refinement, Marching Cubes
 // and the status words, each step one launch over all items (the indexed
-// mesh, when asked for, adds two launches per item that wants it).
+// mesh, when asked for, adds four launches).
 static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_options &o, const gh_mesh *outs,
                          int nsm, cudaStream_t st) {
     const int tiles = o.mlp_tiles == 1 ? 1 : 2;
@@ -1078,12 +1075,13 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             vertices_mlp_fp32(first, di, n, nsm, true, st);
         }
     }
+    bool any_index = false;
+    for (int b = 0; b < B; ++b) any_index = any_index || wants_index(outs[b]);
+    if (any_index) {
+        launch_index_mesh_b(P.d_items, B, nsm, st);
+        launches += 4;
+    }
     launch_mc_b(P.d_items, B, nsm, st);
-    for (int b = 0; b < B; ++b)
-        if (wants_index(outs[b])) {
-            launch_index_mesh(P.g[b], sd[b]->scr, outs[b], nsm, st);
-            launches += 5;  // at most
-        }
     launch_finalize_b(P.d_items, B, st);
     g_prof.recorded = false;
     g_prof.launches = launches;
@@ -1198,8 +1196,6 @@ extern "C" int gh_polygonize_batch(int B, const gh_grid *grids, const gh_sdb *co
                           (long long)outs[b].capacity_tris, c.tris);
             else if (outs[b].cell_ids && c.cells > (unsigned long long)outs[b].capacity_cells)
                 rc = fail(GH_ERR_CAPACITY, "item %d: cell buffer too small", b);
-            else if (c.flags & FLAG_INDEX_MISS)
-                rc = fail(GH_ERR_CUDA, "item %d: indexed output: a triangle edge was not listed", b);
             else if (outs[b].vert_xyz && c.mesh_verts > (unsigned long long)outs[b].capacity_verts)
                 rc = fail(GH_ERR_CAPACITY, "item %d: vertex buffer holds %lld, %llu needed", b,
                           (long long)outs[b].capacity_verts, c.mesh_verts);

@@ -35,7 +35,6 @@ enum : unsigned long long {
     FLAG_CELL_OVERFLOW = 8ull,   // caller's cell buffer too small
     FLAG_NONFINITE = 16ull,      // f was NaN or inf somewhere
     FLAG_TIMEOUT = 32ull,        // a bounded device wait gave up
-    FLAG_INDEX_MISS = 64ull,     // indexed output: a triangle edge without a listed end point
 };
 
 // Grid parameters as the kernels see them (FP32).
@@ -209,6 +208,8 @@ __host__ __device__ inline uint32_t mark_col(unsigned long long m) { return (uin
 __host__ __device__ inline uint32_t mark_k(unsigned long long m) { return (uint32_t)((m >> 24) & 0xFFFFull); }
 __host__ __device__ inline uint32_t mark_rank(unsigned long long m) { return (uint32_t)((m >> 40) & 0xFFFFull); }
 
+__host__ __device__ inline bool wants_index(const gh_mesh &m) { return m.vert_xyz != nullptr || m.tri_idx != nullptr; }
+
 // The limit of the engines' bounded waits on their own work, in ns (gh_api.cu;
 // gh_set_wait_limit_ns; 2 s unless set).
 unsigned long long wait_limit_ns();
@@ -271,16 +272,18 @@ void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, flo
 // space (n_mid x ceil(V/128)*128 x W/32 words)
 void launch_adj_mlp_x6(const MlpDev &m, const float *P, const float *dL, long long V, float *A, float *D, float *s,
                        uint32_t *mask, long long ldl, int nsm, cudaStream_t st);
-// exclusive scan of n uint32 into out[0..n] (k_pipeline.cu); bsum holds
-// ceil(n / 4096) partials; *total gets the sum
-void scan_u32_dev(const uint32_t *in, long long n, uint32_t *out, uint32_t *bsum, unsigned long long *total,
-                  Counters *ctr, cudaStream_t st);
+// exclusive scan of *n <= nmax uint32 into out[0..*n] (k_pipeline.cu); bsum
+// holds ceil(nmax / 4096) partials; *total gets the sum
+void scan_u32_dev(const uint32_t *in, long long nmax, const unsigned long long *n, uint32_t *out, uint32_t *bsum,
+                  unsigned long long *total, Counters *ctr, cudaStream_t st);
+void launch_index_scan_b(const Item *items, int n, int nsm, cudaStream_t st);  // of the items with an indexed output
 long long scan_partials(long long n);
 // derived weight layouts of a neural SDB from its packed parameters (k_prep.cu)
 void launch_prep_mlp(const float *params, int W, int n_mid, float *wt, float *wtb, uint16_t *wbf, uint16_t *wx6,
                      uint16_t *wx6t, float *bm, cudaStream_t st);
-// indexed mesh output after Marching Cubes (k_index.cu)
+// the indexed mesh's vertices and their numbers, before Marching Cubes, which writes the indices (k_index.cu)
 void launch_index_mesh(const GridP &g, Scratch &s, const gh_mesh &out, int nsm, cudaStream_t st);
+void launch_index_mesh_b(const Item *items, int n, int nsm, cudaStream_t st);
 
 // implicit-surface adjoint (k_adjoint.cu)
 struct AdjBuffers {

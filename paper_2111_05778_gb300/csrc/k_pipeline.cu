@@ -585,31 +585,39 @@ __device__ __forceinline__ void scan_apply_tile(const uint32_t *__restrict__ in,
 }
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t *__restrict__ in, long long n,
-                                                         uint32_t *__restrict__ bsum, const Counters *ctr) {
+                                                         const unsigned long long *ndev, uint32_t *__restrict__ bsum,
+                                                         const Counters *ctr) {
     __shared__ uint32_t wsum[32];
     if (ctr->flags & STOP_FLAGS) return;
+    if (ndev) n = (long long)*ndev;
+    if ((long long)blockIdx.x * SCAN_TILE >= n) return;
     scan_reduce_tile(in, n, bsum, blockIdx.x, wsum);
 }
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_apply(const uint32_t *__restrict__ in, long long n,
+                                                        const unsigned long long *ndev,
                                                         const uint32_t *__restrict__ bsum, uint32_t *__restrict__ out,
                                                         unsigned long long *total, long long cap, Counters *ctr) {
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t prefix;
     if (ctr->flags & STOP_FLAGS) return;
-    scan_apply_tile(in, n, bsum, out, total, cap, &ctr->flags, blockIdx.x, gridDim.x, wsum, &prefix);
+    if (ndev) n = (long long)*ndev;
+    const long long nt = n > 0 ? (n + SCAN_TILE - 1) / SCAN_TILE : 1;
+    if (blockIdx.x >= nt) return;
+    scan_apply_tile(in, n, bsum, out, total, cap, &ctr->flags, blockIdx.x, nt, wsum, &prefix);
 }
 
-static void scan_u32(const uint32_t *in, long long n, uint32_t *out, uint32_t *bsum, unsigned long long *total,
-                     long long cap, Counters *ctr, cudaStream_t st) {
+// ndev: the length on the device (n is then its bound)
+static void scan_u32(const uint32_t *in, long long n, const unsigned long long *ndev, uint32_t *out, uint32_t *bsum,
+                     unsigned long long *total, long long cap, Counters *ctr, cudaStream_t st) {
     const int nb = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
-    k_scan_reduce<<<nb, SCAN_T, 0, st>>>(in, n, bsum, ctr);
-    k_scan_apply<<<nb, SCAN_T, 0, st>>>(in, n, bsum, out, total, cap, ctr);
+    k_scan_reduce<<<nb, SCAN_T, 0, st>>>(in, n, ndev, bsum, ctr);
+    k_scan_apply<<<nb, SCAN_T, 0, st>>>(in, n, ndev, bsum, out, total, cap, ctr);
 }
 
-void scan_u32_dev(const uint32_t *in, long long n, uint32_t *out, uint32_t *bsum, unsigned long long *total,
-                  Counters *ctr, cudaStream_t st) {
-    scan_u32(in, n, out, bsum, total, 0, ctr, st);
+void scan_u32_dev(const uint32_t *in, long long nmax, const unsigned long long *n, uint32_t *out, uint32_t *bsum,
+                  unsigned long long *total, Counters *ctr, cudaStream_t st) {
+    scan_u32(in, nmax, n, out, bsum, total, 0, ctr, st);
 }
 
 long long scan_partials(long long n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
@@ -634,69 +642,85 @@ __global__ void k_scatter_marks(Scratch s) {
 // ---------------------------------------------------------------------------
 // 3. Lattice lines.  Line (a,b), 0 <= a,b <= N, holds the lattice vertices
 //    (a,b,c).  A marked cell (i,j,k) needs c = k and c = k+1 on the lines
-//    (i,j), (i+1,j), (i,j+1), (i+1,j+1).  Each thread gathers the vertices of
-//    one line as a bit set over c = 0..N in shared memory (its own words,
-//    interleaved with the other threads' so that equal word indices hit
-//    different banks), reading the mark lists of the four columns around the
-//    line with independent loads; pass 1 counts the set bits, pass 2 writes
-//    the keys in ascending c.
+//    (i,j), (i+1,j), (i,j+1), (i+1,j+1).  A warp gathers the vertices of 32
+//    neighbouring lines (a, b0..b0+31) as bit sets over c = 0..N in shared
+//    memory: the marks of the columns (a-1, b0-1..b0+31) and (a, b0-1..b0+31)
+//    are two contiguous pieces of the grouped marks, which the lanes read
+//    together, each mark setting its bits in the two lines it touches.  (One
+//    lane per line walking its four columns' marks took 49 and 57 us at
+//    N = 512, 36 primitives: a warp waited for its longest line; now 24 and 32.)
+//    Pass 1 counts the set bits, pass 2 writes the keys in ascending c.
 // ---------------------------------------------------------------------------
 constexpr int LINES_T = 128;
 
-// the corners c = k, k + 1 of a marked cell (none for a cell marked empty)
-__device__ __forceinline__ void set_cells(uint32_t *bits, unsigned long long r) {
-    if (mark_empty(r)) return;
-    const uint32_t k = mark_k(r);
-    bits[(k >> 5) * LINES_T] |= 1u << (k & 31);
-    const uint32_t k1 = k + 1;  // k + 1 <= N
-    bits[(k1 >> 5) * LINES_T] |= 1u << (k1 & 31);
+// bits k and k + 1 of line l (word w of the line at bits[w * 32 + l])
+__device__ __forceinline__ void set_corners(uint32_t *bits, int l, uint32_t k) {
+    uint32_t *p = bits + (k >> 5) * 32 + l;
+    const uint32_t sh = k & 31;
+    atomicOr(p, 3u << sh);
+    if (sh == 31) atomicOr(p + 32, 1u);
 }
 
+// warps of a launch over the lines of an N-grid
+__host__ __device__ inline long long line_tiles(int N) { return (long long)(N + 1) * ((N + 1 + 31) / 32); }
+
+// bits: the warp's own bit sets, at least (N + 1 + 31) / 32 * 32 words
 template <bool EMIT>
 __device__ __forceinline__ void lines_pass(const GridP &g, const Scratch &s, long long t0, long long stride,
-                                           uint32_t *lbits) {
-    const int N = g.N, N1 = N + 1, NW = (N1 + 31) >> 5;
-    uint32_t *bits = lbits + threadIdx.x;  // word w at bits[w * LINES_T]
+                                           uint32_t *bits) {
+    const int N = g.N, N1 = N + 1, NW = (N1 + 31) >> 5, TPR = (N1 + 31) / 32, lane = threadIdx.x & 31;
     const unsigned long long *__restrict__ mk = s.marks_csr;
     const uint32_t *__restrict__ off = s.coloff;
-    const long long nlines = (long long)N1 * N1;
     const unsigned long long cap = (unsigned long long)s.cap_verts;
-    for (long long line = t0; line < nlines; line += stride) {
-        const int a = (int)(line / N1), b = (int)(line - (long long)a * N1);
-        for (int w = 0; w < NW; ++w) bits[w * LINES_T] = 0u;
-        for (int di = -1; di <= 0; ++di)
-            for (int dj = -1; dj <= 0; ++dj) {
-                const int i = a + di, j = b + dj;
-                if (i < 0 || j < 0 || i >= N || j >= N) continue;
-                const uint32_t col = (uint32_t)i * N + j;
-                uint32_t m = off[col];
-                const uint32_t e = off[col + 1];
-                for (; m + 4 <= e; m += 4) {
-                    const unsigned long long r0 = __ldg(mk + m), r1 = __ldg(mk + m + 1), r2 = __ldg(mk + m + 2),
-                                             r3 = __ldg(mk + m + 3);
-                    set_cells(bits, r0);
-                    set_cells(bits, r1);
-                    set_cells(bits, r2);
-                    set_cells(bits, r3);
-                }
-                for (; m < e; ++m) set_cells(bits, __ldg(mk + m));
-            }
-        if (!EMIT) {
-            uint32_t cnt = 0;
-            for (int w = 0; w < NW; ++w) cnt += (uint32_t)__popc(bits[w * LINES_T]);
-            s.linecount[line] = cnt;
-        } else {
-            unsigned long long o = s.lineoff[line];
-            for (int w = 0; w < NW; ++w) {
-                uint32_t v = bits[w * LINES_T];
-                while (v) {
-                    const int bit = __ffs(v) - 1;
-                    v &= v - 1;
-                    if (o < cap) s.vkey[o] = (unsigned long long)line | ((unsigned long long)(32 * w + bit) << 32);
-                    ++o;
+    const long long tiles = line_tiles(N);
+    for (long long t = t0; t < tiles; t += stride) {
+        const int a = (int)(t / TPR), b0 = (int)(t - (long long)a * TPR) * 32;
+        for (int w = 0; w < NW; ++w) bits[w * 32 + lane] = 0u;
+        __syncwarp();
+        const int jlo = b0 > 0 ? b0 - 1 : 0, jhi = b0 + 31 < N ? b0 + 31 : N - 1;
+#pragma unroll
+        for (int di = -1; di <= 0; ++di) {
+            const int i = a + di;
+            if (i < 0 || i >= N || jlo > jhi) continue;
+            const uint32_t c0 = (uint32_t)i * N;
+            const uint32_t m0 = off[c0 + jlo], m1 = off[c0 + jhi + 1];
+            // a wall along z puts thousands of marks in one tile: four loads in flight
+            for (uint32_t mb = m0 + lane; mb < m1; mb += 128) {
+                unsigned long long r[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) r[u] = mb + 32 * u < m1 ? __ldg(mk + mb + 32 * u) : MARK_EMPTY;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (mark_empty(r[u])) continue;
+                    const int l = (int)(mark_col(r[u]) - c0) - b0;  // line j - b0; the mark also touches line j + 1
+                    const uint32_t k = mark_k(r[u]);
+                    if (l >= 0) set_corners(bits, l, k);
+                    if (l < 31) set_corners(bits, l + 1, k);
                 }
             }
         }
+        __syncwarp();
+        const int b = b0 + lane;
+        if (b <= N) {
+            const long long line = (long long)a * N1 + b;
+            if (!EMIT) {
+                uint32_t cnt = 0;
+                for (int w = 0; w < NW; ++w) cnt += (uint32_t)__popc(bits[w * 32 + lane]);
+                s.linecount[line] = cnt;
+            } else {
+                unsigned long long o = s.lineoff[line];
+                for (int w = 0; w < NW; ++w) {
+                    uint32_t v = bits[w * 32 + lane];
+                    while (v) {
+                        const int bit = __ffs(v) - 1;
+                        v &= v - 1;
+                        if (o < cap) s.vkey[o] = (unsigned long long)line | ((unsigned long long)(32 * w + bit) << 32);
+                        ++o;
+                    }
+                }
+            }
+        }
+        __syncwarp();  // the bit sets are cleared for the warp's next tile
     }
 }
 
@@ -704,17 +728,18 @@ template <bool EMIT>
 __global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s) {
     extern __shared__ uint32_t lbits[];
     if (s.ctr->flags & STOP_FLAGS) return;
-    lines_pass<EMIT>(g, s, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x, lbits);
+    lines_pass<EMIT>(g, s, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
+                     ((long long)gridDim.x * blockDim.x) >> 5, lbits + (threadIdx.x >> 5) * ((g.N + 1 + 31) / 32) * 32);
 }
 
 void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st) {
     const long long ncols = (long long)g.N * g.N, nlines = (long long)(g.N + 1) * (g.N + 1);
-    scan_u32(s.colcount, ncols, s.coloff, s.blocksum, nullptr, 0, s.ctr, st);
+    scan_u32(s.colcount, ncols, nullptr, s.coloff, s.blocksum, nullptr, 0, s.ctr, st);
     k_scatter_marks<<<1024, 256, 0, st>>>(s);
-    const int lb = (int)((nlines + LINES_T - 1) / LINES_T);
+    const int lb = (int)((line_tiles(g.N) + LINES_T / 32 - 1) / (LINES_T / 32));
     const size_t lsm = (size_t)((g.N + 1 + 31) / 32) * LINES_T * sizeof(uint32_t);  // <= 33 KB at N = 2048
     k_lines<false><<<lb, LINES_T, lsm, st>>>(g, s);
-    scan_u32(s.linecount, nlines, s.lineoff, s.blocksum, &s.ctr->verts, s.cap_verts, s.ctr, st);
+    scan_u32(s.linecount, nlines, nullptr, s.lineoff, s.blocksum, &s.ctr->verts, s.cap_verts, s.ctr, st);
     k_lines<true><<<lb, LINES_T, lsm, st>>>(g, s);
 }
 
@@ -881,9 +906,15 @@ struct BlockSlots {
     unsigned long long t[8], c[8], tb[8], cb[8], base_t, base_c;
 };
 
+// idx (with s, for an indexed mesh): list entries of the corners c = k (the
+// next entry is c = k + 1).  Every crossing edge of a cell leaves one of its
+// corners, so a triangle's vertex numbers follow from the numbers of its
+// corners' entries without a search (a pass over the written edge keys that
+// searched each took 40 us for 1.4 M triangles).
 __device__ __forceinline__ void emit_cells(const GridP &g, Counters *ctr, const gh_mesh &out, bool valid, int i, int j,
                                            int k, const float (&fv)[8], float *stage, const McTab &tab,
-                                           BlockSlots *bs = nullptr) {
+                                           BlockSlots *bs = nullptr, const Scratch *s = nullptr,
+                                           const uint32_t *idx = nullptr) {
     const int N = g.N, N1 = N + 1;
     const unsigned long long N13 = (unsigned long long)N1 * N1 * N1;
     const int lane = threadIdx.x & 31;
@@ -975,6 +1006,11 @@ __device__ __forceinline__ void emit_cells(const GridP &g, Counters *ctr, const 
                 pos[3 * v + 1] = py;
                 pos[3 * v + 2] = pz;
             }
+            if (idx) {
+                const uint32_t li = idx[blo & 3] + (uint32_t)(blo >> 2);
+                const uint32_t id = s->ebase[li] + (uint32_t)__popc((uint32_t)s->vflag[li] & ((1u << ax) - 1u));
+                if (ti < cap) out.tri_idx[3 * ti + v] = (int32_t)id;
+            }
             key[v] = (unsigned long long)ax * N13 + (unsigned long long)la +
                      (unsigned long long)N1 * ((unsigned long long)lb + (unsigned long long)N1 * lc);
         }
@@ -995,7 +1031,9 @@ __device__ __forceinline__ void emit_cells(const GridP &g, Counters *ctr, const 
 }
 
 // Marching Cubes on the marked cells; the whole block calls, its cells start
-// at b0 and step by stride (multiples of the block size).
+// at b0 and step by stride (multiples of the block size).  INDEX: the vertices
+// are numbered (launch_index_mesh), the triangles' vertex indices are written too.
+template <bool INDEX>
 __device__ __forceinline__ void mc_cells(const GridP &g, const Scratch &s, const gh_mesh &out, float *stage,
                                          const McTab &tab, BlockSlots *bs, unsigned long long b0,
                                          unsigned long long stride) {
@@ -1018,18 +1056,19 @@ __device__ __forceinline__ void mc_cells(const GridP &g, const Scratch &s, const
                 fv[q + 4] = s.vval[idx[q] + 1];
             }
         }
-        emit_cells(g, s.ctr, out, valid, i, j, k, fv, stage, tab, bs);
+        emit_cells(g, s.ctr, out, valid, i, j, k, fv, stage, tab, bs, &s, INDEX ? idx : nullptr);
     }
 }
 
+template <bool INDEX>
 __global__ void __launch_bounds__(256) k_mc(GridP g, Scratch s, gh_mesh out) {
     __shared__ float stage[8][EMIT_STAGE];
     __shared__ McTab tab;
     __shared__ BlockSlots bs;
     if (s.ctr->flags & STOP_FLAGS) return;
     load_tab(tab);
-    mc_cells(g, s, out, stage[threadIdx.x >> 5], tab, &bs, blockIdx.x * (unsigned long long)blockDim.x,
-             (unsigned long long)gridDim.x * blockDim.x);
+    mc_cells<INDEX>(g, s, out, stage[threadIdx.x >> 5], tab, &bs, blockIdx.x * (unsigned long long)blockDim.x,
+                    (unsigned long long)gridDim.x * blockDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1104,8 +1143,9 @@ static int resident_per_sm(K kernel) {
 }
 
 void launch_mc(const GridP &g, Scratch &s, const gh_mesh &out, int nsm, cudaStream_t st) {
-    static const int per_sm = resident_per_sm(k_mc);
-    k_mc<<<nsm * per_sm, 256, 0, st>>>(g, s, out);
+    static const int per_sm = resident_per_sm(k_mc<false>), per_sm_i = resident_per_sm(k_mc<true>);
+    if (out.tri_idx) k_mc<true><<<nsm * per_sm_i, 256, 0, st>>>(g, s, out);
+    else k_mc<false><<<nsm * per_sm, 256, 0, st>>>(g, s, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1477,7 +1517,6 @@ __device__ __forceinline__ void finalize(const Scratch &s, const gh_mesh &out, l
     if (c.tris > (unsigned long long)out.capacity_tris) status = GH_ERR_CAPACITY;
     if (out.cell_ids && c.cells > (unsigned long long)out.capacity_cells) status = GH_ERR_CAPACITY;
     if (out.vert_xyz && c.mesh_verts > (unsigned long long)out.capacity_verts) status = GH_ERR_CAPACITY;
-    if (c.flags & FLAG_INDEX_MISS) status = GH_ERR_CUDA;
     if (c.flags & FLAG_TIMEOUT) status = GH_ERR_CUDA;  // the other counters are then meaningless
     if (out.n_tris) *out.n_tris = (long long)c.tris;
     if (out.n_verts) *out.n_verts = (long long)c.mesh_verts;
@@ -1517,16 +1556,32 @@ void launch_init_b(const Item *items, int n, cudaStream_t st) { k_init_b<<<n, 32
 
 __device__ __forceinline__ bool item_stopped(const Item &it) { return (it.s.ctr->flags & STOP_FLAGS) != 0; }
 
-// which = 0: column counts -> column offsets; 1: line counts -> line offsets (total = vertices)
+// which = 0: column counts -> column offsets; 1: line counts -> line offsets (total = vertices); 2: crossing
+// edges per list entry -> numbers of the mesh vertices (items with an indexed output)
+struct BatchScan {
+    const uint32_t *in;
+    uint32_t *out, *bsum;
+    unsigned long long *total;
+    long long len, cap;
+};
+
+__device__ __forceinline__ bool batch_scan(const Item &it, int which, BatchScan &q) {
+    const Scratch &s = it.s;
+    const long long N = it.g.N;
+    if (item_stopped(it)) return false;
+    if (which == 0) q = BatchScan{s.colcount, s.coloff, s.blocksum, nullptr, N * N, 0};
+    else if (which == 1) q = BatchScan{s.linecount, s.lineoff, s.blocksum, &s.ctr->verts, (N + 1) * (N + 1), s.cap_verts};
+    else q = BatchScan{s.rlist, s.ebase, s.ebsum, &s.ctr->mesh_verts, (long long)s.ctr->verts, 0};
+    return which < 2 || wants_index(it.out);
+}
+
 __global__ void __launch_bounds__(SCAN_T) k_scan_reduce_b(const Item *__restrict__ items, int n, int which) {
     __shared__ uint32_t wsum[32];
     for (int b = 0; b < n; ++b) {
-        const Item &it = items[b];
-        if (item_stopped(it)) continue;
-        const long long N = it.g.N, len = which ? (N + 1) * (N + 1) : N * N;
-        const long long nt = (len + SCAN_TILE - 1) / SCAN_TILE;
-        for (long long t = blockIdx.x; t < nt; t += gridDim.x)
-            scan_reduce_tile(which ? it.s.linecount : it.s.colcount, len, it.s.blocksum, t, wsum);
+        BatchScan q;
+        if (!batch_scan(items[b], which, q)) continue;
+        const long long nt = (q.len + SCAN_TILE - 1) / SCAN_TILE;
+        for (long long t = blockIdx.x; t < nt; t += gridDim.x) scan_reduce_tile(q.in, q.len, q.bsum, t, wsum);
     }
 }
 
@@ -1534,15 +1589,17 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_apply_b(const Item *__restrict_
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t prefix;
     for (int b = 0; b < n; ++b) {
-        const Item &it = items[b];
-        if (item_stopped(it)) continue;
-        const long long N = it.g.N, len = which ? (N + 1) * (N + 1) : N * N;
-        const long long nt = (len + SCAN_TILE - 1) / SCAN_TILE;
+        BatchScan q;
+        if (!batch_scan(items[b], which, q)) continue;
+        const long long nt = q.len > 0 ? (q.len + SCAN_TILE - 1) / SCAN_TILE : 1;
         for (long long t = blockIdx.x; t < nt; t += gridDim.x)
-            scan_apply_tile(which ? it.s.linecount : it.s.colcount, len, it.s.blocksum,
-                            which ? it.s.lineoff : it.s.coloff, which ? &it.s.ctr->verts : nullptr,
-                            which ? it.s.cap_verts : 0, &it.s.ctr->flags, t, nt, wsum, &prefix);
+            scan_apply_tile(q.in, q.len, q.bsum, q.out, q.total, q.cap, &items[b].s.ctr->flags, t, nt, wsum, &prefix);
     }
+}
+
+void launch_index_scan_b(const Item *items, int n, int nsm, cudaStream_t st) {
+    k_scan_reduce_b<<<nsm * 2, SCAN_T, 0, st>>>(items, n, 2);
+    k_scan_apply_b<<<nsm * 2, SCAN_T, 0, st>>>(items, n, 2);
 }
 
 __global__ void k_scatter_marks_b(const Item *__restrict__ items, int n) {
@@ -1555,13 +1612,14 @@ __global__ void k_scatter_marks_b(const Item *__restrict__ items, int n) {
 }
 
 template <bool EMIT>
-__global__ void __launch_bounds__(LINES_T) k_lines_b(const Item *__restrict__ items, int n) {
+__global__ void __launch_bounds__(LINES_T) k_lines_b(const Item *__restrict__ items, int n, int max_words) {
     extern __shared__ uint32_t lbits[];
+    uint32_t *bits = lbits + (threadIdx.x >> 5) * max_words * 32;  // the same place for every item: warps drift
     for (int b = 0; b < n; ++b) {
         const Item &it = items[b];
         if (item_stopped(it)) continue;
-        lines_pass<EMIT>(it.g, it.s, blockIdx.x * (long long)blockDim.x + threadIdx.x,
-                         (long long)gridDim.x * blockDim.x, lbits);
+        lines_pass<EMIT>(it.g, it.s, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
+                         ((long long)gridDim.x * blockDim.x) >> 5, bits);
     }
 }
 
@@ -1570,11 +1628,12 @@ void launch_build_lists_b(const Item *items, int n, int max_N, int nsm, cudaStre
     k_scan_reduce_b<<<grid, SCAN_T, 0, st>>>(items, n, 0);
     k_scan_apply_b<<<grid, SCAN_T, 0, st>>>(items, n, 0);
     k_scatter_marks_b<<<nsm * 8, 256, 0, st>>>(items, n);
-    const size_t lsm = (size_t)((max_N + 1 + 31) / 32) * LINES_T * sizeof(uint32_t);
-    k_lines_b<false><<<nsm * 16, LINES_T, lsm, st>>>(items, n);
+    const int mw = (max_N + 1 + 31) / 32;
+    const size_t lsm = (size_t)mw * LINES_T * sizeof(uint32_t);
+    k_lines_b<false><<<nsm * 16, LINES_T, lsm, st>>>(items, n, mw);
     k_scan_reduce_b<<<grid, SCAN_T, 0, st>>>(items, n, 1);
     k_scan_apply_b<<<grid, SCAN_T, 0, st>>>(items, n, 1);
-    k_lines_b<true><<<nsm * 16, LINES_T, lsm, st>>>(items, n);
+    k_lines_b<true><<<nsm * 16, LINES_T, lsm, st>>>(items, n, mw);
 }
 
 __global__ void __launch_bounds__(256) k_eval_vertices_csg_b(const Item *__restrict__ items, int n) {
@@ -1623,8 +1682,10 @@ __global__ void __launch_bounds__(256) k_mc_b(const Item *__restrict__ items, in
     for (int b = 0; b < n; ++b) {
         const Item &it = items[b];
         if (item_stopped(it)) continue;
-        mc_cells(it.g, it.s, it.out, stage[threadIdx.x >> 5], tab, &bs, blockIdx.x * (unsigned long long)blockDim.x,
-                 (unsigned long long)gridDim.x * blockDim.x);
+        const unsigned long long b0 = blockIdx.x * (unsigned long long)blockDim.x;
+        const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+        if (it.out.tri_idx) mc_cells<true>(it.g, it.s, it.out, stage[threadIdx.x >> 5], tab, &bs, b0, stride);
+        else mc_cells<false>(it.g, it.s, it.out, stage[threadIdx.x >> 5], tab, &bs, b0, stride);
     }
 }
 
