@@ -253,6 +253,8 @@ struct gh_sdb {
 struct PoolEntry {
     Scratch scr;
     int N, device;
+    float *adj;  // adjoint work buffer (neural SDBs that were differentiated)
+    size_t adj_floats;
 };
 static std::mutex g_pool_mu;
 static std::vector<PoolEntry> g_pool;
@@ -347,13 +349,23 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     // (k_prep.cu); layer 0, biases of layer 0 and the output layer are read
     // in place from the uploaded block
     const size_t WW = (size_t)W * W;
-    float *d_wt, *d_wtb, *d_bm;
-    uint16_t *d_wbf, *d_wx6, *d_wx6t;
-    if (dev_alloc(s, &s->d_params, (size_t)np) || dev_alloc(s, &d_wt, (size_t)h.n_mid * WW) ||
-        dev_alloc(s, &d_wtb, (size_t)h.n_mid * WW) || dev_alloc(s, &d_bm, (size_t)h.n_mid * W) ||
-        dev_alloc(s, &d_wbf, (size_t)h.n_mid * WW) || dev_alloc(s, &d_wx6, (size_t)3 * h.n_mid * WW) ||
-        dev_alloc(s, &d_wx6t, (size_t)3 * h.n_mid * WW))
+    // (one allocation for all of them: each costs the host tens of microseconds
+    // to make and to free, and a training step makes a new SDB)
+    const size_t mw = (size_t)h.n_mid * WW;
+    auto up = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
+    unsigned char *base;
+    if (dev_alloc(s, &base, up(sizeof(float) * np) + 2 * up(sizeof(float) * mw) + up(sizeof(float) * h.n_mid * W) +
+                                up(2 * mw) + 2 * up(6 * mw)))
         return GH_ERR_CUDA;
+    auto take = [&](size_t bytes) {
+        unsigned char *p = base;
+        base += up(bytes);
+        return (void *)p;
+    };
+    s->d_params = (float *)take(sizeof(float) * np);
+    float *d_wt = (float *)take(sizeof(float) * mw), *d_wtb = (float *)take(sizeof(float) * mw);
+    float *d_bm = (float *)take(sizeof(float) * h.n_mid * W);
+    uint16_t *d_wbf = (uint16_t *)take(2 * mw), *d_wx6 = (uint16_t *)take(6 * mw), *d_wx6t = (uint16_t *)take(6 * mw);
     GH_CUDA(cudaMemcpy(s->d_params, P, sizeof(float) * np, cudaMemcpyHostToDevice));
     launch_prep_mlp(s->d_params, W, h.n_mid, d_wt, d_wtb, d_wbf, d_wx6, d_wx6t, d_bm, 0);
     GH_CUDA(cudaGetLastError());
@@ -393,6 +405,7 @@ extern "C" int gh_release_cache(void) {
                         c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.cull};
         for (void *p : ptrs)
             if (p) cudaFree(p);
+        if (e.adj) cudaFree(e.adj);
     }
     g_pool.clear();
     cudaSetDevice(cur);
@@ -435,21 +448,28 @@ static void free_scratch(gh_sdb *s) {
     s->scr_N = 0;
 }
 
+// Adjoint buffers above this (1 GB: 2 (n_mid + 1) width floats per vertex, 85 k
+// vertices at width 256 and 5 hidden layers) stay out of the pool.
+constexpr size_t POOL_ADJ_FLOATS = (size_t)1 << 28;
+
 extern "C" int gh_destroy_sdb(gh_sdb *s) {
     if (!s) return GH_OK;
+    // these frees wait for the device, so the pooled buffers below are idle
+    if (s->seeds) cudaFree(s->seeds);
+    if (s->d_item) cudaFree(s->d_item);
+    for (void *p : s->dbufs) cudaFree(p);
     if (s->scr.ctr) {
         std::lock_guard<std::mutex> lk(g_pool_mu);
         if (g_pool.size() < POOL_MAX) {
-            g_pool.push_back(PoolEntry{s->scr, s->scr_N, s->device});
+            const bool keep = s->adj_floats <= POOL_ADJ_FLOATS;
+            g_pool.push_back(PoolEntry{s->scr, s->scr_N, s->device, keep ? s->adj : nullptr, keep ? s->adj_floats : 0});
             s->scr = Scratch{};
             s->scr_N = 0;
+            if (keep) s->adj = nullptr;
         }
     }
     free_scratch(s);
     if (s->adj) cudaFree(s->adj);
-    if (s->seeds) cudaFree(s->seeds);
-    if (s->d_item) cudaFree(s->d_item);
-    for (void *p : s->dbufs) cudaFree(p);
     delete s;
     return GH_OK;
 }
@@ -466,6 +486,13 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
                 c = e.scr;
                 s->scr_N = e.N;
                 s->item_valid = false;
+                if (s->adj_floats < e.adj_floats) {
+                    if (s->adj) cudaFree(s->adj);
+                    s->adj = e.adj;
+                    s->adj_floats = e.adj_floats;
+                } else if (e.adj) {
+                    cudaFree(e.adj);
+                }
                 g_pool.erase(g_pool.begin() + (long)q);
                 break;
             }
@@ -1081,7 +1108,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         launch_index_mesh_b(P.d_items, B, nsm, st);
         launches += 4;
     }
-    launch_mc_b(P.d_items, B, nsm, st);
+    launch_mc_b(P.d_items, B, any_index, nsm, st);
     launch_finalize_b(P.d_items, B, st);
     g_prof.recorded = false;
     g_prof.launches = launches;
@@ -1300,8 +1327,9 @@ extern "C" int gh_backward(const gh_sdb *cs, const float *verts, const float *dL
     std::lock_guard<std::mutex> lk(s->mu);
     const int W = s->mlp.width, L = s->mlp.n_mid, S = 76;  // 2 x 76 weight-gradient tiles: one per SM
     // vertices per chunk: the stored activations and deltas of a chunk take
-    // 2 (L + 1) W floats per vertex (1.6 GB at W = 256, L = 5)
-    constexpr int VCHUNK = GH_ADJOINT_CHUNK;
+    // 2 (L + 1) W floats per vertex (1.6 GB at W = 256, L = 5, a full chunk; a
+    // smaller mesh takes no more than its vertices need)
+    const int VCHUNK = V < GH_ADJOINT_CHUNK ? (int)((V + 4095) / 4096 * 4096) : GH_ADJOINT_CHUNK;
     const size_t need = adjoint_buffer_floats(W, L, VCHUNK, S, nsm);
     if (s->adj_floats < need) {
         if (s->adj) cudaFree(s->adj);

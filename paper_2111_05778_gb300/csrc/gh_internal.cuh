@@ -235,7 +235,7 @@ void launch_init_b(const Item *items, int n, cudaStream_t st);
 void launch_build_lists_b(const Item *items, int n, int max_N, int nsm, cudaStream_t st);
 void launch_eval_vertices_csg_b(const Item *items, int n, int max_prims, int nsm, cudaStream_t st);
 void launch_refine_select_b(const Item *items, int n, int nsm, cudaStream_t st);  // neural items only
-void launch_mc_b(const Item *items, int n, int nsm, cudaStream_t st);
+void launch_mc_b(const Item *items, int n, bool index, int nsm, cudaStream_t st);
 void launch_finalize_b(const Item *items, int n, cudaStream_t st);
 // continuation (Sec. 2) for analytic SDBs: seed search from host-given points
 // (seeds: device [n][3]) and the surface crawl with Marching Cubes per cell

@@ -1056,7 +1056,7 @@ __device__ __forceinline__ void mc_cells(const GridP &g, const Scratch &s, const
                 fv[q + 4] = s.vval[idx[q] + 1];
             }
         }
-        emit_cells(g, s.ctr, out, valid, i, j, k, fv, stage, tab, bs, &s, INDEX ? idx : nullptr);
+        emit_cells(g, s.ctr, out, valid, i, j, k, fv, stage, tab, bs, &s, INDEX && out.tri_idx ? idx : nullptr);
     }
 }
 
@@ -1674,24 +1674,32 @@ void launch_refine_select_b(const Item *items, int n, int nsm, cudaStream_t st) 
     for (int phase = 0; phase < 3; ++phase) k_refine_b<<<nsm * 8, 256, 0, st>>>(items, n, phase);
 }
 
-__global__ void __launch_bounds__(256) k_mc_b(const Item *__restrict__ items, int n) {
+// The item's descriptor is staged in shared memory: held in registers (80 a
+// thread instead of 48) it cost a third of the resident warps that hide this
+// kernel's loads.
+template <bool INDEX>
+__global__ void __launch_bounds__(256, 5) k_mc_b(const Item *__restrict__ items, int n) {
     __shared__ float stage[8][EMIT_STAGE];
     __shared__ McTab tab;
     __shared__ BlockSlots bs;
+    __shared__ Item it;
     load_tab(tab);
     for (int b = 0; b < n; ++b) {
-        const Item &it = items[b];
-        if (item_stopped(it)) continue;
-        const unsigned long long b0 = blockIdx.x * (unsigned long long)blockDim.x;
-        const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-        if (it.out.tri_idx) mc_cells<true>(it.g, it.s, it.out, stage[threadIdx.x >> 5], tab, &bs, b0, stride);
-        else mc_cells<false>(it.g, it.s, it.out, stage[threadIdx.x >> 5], tab, &bs, b0, stride);
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(items + b);
+        for (int i = threadIdx.x; i < (int)(sizeof(Item) / 4); i += blockDim.x) reinterpret_cast<uint32_t *>(&it)[i] = src[i];
+        __syncthreads();
+        if (!item_stopped(it))
+            mc_cells<INDEX>(it.g, it.s, it.out, stage[threadIdx.x >> 5], tab, &bs,
+                            blockIdx.x * (unsigned long long)blockDim.x, (unsigned long long)gridDim.x * blockDim.x);
+        __syncthreads();  // the next item's descriptor replaces this one
     }
 }
 
-void launch_mc_b(const Item *items, int n, int nsm, cudaStream_t st) {
-    static const int per_sm = resident_per_sm(k_mc_b);
-    k_mc_b<<<nsm * per_sm, 256, 0, st>>>(items, n);
+// index: some item wants triangle indices
+void launch_mc_b(const Item *items, int n, bool index, int nsm, cudaStream_t st) {
+    static const int per_sm = resident_per_sm(k_mc_b<false>), per_sm_i = resident_per_sm(k_mc_b<true>);
+    if (index) k_mc_b<true><<<nsm * per_sm_i, 256, 0, st>>>(items, n);
+    else k_mc_b<false><<<nsm * per_sm, 256, 0, st>>>(items, n);
 }
 
 __global__ void k_finalize_b(const Item *__restrict__ items, int n) {

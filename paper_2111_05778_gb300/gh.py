@@ -290,8 +290,9 @@ class Buffers:
         self.cell_cases = torch.empty(max(self.cap_cells, 1), dtype=torch.uint8, device=dev) if cap_cells else None
         self.verts = torch.empty((max(self.cap_verts, 1), 3), dtype=torch.float32, device=dev) if cap_verts else None
         self.faces = torch.empty((max(self.cap_tris, 1), 3), dtype=torch.int32, device=dev) if cap_verts else None
-        self.counts = torch.zeros(3, dtype=torch.int64, device=dev)  # n_tris, n_cells, n_verts
-        self.stats = torch.zeros(16, dtype=torch.int64, device=dev)
+        self._results = torch.zeros(19, dtype=torch.int64, device=dev)  # one block: one copy reads both
+        self.counts = self._results[:3]  # n_tris, n_cells, n_verts
+        self.stats = self._results[3:]
         self.desc = MeshDesc()
         d = self.desc
         d.tri_xyz = self.tri_xyz.data_ptr()
@@ -311,6 +312,11 @@ class Buffers:
     def stats_dict(self):
         v = self.stats.cpu().numpy()
         return {n: int(v[i]) for i, n in enumerate(STAT_FIELDS)}
+
+    def results(self):
+        """(counts, stats_dict()) in one copy to the host."""
+        v = self._results.cpu().numpy()
+        return v[:3], {n: int(v[3 + i]) for i, n in enumerate(STAT_FIELDS)}
 
 
 def options(precision="fp32", tau_mode=GH_TAU_DIAGONAL, eps=None, sync=True, ray_block=0, mlp_tiles=0,
@@ -346,18 +352,20 @@ def polygonize(sdb: Sdb, N, lo=-1.0, hi=1.0, precision="fp32", tau_mode=GH_TAU_D
     the on-device indexed mesh (Mesh.verts, Mesh.faces)."""
     keys = bool(keys) or bool(indexed)
     key = (int(N), keys, bool(cells), bool(indexed))
-    cap = sdb._cap.get(key, 4 * int(N) * int(N) + 4096)
+    # first guess of the triangles: 4 per column for one closed surface, 8 for a
+    # scene (a guess too small costs a second polygonization)
+    cap = sdb._cap.get(key, (8 if sdb.kind == GH_SDB_CSG else 4) * int(N) * int(N) + 4096)
     for _ in range(3):
         capv = cap // 2 + 4096 if indexed else 0
         bufs = Buffers(cap, keys=keys, cap_cells=cap if cells else 0, cap_verts=capv)
         rc = polygonize_into(sdb, N, bufs, lo, hi, precision, tau_mode, eps, True, stream, method=method)
-        counts = bufs.counts.cpu().numpy()
+        counts, stats = bufs.results()
         if rc == GH_OK:
             sdb._cap[key] = cap
             T, C, V = int(counts[0]), int(counts[1]), int(counts[2])
             return Mesh(bufs.tri_xyz[:T], bufs.tri_keys[:T] if keys else None,
                         bufs.cell_ids[:C] if cells else None, bufs.cell_cases[:C] if cells else None,
-                        bufs.stats_dict(), bufs.verts[:V] if indexed else None,
+                        stats, bufs.verts[:V] if indexed else None,
                         bufs.faces[:T] if indexed else None)
         cap = int(max(counts[0], counts[1], 2 * counts[2]) * 1.1) + 4096
     raise GhError(GH_ERR_CAPACITY, "output buffers kept overflowing")
@@ -448,12 +456,13 @@ class Batch:
 
     def mesh(self, b) -> "Mesh":
         bb = self.bufs[b]
-        T, C, V = [int(x) for x in bb.counts.cpu().numpy()]
+        counts, stats = bb.results()
+        T, C, V = [int(x) for x in counts]
         ind = bb.verts is not None
         cl = bb.cell_ids is not None
         return Mesh(bb.tri_xyz[:T], bb.tri_keys[:T] if bb.tri_keys is not None else None,
                     bb.cell_ids[:C] if cl else None, bb.cell_cases[:C] if cl else None,
-                    bb.stats_dict(), bb.verts[:V] if ind else None, bb.faces[:T] if ind else None)
+                    stats, bb.verts[:V] if ind else None, bb.faces[:T] if ind else None)
 
 
 def polygonize_batch(sdbs, Ns, lo=-1.0, hi=1.0, precision="fp32", keys=False, eps=None, ray_block=0, mlp_tiles=0,
