@@ -402,7 +402,7 @@ extern "C" int gh_release_cache(void) {
         cudaSetDevice(e.device);
         Scratch &c = e.scr;
         void *ptrs[] = {c.ctr, c.marks_raw, c.marks_csr, c.colcount, c.coloff, c.linecount, c.lineoff,
-                        c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.cull};
+                        c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.lb, c.lbe, c.cull};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         if (e.adj) cudaFree(e.adj);
@@ -441,7 +441,7 @@ extern "C" int gh_create_sdb(const gh_sdb_desc *desc, gh_sdb **out) {
 static void free_scratch(gh_sdb *s) {
     Scratch &c = s->scr;
     void *ptrs[] = {c.ctr, c.marks_raw, c.marks_csr, c.colcount, c.coloff, c.linecount, c.lineoff,
-                    c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.cull};
+                    c.blocksum, c.vkey, c.vval, c.vflag, c.rlist, c.lat, c.ebase, c.ebsum, c.vis, c.lb, c.lbe, c.cull};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     s->scr = Scratch{};
@@ -529,6 +529,9 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
     GH_CUDA(cudaMalloc((void **)&c.linecount, sizeof(uint32_t) * nlines));
     GH_CUDA(cudaMalloc((void **)&c.lineoff, sizeof(uint32_t) * (nlines + 1)));
     GH_CUDA(cudaMalloc((void **)&c.blocksum, sizeof(uint32_t) * 4096));
+    GH_CUDA(cudaMalloc((void **)&c.lb, sizeof(unsigned long long) * lb_words(NN)));
+    GH_CUDA(cudaMemset(c.lb, 0, sizeof(unsigned long long) * lb_words(NN)));  // call number 0, no words written
+    GH_CUDA(cudaStreamSynchronize(0));
     GH_CUDA(cudaMalloc((void **)&c.vkey, sizeof(unsigned long long) * cv));
     GH_CUDA(cudaMalloc((void **)&c.vval, sizeof(float) * cv));
     GH_CUDA(cudaMalloc((void **)&c.vflag, cv));
@@ -558,11 +561,16 @@ static int ensure_index(gh_sdb *s) {
     if (c.cap_index >= c.cap_verts && c.ebase) return GH_OK;
     if (c.ebase) cudaFree(c.ebase);
     if (c.ebsum) cudaFree(c.ebsum);
+    if (c.lbe) cudaFree(c.lbe);
     c.ebase = nullptr;
     c.ebsum = nullptr;
+    c.lbe = nullptr;
     c.cap_index = 0;
     GH_CUDA(cudaMalloc((void **)&c.ebase, sizeof(uint32_t) * (c.cap_verts + 1)));
     GH_CUDA(cudaMalloc((void **)&c.ebsum, sizeof(uint32_t) * scan_partials(c.cap_verts)));
+    GH_CUDA(cudaMalloc((void **)&c.lbe, sizeof(unsigned long long) * lbe_words(c.cap_verts)));
+    GH_CUDA(cudaMemset(c.lbe, 0, sizeof(unsigned long long) * lbe_words(c.cap_verts)));
+    GH_CUDA(cudaStreamSynchronize(0));
     c.cap_index = c.cap_verts;
     s->item_valid = false;
     return GH_OK;
@@ -680,7 +688,7 @@ static inline void mark_phase(int i, cudaStream_t st) {
 }
 
 // Kernel launches per phase (fixed by the launch sequence below).
-static constexpr int LAUNCHES_HOP = 2, LAUNCHES_LISTS = 7, LAUNCHES_VERTS = 1, LAUNCHES_REFINE = 4,
+static constexpr int LAUNCHES_HOP = 2, LAUNCHES_LISTS = 3, LAUNCHES_VERTS = 1, LAUNCHES_REFINE = 4,
                      LAUNCHES_MC = 2;
 
 // FP32 evaluation of a neural SDB: on the tensor cores with split-BF16
@@ -1424,7 +1432,7 @@ extern "C" int gh_polygonize_csg_noalloc(const gh_grid *grid, const gh_csg_prim 
     off += up256(4 * nlines);
     c.lineoff = (uint32_t *)(q + off);
     off += up256(4 * (nlines + 1));
-    c.blocksum = (uint32_t *)(q + off);
+    c.lb = (unsigned long long *)(q + off);  // at most 1 + 16 + 579 words, zero at load
     off += up256(4 * 4096);
     const size_t per = 2 * 8 + 2 * (8 + 4);  // marks raw + grouped, two vertices (key + value) per mark
     const size_t M = ((GH_NOALLOC_SCRATCH_BYTES - off - 4 * 256) / per) & ~(size_t)255;

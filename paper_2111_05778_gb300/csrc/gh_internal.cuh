@@ -25,7 +25,8 @@ struct Counters {
     unsigned long long mesh_verts; // indexed output: crossing lattice edges
     unsigned long long q_head;     // continuation: next queue slot to take
     unsigned long long q_pending;  // continuation: cells queued and not yet finished
-    unsigned long long pad[2];
+    unsigned long long tick[3];    // tiles taken by the one-pass scans: columns, lines, edges
+    unsigned long long pad[1];
 };
 
 enum : unsigned long long {
@@ -171,6 +172,8 @@ struct Scratch {
     long long cap_index;            // entries ebase was sized for (0: none)
     uint32_t *vis;                  // continuation: visited bit per cell [N^3 / 32 words]
     long long cap_vis;              // words of vis
+    unsigned long long *lb;         // one-pass scans: [0] call number, then a status word per tile of columns and lines
+    unsigned long long *lbe;        // the same per tile of list entries (indexed output)
     uint32_t *cull;                 // analytic SDBs: primitive masks per block of cells (NULL: fold every primitive)
     long long cap_cull;             // words of cull
 };
@@ -272,12 +275,10 @@ void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, flo
 // space (n_mid x ceil(V/128)*128 x W/32 words)
 void launch_adj_mlp_x6(const MlpDev &m, const float *P, const float *dL, long long V, float *A, float *D, float *s,
                        uint32_t *mask, long long ldl, int nsm, cudaStream_t st);
-// exclusive scan of *n <= nmax uint32 into out[0..*n] (k_pipeline.cu); bsum
-// holds ceil(nmax / 4096) partials; *total gets the sum
-void scan_u32_dev(const uint32_t *in, long long nmax, const unsigned long long *n, uint32_t *out, uint32_t *bsum,
-                  unsigned long long *total, Counters *ctr, cudaStream_t st);
 void launch_index_scan_b(const Item *items, int n, int nsm, cudaStream_t st);  // of the items with an indexed output
 long long scan_partials(long long n);
+long long lb_words(int N);              // words of Scratch::lb
+long long lbe_words(long long nverts);  // words of Scratch::lbe
 // derived weight layouts of a neural SDB from its packed parameters (k_prep.cu)
 void launch_prep_mlp(const float *params, int W, int n_mid, float *wt, float *wtb, uint16_t *wbf, uint16_t *wx6,
                      uint16_t *wx6t, float *bm, cudaStream_t st);

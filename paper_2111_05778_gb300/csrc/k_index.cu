@@ -17,6 +17,7 @@
 // Marching Cubes interpolation t = f(A) / (f(A) - f(B)) from A with the same
 // operations, so they are bit-identical to the triangle soup's.
 #include "gh_internal.cuh"
+#include "lookback.cuh"
 
 namespace gh {
 
@@ -35,77 +36,149 @@ __device__ __forceinline__ long long find_point(const Scratch &s, uint32_t line,
     return (uint32_t)(s.vkey[lo] >> 32) == c ? (long long)lo : -1;
 }
 
-// Walks the list: visit(v, a, b, c, f, fn, m) for each entry v: its lattice
-// coordinates and value, the value fn[ax] of the upper end point of its edge
-// along each axis, and the mask m of the axes whose edge crosses.
-template <typename F>
-__device__ __forceinline__ void walk_edges(const GridP &g, const Scratch &s, unsigned long long t0,
-                                           unsigned long long stride, F visit) {
-    const unsigned long long V = s.ctr->verts;
+// A list entry: its lattice coordinates and value, the value fn[ax] of the
+// upper end point of its edge along each axis, and the mask m of the axes whose
+// edge crosses.  hint[ax]: where the upper end point along x and y is looked
+// for first (one past the entry before's); returned for the next entry.
+struct Edges {
+    uint32_t a, b, c;
+    float f, fn[3];
+    int m;
+};
+
+__device__ __forceinline__ Edges edges_of(const GridP &g, const Scratch &s, unsigned long long v, unsigned long long V,
+                                          long long (&hint)[2]) {
     const uint32_t N = (uint32_t)g.N, N1 = N + 1;
-    for (unsigned long long v = t0; v < V; v += stride) {
-        const unsigned long long key = s.vkey[v];
-        const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), c = (uint32_t)(key >> 32);
-        const uint32_t a = line / N1, b = line - a * N1;
-        const float f = s.vval[v];
-        const bool neg = f < 0.f;
-        const long long nx = a < N ? find_point(s, line + N1, c) : -1;
-        const long long ny = b < N ? find_point(s, line + 1, c) : -1;
-        const unsigned long long kz = v + 1 < V ? s.vkey[v + 1] : ~0ull;  // upper neighbour along z, if it is one
-        const long long nz = (uint32_t)(kz & 0xFFFFFFFFull) == line && (uint32_t)(kz >> 32) == c + 1u ? (long long)v + 1 : -1;
-        const long long nb[3] = {nx, ny, nz};
-        float fn[3] = {0.f, 0.f, 0.f};
-        int m = 0;
+    const unsigned long long key = s.vkey[v];
+    const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull);
+    Edges e;
+    e.c = (uint32_t)(key >> 32);
+    e.a = line / N1;
+    e.b = line - e.a * N1;
+    e.f = s.vval[v];
+    e.fn[0] = e.fn[1] = e.fn[2] = 0.f;
+    e.m = 0;
+    const bool neg = e.f < 0.f;
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax)
-            if (nb[ax] >= 0) {
-                fn[ax] = s.vval[nb[ax]];
-                if ((fn[ax] < 0.f) != neg) m |= 1 << ax;
-            }
-        visit(v, a, b, c, f, fn, m);
+    for (int ax = 0; ax < 2; ++ax) {
+        if ((ax == 0 ? e.a : e.b) >= N) {
+            hint[ax] = -1;
+            continue;
+        }
+        const uint32_t nline = ax == 0 ? line + N1 : line + 1u;
+        const unsigned long long want = (unsigned long long)nline | ((unsigned long long)e.c << 32);
+        long long nb = hint[ax];
+        if (nb < 0 || (unsigned long long)nb >= V || s.vkey[nb] != want) nb = find_point(s, nline, e.c);
+        hint[ax] = nb >= 0 ? nb + 1 : -1;
+        if (nb >= 0) {
+            e.fn[ax] = s.vval[nb];
+            if ((e.fn[ax] < 0.f) != neg) e.m |= 1 << ax;
+        }
+    }
+    if (v + 1 < V && s.vkey[v + 1] == key + (1ull << 32)) {  // the next entry: the upper neighbour along z, if it is one
+        e.fn[2] = s.vval[v + 1];
+        if ((e.fn[2] < 0.f) != neg) e.m |= 4;
+    }
+    return e;
+}
+
+// The positions of an entry's vertices, numbered from id on.
+__device__ __forceinline__ void put_vertices(const GridP &g, const gh_mesh &out, const Edges &e, unsigned long long id) {
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        if (!(e.m & (1 << ax))) continue;
+        const float tt = e.f / (e.f - e.fn[ax]);
+        float px = fmaf((float)e.a, g.h, g.lo[0]);
+        float py = fmaf((float)e.b, g.h, g.lo[1]);
+        float pz = fmaf((float)e.c, g.h, g.lo[2]);
+        if (ax == 0) px = fmaf(tt, g.h, px);
+        else if (ax == 1) py = fmaf(tt, g.h, py);
+        else pz = fmaf(tt, g.h, pz);
+        if (id < (unsigned long long)out.capacity_verts) {
+            out.vert_xyz[3 * id] = px;
+            out.vert_xyz[3 * id + 1] = py;
+            out.vert_xyz[3 * id + 2] = pz;
+        }
+        ++id;
     }
 }
 
-// per list entry: the crossing mask (into vflag) and its population (into
-// rlist, whose refinement list is no longer needed)
-__device__ __forceinline__ void edge_count(const GridP &g, const Scratch &s, unsigned long long t0,
-                                           unsigned long long stride) {
-    walk_edges(g, s, t0, stride, [&](unsigned long long v, uint32_t, uint32_t, uint32_t, float, const float(&)[3], int m) {
-        s.vflag[v] = (uint8_t)m;
-        s.rlist[v] = (uint32_t)__popc(m);
-    });
-}
+// One call: count, number and emit in one pass.  Blocks take tiles of 1,024
+// entries; a thread has four consecutive ones, whose neighbours mostly follow
+// each other too, so that only the first is searched for.  (A counting pass, a
+// two-pass scan and an emitting pass took 61 us for 1.6 M entries, this 55, and
+// at 10 k entries three launches less count more.)
+constexpr int EDGE_T = 256, EDGE_E = 4, EDGE_TILE = EDGE_T * EDGE_E;
 
-__device__ __forceinline__ void emit_vertices(const GridP &g, const Scratch &s, const gh_mesh &out,
-                                              unsigned long long t0, unsigned long long stride) {
-    walk_edges(g, s, t0, stride, [&](unsigned long long v, uint32_t a, uint32_t b, uint32_t c, float fa,
-                                     const float(&fn)[3], int m) {
-        if (!m) return;
-        unsigned long long id = s.ebase[v];
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            if (!(m & (1 << ax))) continue;
-            const float tt = fa / (fa - fn[ax]);
-            float px = fmaf((float)a, g.h, g.lo[0]);
-            float py = fmaf((float)b, g.h, g.lo[1]);
-            float pz = fmaf((float)c, g.h, g.lo[2]);
-            if (ax == 0) px = fmaf(tt, g.h, px);
-            else if (ax == 1) py = fmaf(tt, g.h, py);
-            else pz = fmaf(tt, g.h, pz);
-            if (id < (unsigned long long)out.capacity_verts) {
-                out.vert_xyz[3 * id] = px;
-                out.vert_xyz[3 * id + 1] = py;
-                out.vert_xyz[3 * id + 2] = pz;
-            }
-            ++id;
-        }
-    });
-}
-
-__global__ void __launch_bounds__(256) k_emit_vertices(GridP g, Scratch s, gh_mesh out) {
+__global__ void __launch_bounds__(EDGE_T) k_edges(GridP g, Scratch s, gh_mesh out) {
+    __shared__ uint32_t wsum[EDGE_T / 32], base_s;
+    __shared__ unsigned long long tile_s;
     if (s.ctr->flags & STOPF) return;
+    const unsigned long long V = s.ctr->verts;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (;;) {
+        if (threadIdx.x == 0) tile_s = atomicAdd(&s.ctr->tick[2], 1ull);
+        __syncthreads();
+        const unsigned long long tile = tile_s, v0 = tile * EDGE_TILE + (unsigned long long)threadIdx.x * EDGE_E;
+        if (tile * EDGE_TILE >= V) return;
+        Edges e[EDGE_E];
+        long long hint[2] = {-1, -1};
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int k = 0; k < EDGE_E; ++k) {
+            e[k].m = 0;
+            if (v0 + k < V) {
+                e[k] = edges_of(g, s, v0 + k, V, hint);
+                s.vflag[v0 + k] = (uint8_t)e[k].m;
+                cnt += (uint32_t)__popc(e[k].m);
+            }
+        }
+        uint32_t x = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[wid] = x;
+        __syncthreads();
+        uint32_t tot = 0, wb = 0;
+        for (int q = 0; q < EDGE_T / 32; ++q) {
+            if (q < wid) wb += wsum[q];
+            tot += wsum[q];
+        }
+        if (wid == 0) {
+            const uint32_t p = lb_prefix(s.lbe, s.lb[0], (long long)tile, tot, s.ctr);
+            if (lane == 0) base_s = p;
+        }
+        __syncthreads();
+        uint32_t id = base_s + wb + x - cnt;
+#pragma unroll
+        for (int k = 0; k < EDGE_E; ++k) {
+            if (v0 + k >= V) break;
+            s.ebase[v0 + k] = id;
+            if (out.vert_xyz && e[k].m) put_vertices(g, out, e[k], id);
+            id += (uint32_t)__popc(e[k].m);
+            if (v0 + k == V - 1) s.ctr->mesh_verts = id;
+        }
+        __syncthreads();  // tile_s and the sums are rewritten
+    }
+}
+
+// Batches: counted, scanned (two passes) and emitted over all items, grid
+// strides without tickets.  Per entry the crossing mask goes into vflag and its
+// population into rlist, whose refinement list is no longer needed.
+__global__ void __launch_bounds__(256) k_edge_count_b(const Item *__restrict__ items, int n) {
     const unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-    emit_vertices(g, s, out, t, (unsigned long long)gridDim.x * blockDim.x);
+    for (int b = 0; b < n; ++b) {
+        const Item &it = items[b];
+        if (!wants_index(it.out) || (it.s.ctr->flags & STOPF)) continue;
+        const unsigned long long V = it.s.ctr->verts;
+        for (unsigned long long v = t; v < V; v += (unsigned long long)gridDim.x * blockDim.x) {
+            long long hint[2] = {-1, -1};
+            const Edges e = edges_of(it.g, it.s, v, V, hint);
+            it.s.vflag[v] = (uint8_t)e.m;
+            it.s.rlist[v] = (uint32_t)__popc(e.m);
+        }
+    }
 }
 
 __global__ void __launch_bounds__(256) k_emit_vertices_b(const Item *__restrict__ items, int n) {
@@ -113,34 +186,21 @@ __global__ void __launch_bounds__(256) k_emit_vertices_b(const Item *__restrict_
     for (int b = 0; b < n; ++b) {
         const Item &it = items[b];
         if (!it.out.vert_xyz || (it.s.ctr->flags & STOPF)) continue;
-        emit_vertices(it.g, it.s, it.out, t, (unsigned long long)gridDim.x * blockDim.x);
-    }
-}
-
-__global__ void __launch_bounds__(256) k_edge_count(GridP g, Scratch s) {
-    if (s.ctr->flags & STOPF) return;
-    const unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-    edge_count(g, s, t, (unsigned long long)gridDim.x * blockDim.x);
-}
-
-__global__ void __launch_bounds__(256) k_edge_count_b(const Item *__restrict__ items, int n) {
-    const unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-    for (int b = 0; b < n; ++b) {
-        const Item &it = items[b];
-        if (!wants_index(it.out) || (it.s.ctr->flags & STOPF)) continue;
-        edge_count(it.g, it.s, t, (unsigned long long)gridDim.x * blockDim.x);
+        const unsigned long long V = it.s.ctr->verts;
+        for (unsigned long long v = t; v < V; v += (unsigned long long)gridDim.x * blockDim.x) {
+            if (!it.s.vflag[v]) continue;
+            long long hint[2] = {-1, -1};
+            put_vertices(it.g, it.out, edges_of(it.g, it.s, v, V, hint), it.s.ebase[v]);
+        }
     }
 }
 
 }  // namespace
 
+long long lbe_words(long long nverts) { return nverts / EDGE_TILE + 1; }
+
 void launch_index_mesh(const GridP &g, Scratch &s, const gh_mesh &out, int nsm, cudaStream_t st) {
-    const long long n = s.cap_verts;
-    long long nb = (n + 255) / 256;
-    if (nb > nsm * 8) nb = nsm * 8;
-    k_edge_count<<<(int)nb, 256, 0, st>>>(g, s);
-    scan_u32_dev(s.rlist, n, &s.ctr->verts, s.ebase, s.ebsum, &s.ctr->mesh_verts, s.ctr, st);
-    if (out.vert_xyz) k_emit_vertices<<<(int)nb, 256, 0, st>>>(g, s, out);
+    k_edges<<<nsm * 4, EDGE_T, 0, st>>>(g, s, out);
 }
 
 void launch_index_mesh_b(const Item *items, int n, int nsm, cudaStream_t st) {

@@ -19,6 +19,7 @@
 //                     lookup, edge interpolation, warp prefix-sum emit with one
 //                     atomic per warp.
 #include "gh_internal.cuh"
+#include "lookback.cuh"
 
 namespace gh {
 
@@ -346,12 +347,13 @@ void launch_stage_prims(const Prim *src, Prim *dst, int nprim, cudaStream_t st) 
 }
 
 // ---------------------------------------------------------------------------
-__global__ void k_init(Counters *c) {
+__global__ void k_init(Counters *c, unsigned long long *lb) {
+    if (threadIdx.x == 0) lb[0] = (lb[0] + 1ull) & 0x3FFFFFFFull;  // this call's number (lookback.cuh)
     unsigned long long *p = reinterpret_cast<unsigned long long *>(c);
     if (threadIdx.x < sizeof(Counters) / 8) p[threadIdx.x] = 0ull;
 }
 
-void launch_init(Scratch &s, cudaStream_t st) { k_init<<<1, 32, 0, st>>>(s.ctr); }
+void launch_init(Scratch &s, cudaStream_t st) { k_init<<<1, 32, 0, st>>>(s.ctr, s.lb); }
 
 // ---------------------------------------------------------------------------
 // 1. Persistent hopper for analytic SDBs over a batch of items.  Lanes take
@@ -507,8 +509,8 @@ void launch_hop_csg(const Item *items, int n_items, int max_prims, int nsm, int 
 }
 
 // ---------------------------------------------------------------------------
-// 2. Exclusive scan of uint32 counts (two passes; out has n + 1 entries and
-//    out[n] is the total, also stored in *total when total != NULL).
+// 2. Exclusive scan of uint32 counts (batches: two passes; out has n + 1
+//    entries and out[n] is the total, also stored in *total when total != NULL).
 // ---------------------------------------------------------------------------
 static constexpr int SCAN_T = 1024, SCAN_IPT = 4, SCAN_TILE = SCAN_T * SCAN_IPT;
 
@@ -584,43 +586,39 @@ __device__ __forceinline__ void scan_apply_tile(const uint32_t *__restrict__ in,
     __syncthreads();  // *prefix is rewritten by the block's next tile
 }
 
-__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t *__restrict__ in, long long n,
-                                                         const unsigned long long *ndev, uint32_t *__restrict__ bsum,
-                                                         const Counters *ctr) {
+// Column counts -> column offsets of one call, in one pass.
+__global__ void __launch_bounds__(SCAN_T) k_scan_columns(Scratch s, long long n) {
     __shared__ uint32_t wsum[32];
-    if (ctr->flags & STOP_FLAGS) return;
-    if (ndev) n = (long long)*ndev;
-    if ((long long)blockIdx.x * SCAN_TILE >= n) return;
-    scan_reduce_tile(in, n, bsum, blockIdx.x, wsum);
-}
-
-__global__ void __launch_bounds__(SCAN_T) k_scan_apply(const uint32_t *__restrict__ in, long long n,
-                                                        const unsigned long long *ndev,
-                                                        const uint32_t *__restrict__ bsum, uint32_t *__restrict__ out,
-                                                        unsigned long long *total, long long cap, Counters *ctr) {
-    __shared__ uint32_t wsum[32];
-    __shared__ uint32_t prefix;
-    if (ctr->flags & STOP_FLAGS) return;
-    if (ndev) n = (long long)*ndev;
-    const long long nt = n > 0 ? (n + SCAN_TILE - 1) / SCAN_TILE : 1;
-    if (blockIdx.x >= nt) return;
-    scan_apply_tile(in, n, bsum, out, total, cap, &ctr->flags, blockIdx.x, nt, wsum, &prefix);
-}
-
-// ndev: the length on the device (n is then its bound)
-static void scan_u32(const uint32_t *in, long long n, const unsigned long long *ndev, uint32_t *out, uint32_t *bsum,
-                     unsigned long long *total, long long cap, Counters *ctr, cudaStream_t st) {
-    const int nb = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
-    k_scan_reduce<<<nb, SCAN_T, 0, st>>>(in, n, ndev, bsum, ctr);
-    k_scan_apply<<<nb, SCAN_T, 0, st>>>(in, n, ndev, bsum, out, total, cap, ctr);
-}
-
-void scan_u32_dev(const uint32_t *in, long long nmax, const unsigned long long *n, uint32_t *out, uint32_t *bsum,
-                  unsigned long long *total, Counters *ctr, cudaStream_t st) {
-    scan_u32(in, nmax, n, out, bsum, total, 0, ctr, st);
+    __shared__ uint32_t prefix, tile_s;
+    if (s.ctr->flags & STOP_FLAGS) return;
+    if (threadIdx.x == 0) tile_s = (uint32_t)atomicAdd(&s.ctr->tick[0], 1ull);
+    __syncthreads();
+    const long long tile = tile_s, base = tile * SCAN_TILE + (long long)threadIdx.x * SCAN_IPT;
+    uint32_t v[SCAN_IPT], sum = 0;
+#pragma unroll
+    for (int i = 0; i < SCAN_IPT; ++i) {
+        v[i] = base + i < n ? s.colcount[base + i] : 0u;
+        sum += v[i];
+    }
+    uint32_t tot;
+    const uint32_t loc = block_excl_scan(sum, wsum, tot);
+    if (threadIdx.x < 32) {
+        const uint32_t p = lb_prefix(s.lb + 1, s.lb[0], tile, tot, s.ctr);
+        if (threadIdx.x == 0) prefix = p;
+    }
+    __syncthreads();
+    uint32_t run = prefix + loc;
+#pragma unroll
+    for (int i = 0; i < SCAN_IPT; ++i) {
+        if (base + i < n) s.coloff[base + i] = run;
+        run += v[i];
+    }
+    if (base < n && base + SCAN_IPT >= n) s.coloff[n] = run;  // the thread of the last entry: the total
 }
 
 long long scan_partials(long long n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
+
+static long long column_tiles(int N) { return ((long long)N * N + SCAN_TILE - 1) / SCAN_TILE; }
 
 // ---------------------------------------------------------------------------
 // Marks grouped by column.
@@ -649,7 +647,8 @@ __global__ void k_scatter_marks(Scratch s) {
 //    together, each mark setting its bits in the two lines it touches.  (One
 //    lane per line walking its four columns' marks took 49 and 57 us at
 //    N = 512, 36 primitives: a warp waited for its longest line; now 24 and 32.)
-//    Pass 1 counts the set bits, pass 2 writes the keys in ascending c.
+//    The set bits are counted, the counts scanned over the lines
+//    (lookback.cuh) and the keys written in ascending c.
 // ---------------------------------------------------------------------------
 constexpr int LINES_T = 128;
 
@@ -664,83 +663,117 @@ __device__ __forceinline__ void set_corners(uint32_t *bits, int l, uint32_t k) {
 // warps of a launch over the lines of an N-grid
 __host__ __device__ inline long long line_tiles(int N) { return (long long)(N + 1) * ((N + 1 + 31) / 32); }
 
-// bits: the warp's own bit sets, at least (N + 1 + 31) / 32 * 32 words
-template <bool EMIT>
-__device__ __forceinline__ void lines_pass(const GridP &g, const Scratch &s, long long t0, long long stride,
-                                           uint32_t *bits) {
+// The bit sets of tile t's 32 lines; bits: the warp's own, at least
+// (N + 1 + 31) / 32 * 32 words.  Returns this lane's line, or -1.
+__device__ __forceinline__ long long gather_lines(const GridP &g, const Scratch &s, long long t, uint32_t *bits) {
     const int N = g.N, N1 = N + 1, NW = (N1 + 31) >> 5, TPR = (N1 + 31) / 32, lane = threadIdx.x & 31;
     const unsigned long long *__restrict__ mk = s.marks_csr;
     const uint32_t *__restrict__ off = s.coloff;
+    const int a = (int)(t / TPR), b0 = (int)(t - (long long)a * TPR) * 32;
+    for (int w = 0; w < NW; ++w) bits[w * 32 + lane] = 0u;
+    __syncwarp();
+    const int jlo = b0 > 0 ? b0 - 1 : 0, jhi = b0 + 31 < N ? b0 + 31 : N - 1;
+#pragma unroll
+    for (int di = -1; di <= 0; ++di) {
+        const int i = a + di;
+        if (i < 0 || i >= N || jlo > jhi) continue;
+        const uint32_t c0 = (uint32_t)i * N;
+        const uint32_t m0 = off[c0 + jlo], m1 = off[c0 + jhi + 1];
+        // a wall along z puts thousands of marks in one tile: four loads in flight
+        for (uint32_t mb = m0 + lane; mb < m1; mb += 128) {
+            unsigned long long r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) r[u] = mb + 32 * u < m1 ? __ldg(mk + mb + 32 * u) : MARK_EMPTY;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (mark_empty(r[u])) continue;
+                const int l = (int)(mark_col(r[u]) - c0) - b0;  // line j - b0; the mark also touches line j + 1
+                const uint32_t k = mark_k(r[u]);
+                if (l >= 0) set_corners(bits, l, k);
+                if (l < 31) set_corners(bits, l + 1, k);
+            }
+        }
+    }
+    __syncwarp();
+    return b0 + lane <= N ? (long long)a * N1 + b0 + lane : -1;
+}
+
+__device__ __forceinline__ uint32_t count_line(const uint32_t *bits, int NW) {
+    uint32_t cnt = 0;
+    for (int w = 0; w < NW; ++w) cnt += (uint32_t)__popc(bits[w * 32 + (threadIdx.x & 31)]);
+    return cnt;
+}
+
+// The keys of this lane's line from list entry o on.
+__device__ __forceinline__ void emit_line(const Scratch &s, const uint32_t *bits, int NW, long long line,
+                                          unsigned long long o) {
     const unsigned long long cap = (unsigned long long)s.cap_verts;
-    const long long tiles = line_tiles(N);
-    for (long long t = t0; t < tiles; t += stride) {
-        const int a = (int)(t / TPR), b0 = (int)(t - (long long)a * TPR) * 32;
-        for (int w = 0; w < NW; ++w) bits[w * 32 + lane] = 0u;
-        __syncwarp();
-        const int jlo = b0 > 0 ? b0 - 1 : 0, jhi = b0 + 31 < N ? b0 + 31 : N - 1;
-#pragma unroll
-        for (int di = -1; di <= 0; ++di) {
-            const int i = a + di;
-            if (i < 0 || i >= N || jlo > jhi) continue;
-            const uint32_t c0 = (uint32_t)i * N;
-            const uint32_t m0 = off[c0 + jlo], m1 = off[c0 + jhi + 1];
-            // a wall along z puts thousands of marks in one tile: four loads in flight
-            for (uint32_t mb = m0 + lane; mb < m1; mb += 128) {
-                unsigned long long r[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) r[u] = mb + 32 * u < m1 ? __ldg(mk + mb + 32 * u) : MARK_EMPTY;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (mark_empty(r[u])) continue;
-                    const int l = (int)(mark_col(r[u]) - c0) - b0;  // line j - b0; the mark also touches line j + 1
-                    const uint32_t k = mark_k(r[u]);
-                    if (l >= 0) set_corners(bits, l, k);
-                    if (l < 31) set_corners(bits, l + 1, k);
-                }
-            }
+    for (int w = 0; w < NW; ++w) {
+        uint32_t v = bits[w * 32 + (threadIdx.x & 31)];
+        while (v) {
+            const int bit = __ffs(v) - 1;
+            v &= v - 1;
+            if (o < cap) s.vkey[o] = (unsigned long long)line | ((unsigned long long)(32 * w + bit) << 32);
+            ++o;
         }
-        __syncwarp();
-        const int b = b0 + lane;
-        if (b <= N) {
-            const long long line = (long long)a * N1 + b;
-            if (!EMIT) {
-                uint32_t cnt = 0;
-                for (int w = 0; w < NW; ++w) cnt += (uint32_t)__popc(bits[w * 32 + lane]);
-                s.linecount[line] = cnt;
-            } else {
-                unsigned long long o = s.lineoff[line];
-                for (int w = 0; w < NW; ++w) {
-                    uint32_t v = bits[w * 32 + lane];
-                    while (v) {
-                        const int bit = __ffs(v) - 1;
-                        v &= v - 1;
-                        if (o < cap) s.vkey[o] = (unsigned long long)line | ((unsigned long long)(32 * w + bit) << 32);
-                        ++o;
-                    }
-                }
-            }
-        }
-        __syncwarp();  // the bit sets are cleared for the warp's next tile
     }
 }
 
-template <bool EMIT>
-__global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s) {
+// One call: gather, count, scan and emit in one pass, a block per four tiles.
+__global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s, long long lb0) {
     extern __shared__ uint32_t lbits[];
+    __shared__ uint32_t wsum[LINES_T / 32], base_s, group_s;
     if (s.ctr->flags & STOP_FLAGS) return;
-    lines_pass<EMIT>(g, s, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
-                     ((long long)gridDim.x * blockDim.x) >> 5, lbits + (threadIdx.x >> 5) * ((g.N + 1 + 31) / 32) * 32);
+    if (threadIdx.x == 0) group_s = (uint32_t)atomicAdd(&s.ctr->tick[1], 1ull);
+    __syncthreads();
+    const int NW = (g.N + 1 + 31) >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t *bits = lbits + wid * NW * 32;
+    const long long tiles = line_tiles(g.N), t = (long long)group_s * (LINES_T / 32) + wid;
+    long long line = -1;
+    uint32_t cnt = 0;
+    if (t < tiles) {
+        line = gather_lines(g, s, t, bits);
+        if (line >= 0) cnt = count_line(bits, NW);
+    }
+    uint32_t x = cnt;  // inclusive sum over the warp's lines
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    uint32_t tot = 0, wb = 0;
+    for (int q = 0; q < LINES_T / 32; ++q) {
+        if (q < wid) wb += wsum[q];
+        tot += wsum[q];
+    }
+    if (wid == 0) {
+        const uint32_t p = lb_prefix(s.lb + lb0, s.lb[0], group_s, tot, s.ctr);
+        if (lane == 0) base_s = p;
+    }
+    __syncthreads();
+    if (line < 0) return;
+    const uint32_t o = base_s + wb + x - cnt;
+    s.lineoff[line] = o;
+    emit_line(s, bits, NW, line, o);
+    const long long nlines = (long long)(g.N + 1) * (g.N + 1);
+    if (line == nlines - 1) {
+        s.lineoff[nlines] = o + cnt;
+        s.ctr->verts = o + cnt;
+        if ((long long)(o + cnt) > s.cap_verts) atomicOr(&s.ctr->flags, FLAG_VERT_OVERFLOW);
+    }
 }
 
+static long long line_groups(int N) { return (line_tiles(N) + LINES_T / 32 - 1) / (LINES_T / 32); }
+
+long long lb_words(int N) { return 1 + column_tiles(N) + line_groups(N); }
+
 void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st) {
-    const long long ncols = (long long)g.N * g.N, nlines = (long long)(g.N + 1) * (g.N + 1);
-    scan_u32(s.colcount, ncols, nullptr, s.coloff, s.blocksum, nullptr, 0, s.ctr, st);
+    const long long ct = column_tiles(g.N);
+    k_scan_columns<<<(int)ct, SCAN_T, 0, st>>>(s, (long long)g.N * g.N);
     k_scatter_marks<<<1024, 256, 0, st>>>(s);
-    const int lb = (int)((line_tiles(g.N) + LINES_T / 32 - 1) / (LINES_T / 32));
     const size_t lsm = (size_t)((g.N + 1 + 31) / 32) * LINES_T * sizeof(uint32_t);  // <= 33 KB at N = 2048
-    k_lines<false><<<lb, LINES_T, lsm, st>>>(g, s);
-    scan_u32(s.linecount, nlines, nullptr, s.lineoff, s.blocksum, &s.ctr->verts, s.cap_verts, s.ctr, st);
-    k_lines<true><<<lb, LINES_T, lsm, st>>>(g, s);
+    k_lines<<<(int)line_groups(g.N), LINES_T, lsm, st>>>(g, s, 1 + ct);
 }
 
 // ---------------------------------------------------------------------------
@@ -1611,15 +1644,27 @@ __global__ void k_scatter_marks_b(const Item *__restrict__ items, int n) {
     }
 }
 
+// Batches count and emit in two passes with a scan between: the blocks walk
+// the items with a grid stride, without tickets.
 template <bool EMIT>
 __global__ void __launch_bounds__(LINES_T) k_lines_b(const Item *__restrict__ items, int n, int max_words) {
     extern __shared__ uint32_t lbits[];
     uint32_t *bits = lbits + (threadIdx.x >> 5) * max_words * 32;  // the same place for every item: warps drift
+    const long long t0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const long long stride = ((long long)gridDim.x * blockDim.x) >> 5;
     for (int b = 0; b < n; ++b) {
         const Item &it = items[b];
         if (item_stopped(it)) continue;
-        lines_pass<EMIT>(it.g, it.s, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
-                         ((long long)gridDim.x * blockDim.x) >> 5, bits);
+        const int NW = (it.g.N + 1 + 31) >> 5;
+        const long long tiles = line_tiles(it.g.N);
+        for (long long t = t0; t < tiles; t += stride) {
+            const long long line = gather_lines(it.g, it.s, t, bits);
+            if (line >= 0) {
+                if (EMIT) emit_line(it.s, bits, NW, line, it.s.lineoff[line]);
+                else it.s.linecount[line] = count_line(bits, NW);
+            }
+            __syncwarp();  // the bit sets are cleared for the warp's next tile
+        }
     }
 }
 
