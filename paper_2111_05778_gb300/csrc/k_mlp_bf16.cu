@@ -12,7 +12,7 @@
 // every hidden activation.  The output layer (W -> 1) runs on CUDA cores in
 // FP32.
 //
-// One persistent CTA per SM, 64 threads + 128 or 256 per tile:
+// Persistent CTAs (one per SM; width 64 four), 64 threads + 128 or 256 per tile:
 //   warp 0       TMA producer: 1-D bulk copies (cp.async.bulk) of BF16 weight
 //                K-blocks, stored pre-swizzled in global memory, into a
 //                shared-memory ring (mbarrier complete_tx).
@@ -61,12 +61,17 @@ constexpr int maxmid_of() {
 }
 
 // Threads per row of a tile.  At width 256 one thread would convert 256
-// columns per layer, longer than the other tile's products take; at width 64
-// a second thread only adds barrier arrivals (2^20 points 191 us with one, 194
-// with two).
-template <int W>
+// columns per layer, longer than the other tile's products take; where several
+// CTAs share an SM one thread leaves each the registers it needs.
+template <int W, int TILES>
 constexpr int halves_of() {
-    return W == 64 ? 1 : 2;
+    return W == 256 || (W == 128 && TILES == 2) ? 2 : 1;
+}
+
+// Resident CTAs per SM the registers are budgeted for.
+template <int W, int TILES>
+constexpr int ctas_of() {
+    return TILES == 2 || W == 256 ? 1 : (W == 128 ? 3 : 4);
 }
 
 // Weight ring: stages of KS inputs x W outputs.  Width 256 has room for 64 KB
@@ -83,17 +88,17 @@ constexpr int nslot_of() {
     return W == 256 ? 4 : W / 32;
 }
 
-template <int W>
+template <int W, int TILES>
 struct SmemB {
     static constexpr int NSLOT = nslot_of<W>();
-    uint8_t a[2][W / 64][TM * 128];  // A operands: one per tile, K-blocks of 128 rows x 128 B (1024-aligned)
+    uint8_t a[TILES][W / 64][TM * 128];  // A operands: one per tile, K-blocks of 128 rows x 128 B (1024-aligned)
     uint8_t w[NSLOT][W * 2 * ks_of<W>()];  // weight ring: one K-block of W rows x KS inputs per stage
-    uint8_t b0[2][W * 32];           // per tile: layer-0 operand B0 of its current item, W rows x 16 inputs
+    uint8_t b0[TILES][W * 32];           // per tile: layer-0 operand B0 of its current item, W rows x 16 inputs
                                      // (32-byte swizzle: row n, 16-byte chunk c at (n/8)*256 + (n%8)*32 +
                                      // ((c ^ (n/4)%2) * 16))
-    float bmid[2][maxmid_of<W>() * W];  // per tile: hidden-layer biases
-    float red[2][TM];                // per tile: the second halves' output dot products
-    float wout[2][W];                // per tile: output-layer weights
+    float bmid[TILES][maxmid_of<W>() * W];  // per tile: hidden-layer biases
+    float red[TILES][TM];                // per tile: the second halves' output dot products
+    float wout[TILES][W];                // per tile: output-layer weights
     unsigned long long full[NSLOT], empty[NSLOT], acc_full[2], a_full[2], item_ready[2], drain;
     const uint16_t *cur_wbf[2];      // per tile: weights of its current item
     int done[2];                     // per tile: no more work
@@ -117,8 +122,8 @@ __device__ __forceinline__ void split2(float x, uint32_t &h, uint32_t &l) {
 }
 
 // Row o of tile t's layer-0 operand B0 (two 16-byte chunks, inputs 0..15).
-template <int W>
-__device__ __forceinline__ void put_b0(SmemB<W> &sm, int t, int o, float wx, float wy, float wz, float b) {
+template <int W, int TILES>
+__device__ __forceinline__ void put_b0(SmemB<W, TILES> &sm, int t, int o, float wx, float wy, float wz, float b) {
     uint32_t xh, xl, yh, yl, zh, zl, bh, bl;
     split2(wx, xh, xl);
     split2(wy, yh, yl);
@@ -132,10 +137,10 @@ __device__ __forceinline__ void put_b0(SmemB<W> &sm, int t, int o, float wx, flo
 
 // Item parameters of tile t (its epilogue threads, or all threads at set-up
 // with e and the stride given): B0, hidden biases, output weights.
-template <int W>
-__device__ __forceinline__ void load_item(SmemB<W> &sm, int t, const MlpDev &mm, int e, int stride) {
+template <int W, int TILES>
+__device__ __forceinline__ void load_item(SmemB<W, TILES> &sm, int t, const MlpDev &mm, int e, int stride) {
     for (int o = e; o < W; o += stride) {
-        put_b0<W>(sm, t, o, mm.w0[3 * o], mm.w0[3 * o + 1], mm.w0[3 * o + 2], mm.b0[o]);
+        put_b0<W, TILES>(sm, t, o, mm.w0[3 * o], mm.w0[3 * o + 1], mm.w0[3 * o + 2], mm.b0[o]);
         sm.wout[t][o] = mm.wout[o];
     }
     for (int i = e; i < mm.n_mid * W; i += stride) sm.bmid[t][i] = mm.bm[i];
@@ -152,25 +157,25 @@ __device__ __forceinline__ void load_item(SmemB<W> &sm, int t, const MlpDev &mm,
 // biases and output weights; the producer streams the weights of whichever
 // item the phase's tile is on.
 template <int W, int MODE, int TILES>
-__global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W>() * TILES, 1)
+__global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, ctas_of<W, TILES>())
     k_mlp_bf16(const Item *__restrict__ items, int n_items, const float *__restrict__ pts, long long npts,
                float *__restrict__ outv, unsigned long long wait_ns) {
     extern __shared__ uint8_t smem_raw[];
-    constexpr int HALVES = halves_of<W>(), ET = TM * HALVES;  // epilogue threads per row, per tile
+    constexpr int HALVES = halves_of<W, TILES>(), ET = TM * HALVES;  // epilogue threads per row, per tile
     constexpr int KS = ks_of<W>(), KB = W / KS;  // K-blocks per hidden layer
     constexpr int NSLOT = nslot_of<W>();
     constexpr int RS = KB < NSLOT ? KB : NSLOT;  // K-blocks a phase can take over from the one before
     constexpr uint32_t STAGE_BYTES = W * 2 * KS;
     constexpr uint32_t TMEM_COLS = TILES * W < 32 ? 32 : TILES * W;
     constexpr uint32_t IDESC = idesc_bf16(TM, W);
-    SmemB<W> &sm = *reinterpret_cast<SmemB<W> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
+    SmemB<W, TILES> &sm = *reinterpret_cast<SmemB<W, TILES> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *ctl = &sm.ctl;
     Counters *ctr0 = items[0].s.ctr;  // error flags of a timeout go to the first item
     const int n_mid = items[0].m.n_mid;
 
     // ---- set-up ----------------------------------------------------------
-    for (int t = 0; t < TILES; ++t) load_item<W>(sm, t, items[0].m, tid, blockDim.x);
+    for (int t = 0; t < TILES; ++t) load_item<W, TILES>(sm, t, items[0].m, tid, blockDim.x);
     if (tid == 0) {
         for (int i = 0; i < NSLOT; ++i) {
             mbar_init(&sm.full[i], 1);
@@ -269,9 +274,9 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W>() * TILES, 1)
             uint32_t pf = 0u;  // ring: phase of the next stage to land
             int sb = 0;        // and, where the ring holds two layers, its index
             constexpr unsigned long long A_KB = (TM * 128) >> 4, W_ST = STAGE_BYTES >> 4;
-            const unsigned long long ad0 = sdesc(su32(&sm.a[0][0][0])), ad1 = sdesc(su32(&sm.a[1][0][0]));
+            const unsigned long long ad0 = sdesc(su32(&sm.a[0][0][0])), ad1 = sdesc(su32(&sm.a[TILES - 1][0][0]));
             const unsigned long long wd0 = KS == 32 ? sdesc64(su32(sm.w[0])) : sdesc(su32(sm.w[0]));
-            const unsigned long long bd0 = sdesc32(su32(sm.b0[0])), bd1 = sdesc32(su32(sm.b0[1]));
+            const unsigned long long bd0 = sdesc32(su32(sm.b0[0])), bd1 = sdesc32(su32(sm.b0[TILES - 1]));
             const uint16_t *w0 = nullptr, *w1 = nullptr;  // per tile: weights of its current item
             bool go = true, keep = false;
             while (go && !(fin0 && fin1)) {
@@ -495,7 +500,7 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W>() * TILES, 1)
                 g = it->g;
                 col = NONE;
                 done = false;
-                load_item<W>(sm, t, it->m, row + TM * half, ET);
+                load_item<W, TILES>(sm, t, it->m, row + TM * half, ET);
                 bar_sync(bar, ET);  // the new item's parameters are in place
                 continue;
             }
@@ -648,14 +653,14 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W>() * TILES, 1)
 
 template <int W, int MODE, int TILES>
 void launch_bf16(const Item *items, int n_items, const float *p, long long n, float *out, int nsm, cudaStream_t st) {
-    const size_t smem = sizeof(SmemB<W>) + 1024;
+    const size_t smem = sizeof(SmemB<W, TILES>) + 1024;
     cudaFuncSetAttribute(k_mlp_bf16<W, MODE, TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int grid = nsm;
+    int grid = nsm * ctas_of<W, TILES>();
     if (MODE == MODE_POINTS) {
         const long long tiles = (n + 128 * TILES - 1) / (128 * TILES);
         if (grid > tiles) grid = (int)(tiles < 1 ? 1 : tiles);
     }
-    k_mlp_bf16<W, MODE, TILES><<<grid, EPI_T0 + TM * halves_of<W>() * TILES, smem, st>>>(items, n_items, p, n, out, wait_limit_ns());
+    k_mlp_bf16<W, MODE, TILES><<<grid, EPI_T0 + TM * halves_of<W, TILES>() * TILES, smem, st>>>(items, n_items, p, n, out, wait_limit_ns());
 }
 
 }  // namespace
@@ -670,17 +675,25 @@ void launch_bf16(const Item *items, int n_items, const float *p, long long n, fl
 bool bf16_supported(int width) { return width == 64 || width == 128 || width == 256; }
 int bf16_max_mid(int width) { return width == 256 ? maxmid_of<256>() : maxmid_of<128>(); }
 
-#define GH_BF16_T(T, ...)                                \
-    if ((T) == 1) { constexpr int TT = 1; __VA_ARGS__; } \
-    else { constexpr int TT = 2; __VA_ARGS__; }
+// Tiles per CTA: two, or one if the caller asks for it; at width 64 always one,
+// with four CTAs on an SM (2^20 points 187 -> 121 us, hop at N = 1000 3.35 ->
+// 2.55 ms, at N = 300, where the longest rays count more than the throughput,
+// 0.52 -> 0.54).  At width 128 three CTAs of one tile are slower than one of
+// two from N = 300 on (hop at N = 1000 5.11 against 4.83 ms).
+template <int W, int MODE>
+void launch_tiles(int tiles, const Item *items, int n_items, const float *p, long long n, float *out, int nsm,
+                  cudaStream_t st) {
+    constexpr int T = W == 64 ? 1 : 2;
+    if (tiles == 1) launch_bf16<W, MODE, 1>(items, n_items, p, n, out, nsm, st);
+    else launch_bf16<W, MODE, T>(items, n_items, p, n, out, nsm, st);
+}
 
 void launch_hop_mlp_bf16(const Item *items, int n_items, int width, int nsm, int tiles, cudaStream_t st) {
-    GH_BF16_W(width, GH_BF16_T(tiles, (launch_bf16<WW, MODE_HOP, TT>(items, n_items, nullptr, 0, nullptr, nsm, st))))
+    GH_BF16_W(width, (launch_tiles<WW, MODE_HOP>(tiles, items, n_items, nullptr, 0, nullptr, nsm, st)))
 }
 
 void launch_eval_vertices_mlp_bf16(const Item *items, int n_items, int width, int nsm, int tiles, cudaStream_t st) {
-    GH_BF16_W(width,
-              GH_BF16_T(tiles, (launch_bf16<WW, MODE_VERTS, TT>(items, n_items, nullptr, 0, nullptr, nsm, st))))
+    GH_BF16_W(width, (launch_tiles<WW, MODE_VERTS>(tiles, items, n_items, nullptr, 0, nullptr, nsm, st)))
 }
 
 void launch_eval_points_mlp_bf16(const MlpDev &m, const float *p, long long n, float *out, int nsm,
@@ -696,7 +709,7 @@ void launch_eval_points_mlp_bf16(const MlpDev &m, const float *p, long long n, f
     h.kind = 1;
     cudaMemsetAsync(ctr, 0, sizeof(Counters), st);
     cudaMemcpyAsync(ditem, &h, sizeof(Item), cudaMemcpyHostToDevice, st);
-    GH_BF16_W(m.width, (launch_bf16<WW, MODE_POINTS, 2>(ditem, 1, p, n, out, nsm, st)))
+    GH_BF16_W(m.width, (launch_tiles<WW, MODE_POINTS>(2, ditem, 1, p, n, out, nsm, st)))
 }
 
 }  // namespace gh
