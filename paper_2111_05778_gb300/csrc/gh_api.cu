@@ -733,7 +733,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
     }
     if (s->kind == GH_SDB_CSG) {
         if (cull_words(g.N, s->nprim) > 0) {
-            launch_cull(s->d_item, 1, g.N, s->nprim, st);
+            launch_cull(s->d_item, 1, s->nprim, st);
             ++launches;
         }
         launch_hop_csg(s->d_item, 1, s->nprim, nsm, o.ray_block, st);
@@ -1070,12 +1070,8 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         const int n = gr.second - gr.first;
         if (first->kind == GH_SDB_CSG) {
             int mx = 1;
-            int mN = 2;
-            for (int q = gr.first; q < gr.second; ++q) {
-                mx = sd[P.order[q]]->nprim > mx ? sd[P.order[q]]->nprim : mx;
-                mN = P.g[P.order[q]].N > mN ? P.g[P.order[q]].N : mN;
-            }
-            launch_cull(di, n, mN, mx, st);
+            for (int q = gr.first; q < gr.second; ++q) mx = sd[P.order[q]]->nprim > mx ? sd[P.order[q]]->nprim : mx;
+            launch_cull(di, n, mx, st);
             ++launches;
             launch_hop_csg(di, n, mx, nsm, o.ray_block, st);
         } else if (o.precision == GH_FP32) {

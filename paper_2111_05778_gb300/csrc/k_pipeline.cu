@@ -191,7 +191,7 @@ __device__ __forceinline__ float csg_eval(const float4 *P, int n, float x, float
 }
 
 // ---------------------------------------------------------------------------
-// Culling.  The volume is divided into blocks of CULL_B^3 cells; for each, a
+// Culling.  The volume is divided into up to 32^3 blocks of cells; for each, a
 // bit mask says which primitives can matter at any of its points (cell centres
 // and lattice points), and the evaluator folds only those.  With R the radius
 // of the block, every distance and every partial fold is 1-Lipschitz, so its
@@ -204,24 +204,27 @@ __device__ __forceinline__ float csg_eval(const float4 *P, int n, float x, float
 // rotation may miss orthonormality) is added, so the masked fold gives the
 // full fold's value bit for bit.  Scenes with a primitive whose bounding
 // radius is infinite (sizes for which the distance may not be 1-Lipschitz)
-// get full masks.  36 primitives at N = 512: 4 to 7 of 36 remain in a warp's
-// union of masks.  Below CULL_MIN primitives the masks cost more than they
-// save.
+// get full masks.  32 blocks per axis at every N: the masks then cost 14 us for
+// 36 primitives, and 4 to 7 of them remain in a warp's union of masks; blocks of
+// 16 cells left most of them at N = 64 (hop 189 us without masks, 246 with
+// those, 123 with these).  Below CULL_MIN primitives the masks cost more than
+// they save.
 // ---------------------------------------------------------------------------
-static constexpr int CULL_B = 16, CULL_MIN = 6;
+static constexpr int CULL_NB = 32, CULL_MIN = 6;
 
-__host__ __device__ inline int cull_blocks(int N) { return (N + CULL_B - 1) / CULL_B; }
+__host__ __device__ inline int cull_edge(int N) { return (N + CULL_NB - 1) / CULL_NB; }  // cells per block and axis
+__host__ __device__ inline int cull_blocks(int N) { return (N + cull_edge(N) - 1) / cull_edge(N); }
 
 long long cull_words(int N, int nprim) {
     const long long nb = cull_blocks(N);
     return nprim < CULL_MIN ? 0 : nb * nb * nb * ((nprim + 31) / 32);
 }
 
-// mask of the block holding cell (or lattice) index (i, j, k)
-__device__ __forceinline__ const uint32_t *cull_mask(const uint32_t *cull, int N, int nw, int i, int j, int k) {
-    const int nb = cull_blocks(N);
-    const int bi = min(i / CULL_B, nb - 1), bj = min(j / CULL_B, nb - 1), bk = min(k / CULL_B, nb - 1);
-    return cull + (size_t)((bi * nb + bj) * nb + bk) * nw;
+// The block index of a cell or lattice index i: i / cull_edge(N), the last
+// lattice point in the last block (the quotient of i + 1/2 is at least 1/128
+// from an integer, so the product's rounding does not matter).
+__device__ __forceinline__ int cull_index(int i, float inv_edge, int nb) {
+    return min((int)(((float)i + 0.5f) * inv_edge), nb - 1);
 }
 
 // One thread per block (of cells); dist: this thread's distances, nprim floats
@@ -229,10 +232,11 @@ __device__ __forceinline__ const uint32_t *cull_mask(const uint32_t *cull, int N
 __device__ void cull_block(const float4 *P, int nprim, const GridP &g, int b, float *dist, uint32_t *out) {
     const int nb = cull_blocks(g.N), nw = (nprim + 31) / 32, T = blockDim.x;
     const int bk = b % nb, bj = (b / nb) % nb, bi = b / (nb * nb);
-    const float half = 0.5f * CULL_B;
-    const float x = fmaf(bi * CULL_B + half, g.h, g.lo[0]), y = fmaf(bj * CULL_B + half, g.h, g.lo[1]),
-                z = fmaf(bk * CULL_B + half, g.h, g.lo[2]);
-    const float R = 0.8660255f * CULL_B * g.h * 1.0003f;
+    const int edge = cull_edge(g.N);
+    const float half = 0.5f * edge;
+    const float x = fmaf(bi * edge + half, g.h, g.lo[0]), y = fmaf(bj * edge + half, g.h, g.lo[1]),
+                z = fmaf(bk * edge + half, g.h, g.lo[2]);
+    const float R = 0.8660255f * edge * g.h * 1.0003f;
     const float pos = fabsf(x) + fabsf(y) + fabsf(z) + R + 1.f;
     bool full = false;
     for (int i = 0; i < nprim; ++i) {
@@ -365,7 +369,8 @@ void launch_init(Scratch &s, cudaStream_t st) { k_init<<<1, 32, 0, st>>>(s.ctr, 
 //    short: culled primitives are not folded, a column claim is issued one
 //    step before its answer is needed, and marks collect in shared memory and
 //    leave 32 at a time, so that no step waits for an atomic's round trip.
-//    36 primitives at N = 512: 648 -> 235 us, and 14 us for the masks.
+//    36 primitives at N = 512: 648 -> 235 us, and 14 us for the masks; at N = 64
+//    189 -> 123 us with them.
 // ---------------------------------------------------------------------------
 template <bool CULL>
 __device__ __forceinline__ void hop_csg(const Item &it, const float4 *sprim, unsigned long long *buf) {
@@ -378,7 +383,10 @@ __device__ __forceinline__ void hop_csg(const Item &it, const float4 *sprim, uns
     const int N = g.N, nw = (nprim + 31) / 32;
     const uint32_t ncols = (uint32_t)N * (uint32_t)N;
     uint32_t col = NONE, rank = 0, evals = 0;
-    int k = 0, ci = 0, cj = 0;
+    const int nb = CULL ? cull_blocks(N) : 1;
+    const float inv_edge = CULL ? 1.f / (float)cull_edge(N) : 0.f;
+    const uint32_t *colmask = nullptr;  // the masks of the column's blocks
+    int k = 0;
     bool done = false;
     float x = 0.f, y = 0.f;
     unsigned claim = 0;                 // lanes whose claim is on its way
@@ -403,10 +411,10 @@ __device__ __forceinline__ void hop_csg(const Item &it, const float4 *sprim, uns
                     col = column_of_claim((uint32_t)c, N);
                     k = 0;
                     rank = 0;
-                    ci = (int)(col / (uint32_t)N);
-                    cj = (int)(col - (uint32_t)ci * N);
-                    x = fmaf((float)ci + 0.5f, g.h, g.lo[0]);
-                    y = fmaf((float)cj + 0.5f, g.h, g.lo[1]);
+                    const int i = (int)(col / (uint32_t)N), j = (int)(col - (uint32_t)i * N);
+                    x = fmaf((float)i + 0.5f, g.h, g.lo[0]);
+                    y = fmaf((float)j + 0.5f, g.h, g.lo[1]);
+                    if (CULL) colmask = s.cull + (size_t)((cull_index(i, inv_edge, nb) * nb + cull_index(j, inv_edge, nb)) * nb) * nw;
                 } else {
                     done = true;
                 }
@@ -427,7 +435,7 @@ __device__ __forceinline__ void hop_csg(const Item &it, const float4 *sprim, uns
         int step = 1;
         const float z = fmaf((float)k + 0.5f, g.h, g.lo[2]);
         float f = 0.f;
-        if (CULL) f = csg_eval_masked(sprim, nprim, live ? cull_mask(s.cull, N, nw, ci, cj, k) : nullptr, x, y, z);
+        if (CULL) f = csg_eval_masked(sprim, nprim, live ? colmask + cull_index(k, inv_edge, nb) * nw : nullptr, x, y, z);
         else if (live) f = csg_eval(sprim, nprim, x, y, z);
         if (live) {
             ++evals;
@@ -490,10 +498,10 @@ __global__ void __launch_bounds__(512) k_hop_csg(const Item *__restrict__ items,
 }
 
 // The culling masks of n items, before their hopping.
-void launch_cull(const Item *items, int n, int max_N, int max_prims, cudaStream_t st) {
+void launch_cull(const Item *items, int n, int max_prims, cudaStream_t st) {
     if (max_prims < CULL_MIN) return;
-    const long long nb = cull_blocks(max_N);
-    const dim3 grid((unsigned)((nb * nb * nb + CULL_T - 1) / CULL_T), (unsigned)n);
+    constexpr unsigned blocks = CULL_NB * CULL_NB * CULL_NB;  // at most; an item's surplus ones return at once
+    const dim3 grid((blocks + CULL_T - 1) / CULL_T, (unsigned)n);
     const size_t smem = (size_t)max_prims * (sizeof(Prim) + CULL_T * sizeof(float));
     cudaFuncSetAttribute(k_cull, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_cull<<<grid, CULL_T, smem, st>>>(items);
@@ -792,7 +800,8 @@ __device__ __forceinline__ void eval_vertices_csg(const float4 *sprim, int nprim
                                                   unsigned long long t0, unsigned long long stride) {
     const unsigned long long V = s.ctr->verts;
     if (s.cull && nprim >= CULL_MIN) {  // whole warps (t0 - lane starts the warp's vertices)
-        const int lane = threadIdx.x & 31, nw = (nprim + 31) / 32;
+        const int lane = threadIdx.x & 31, nw = (nprim + 31) / 32, nb = cull_blocks(g.N);
+        const float inv_edge = 1.f / (float)cull_edge(g.N);
         const uint32_t N1 = (uint32_t)g.N + 1u;
         for (unsigned long long vb = t0 - (unsigned long long)lane; vb < V; vb += stride) {
             const unsigned long long v = vb + (unsigned long long)lane;
@@ -800,8 +809,9 @@ __device__ __forceinline__ void eval_vertices_csg(const float4 *sprim, int nprim
             const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), a = line / N1, b = line - a * N1;
             float x, y, z;
             vertex_pos(g, key, x, y, z);
-            const float f = csg_eval_masked(
-                sprim, nprim, v < V ? cull_mask(s.cull, g.N, nw, (int)a, (int)b, (int)(key >> 32)) : nullptr, x, y, z);
+            const int blk = (cull_index((int)a, inv_edge, nb) * nb + cull_index((int)b, inv_edge, nb)) * nb +
+                            cull_index((int)(key >> 32), inv_edge, nb);
+            const float f = csg_eval_masked(sprim, nprim, v < V ? s.cull + (size_t)blk * nw : nullptr, x, y, z);
             if (v < V) {
                 if (!isfinite(f)) atomicOr(&s.ctr->flags, FLAG_NONFINITE);
                 s.vval[v] = f;
