@@ -1350,9 +1350,7 @@ extern "C" int gh_backward(const gh_sdb *cs, const float *verts, const float *dL
     b.D = b.Z + (size_t)(L + 1) * b.VC * W;
     b.s = b.D + (size_t)(L + 1) * b.VC * W;
     b.part = b.s + b.VC;
-    b.ones = b.part + adjoint_part_floats(W, L, S, nsm);
-    b.mbits = reinterpret_cast<uint32_t *>(b.ones + b.VC);
-    adjoint_fill_ones(b.ones, b.VC, st);
+    b.mbits = reinterpret_cast<uint32_t *>(b.part + adjoint_part_floats(W, L, S, nsm));
     for (long long v0 = 0; v0 < V; v0 += b.VC) {
         const int n = (int)((V - v0) < b.VC ? (V - v0) : b.VC);
         adjoint_chunk(s->mlp, verts + 3 * v0, dL_dv + 3 * v0, n, dL_dtheta, v0 > 0, b, st);

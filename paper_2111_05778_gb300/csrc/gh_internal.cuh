@@ -288,7 +288,7 @@ void launch_index_mesh_b(const Item *items, int n, int nsm, cudaStream_t st);
 
 // implicit-surface adjoint (k_adjoint.cu)
 struct AdjBuffers {
-    float *Z, *D, *s, *part, *ones;
+    float *Z, *D, *s, *part;
     uint32_t *mbits;  // ReLU masks of z_0..z_{L-1}: (VC / 128) tiles x 256 threads x W / 64 words per layer
     int VC, splits, nsm;
 };
@@ -309,7 +309,6 @@ size_t adjoint_part_floats(int W, int n_mid, int splits, int nsm);
 size_t adjoint_buffer_floats(int W, int n_mid, int VC, int splits, int nsm);
 void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, float *grad, bool accumulate,
                    const AdjBuffers &b, cudaStream_t st);
-void adjoint_fill_ones(float *p, long long n, cudaStream_t st);
 void csg_adjoint(const Prim *prims, int nprim, const float *V, const float *dL, int nv, int *act, float *contrib,
                  float *out, cudaStream_t st);
 

@@ -209,60 +209,88 @@ __global__ void k_adj_reduce(const float *__restrict__ part, int splits, long lo
     }
 }
 
-// part[z][j * NP + a] = sum over rows v of split z of s[v] * X'[v][j] *
-// P[v][a] (NP = 3) or s[v] * X'[v][j] (NP = 1), with X' = relu(X) if RELU,
-// X' = 1 if X is null.  Column sums of the parameter gradients that have one
-// (or three) outputs per unit: b_l, W_0, w_out.  A block of 32 columns x 8
-// row groups: group g adds the split's rows v = g, g + 8, ... in order, and
-// the 8 group sums are added in group order -- a fixed summation order.
-template <int NP, bool RELU>
+// part[z][j] = sum over rows v of split z of s[v] X[v][j]: the bias gradients
+// of the FFMA path's hidden layers.  A block of 32 columns x 8 row groups:
+// group g adds the split's rows v = g, g + 8, ... in order, and the 8 group sums
+// are added in group order -- a fixed summation order.
+__device__ __forceinline__ float group_sum(const float (&red)[8][32][4], int cx, int a) {
+    float t = red[0][cx][a];
+    for (int q = 1; q < 8; ++q) t += red[q][cx][a];
+    return t;
+}
+
 __global__ void __launch_bounds__(256) k_colsum(const float *__restrict__ X, int V, int W, const float *__restrict__ s,
-                                                const float *__restrict__ P, int rows_per_split,
-                                                float *__restrict__ part) {
-    __shared__ float red[8][32][NP];
+                                                int rows_per_split, float *__restrict__ part) {
+    __shared__ float red[8][32][4];
     const int z = blockIdx.y, cx = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int j = blockIdx.x * 32 + cx;
     const int v0 = z * rows_per_split, v1 = min(V, v0 + rows_per_split);
-    float acc[NP];
-#pragma unroll
-    for (int a = 0; a < NP; ++a) acc[a] = 0.f;
-    if (j < W) {
+    float acc = 0.f;
 #pragma unroll 4
-        for (int v = v0 + g; v < v1; v += 8) {
-            float x = X ? X[(size_t)v * W + j] : 1.f;
-            if (RELU) x = fmaxf(x, 0.f);
-            const float sx = s[v] * x;
-            if (NP == 1) {
-                acc[0] += sx;
-            } else {
-#pragma unroll
-                for (int a = 0; a < NP; ++a) acc[a] = fmaf(sx, P[3 * v + a], acc[a]);
-            }
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < NP; ++a) red[g][cx][a] = acc[a];
+    for (int v = v0 + g; v < v1; v += 8) acc = fmaf(s[v], X[(size_t)v * W + j], acc);
+    red[g][cx][0] = acc;
     __syncthreads();
-    if (g == 0 && j < W) {
+    if (g == 0) part[(size_t)z * W + j] = group_sum(red, cx, 0);
+}
+
+// The sums of the first and the last layer in one launch, in the same order:
+// part[z] = { W_0: sum s D[v][j] P[v][a] at 3 j + a | b_0: sum s D[v][j] |
+// w_out: sum s relu(Z[v][j]) | b_out: sum s }, 5 W + 1 floats.  D and Z are read
+// once each.  What bounds it is the latency of the loads (a thread adds 180
+// rows of 111 k vertices), so the three kinds run side by side; as four launches
+// of column sums and four reductions, each alone on the chip, a call of 111 k
+// vertices at width 256 took 1.89 ms instead of 1.79.
+__global__ void __launch_bounds__(256) k_adj_ends(const float *__restrict__ D, const float *__restrict__ Z, int V,
+                                                  int W, const float *__restrict__ s, const float *__restrict__ P,
+                                                  int rows_per_split, float *__restrict__ part) {
+    __shared__ float red[8][32][4];
+    const int z = blockIdx.y, cx = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int nb = W / 32, kind = blockIdx.x / nb;  // 0: W_0 and b_0, 1: w_out, 2: b_out
+    const int j = (blockIdx.x - kind * nb) * 32 + cx;
+    const int v0 = z * rows_per_split, v1 = min(V, v0 + rows_per_split);
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    if (kind == 0) {
+#pragma unroll 8
+        for (int v = v0 + g; v < v1; v += 8) {
+            const float sv = s[v], x = D[(size_t)v * W + j], sx = sv * x;
 #pragma unroll
-        for (int a = 0; a < NP; ++a) {
-            float t = red[0][cx][a];
-            for (int q = 1; q < 8; ++q) t += red[q][cx][a];
-            part[(size_t)z * W * NP + (size_t)j * NP + a] = t;
+            for (int a = 0; a < 3; ++a) acc[a] = fmaf(sx, P[3 * v + a], acc[a]);
+            acc[3] = fmaf(sv, x, acc[3]);
         }
+    } else if (kind == 1) {
+#pragma unroll 8
+        for (int v = v0 + g; v < v1; v += 8) acc[0] = fmaf(s[v], fmaxf(Z[(size_t)v * W + j], 0.f), acc[0]);
+    } else {
+#pragma unroll 8
+        for (int v = v0 + g; v < v1; v += 8) acc[0] += s[v];
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) red[g][cx][a] = acc[a];
+    __syncthreads();
+    if (g != 0) return;
+    float *q = part + (size_t)z * (5 * W + 1);
+    if (kind == 0) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) q[3 * j + a] = group_sum(red, cx, a);
+        q[3 * W + j] = group_sum(red, cx, 3);
+    } else if (kind == 1) {
+        q[4 * W + j] = group_sum(red, cx, 0);
+    } else if (cx == 0) {
+        q[5 * W] = group_sum(red, 0, 0);
     }
 }
 
-template <int NP, bool RELU>
-void colsum(const float *X, int V, int W, const float *s, const float *P, int splits, float *part, cudaStream_t st) {
-    const int rows = (V + splits - 1) / splits;
-    dim3 grid((W + 31) / 32, splits);
-    k_colsum<NP, RELU><<<grid, 256, 0, st>>>(X, V, W, s, P, rows, part);
-}
-
-__global__ void k_fill(float *p, long long n, float v) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        p[i] = v;
+// grad's first 4 W entries (W_0, b_0) and the W + 1 from last on (w_out, b_out)
+// (+)= c * sum_z part[z], z in increasing order
+__global__ void __launch_bounds__(128) k_adj_ends_reduce(const float *__restrict__ part, int splits, int W, float c,
+                                                         float *__restrict__ grad, long long last, int accumulate) {
+    const int e = blockIdx.x * 128 + threadIdx.x, n = 5 * W + 1;
+    if (e >= n) return;
+    float acc = 0.f;
+#pragma unroll 8
+    for (int z = 0; z < splits; ++z) acc += part[(size_t)z * n + e];
+    float *out = grad + (e < 4 * W ? e : last + e - 4 * W);
+    *out = accumulate ? __fadd_rn(*out, __fmul_rn(c, acc)) : __fmul_rn(c, acc);
 }
 
 }  // namespace
@@ -276,7 +304,7 @@ size_t adjoint_part_floats(int W, int n_mid, int splits, int nsm) {
 size_t adjoint_buffer_floats(int W, int n_mid, int VC, int splits, int nsm) {
     const size_t L1 = (size_t)n_mid + 1;
     const size_t mask_words = (size_t)n_mid * ((VC + 127) / 128) * 256 * (W / 64);
-    return L1 * VC * W * 2 + VC + adjoint_part_floats(W, n_mid, splits, nsm) + VC + mask_words;
+    return L1 * VC * W * 2 + VC + adjoint_part_floats(W, n_mid, splits, nsm) + mask_words;
 }
 
 // One chunk of vertices; accumulates into grad (packed like the parameters).
@@ -303,31 +331,21 @@ void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, floa
         k_adj_s<<<(V + 7) / 8, 256, 0, st>>>(P, dL, V, Dl[0], m.w0, W, m.alpha, 1.f / m.beta * m.inv_lam, m.radial, b.s);
     }
     // parameter gradients: sums over the vertices of the chunk
-    const size_t oW0 = 0, ob0 = (size_t)3 * W, omid = ob0 + W;
-    const size_t ow = omid + (size_t)L * ((size_t)W * W + W);
-    const int gb = 512;
-    // W_0 and b_0
-    colsum<3, false>(Dl[0], V, W, b.s, P, S, b.part, st);
-    k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W * 3, c, grad + oW0, accumulate);
-    colsum<1, false>(Dl[0], V, W, b.s, nullptr, S, b.part, st);
-    k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W, c, grad + ob0, accumulate);
+    const size_t omid = (size_t)4 * W, ow = omid + (size_t)L * ((size_t)W * W + W);
+    const int gb = 512, rows = (V + S - 1) / S;
+    // W_0, b_0, w_out (from relu(z_L)), b_out (from the scales alone)
+    k_adj_ends<<<dim3(2 * (W / 32) + 1, S), 256, 0, st>>>(Dl[0], Zl[L], V, W, b.s, P, rows, b.part);
+    k_adj_ends_reduce<<<(5 * W + 1 + 127) / 128, 128, 0, st>>>(b.part, S, W, c, grad, (long long)ow, accumulate);
     const bool tensor = L <= x6_max_mid();
     if (tensor) launch_adj_wgrad(m, b.Z, b.D, b.s, V, ldl, b.part, c, grad + omid, accumulate, b.nsm, st);
     for (int l = 1; l <= (tensor ? 0 : L); ++l) {
         const size_t oW = omid + (size_t)(l - 1) * ((size_t)W * W + W), ob = oW + (size_t)W * W;
         gemm<true, false, false, true>(W, W, V, Dl[l], W, Zl[l - 1], W, b.part, W, nullptr, nullptr, b.s, S, st);
         k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W * W, c, grad + oW, accumulate);
-        colsum<1, false>(Dl[l], V, W, b.s, nullptr, S, b.part, st);
+        k_colsum<<<dim3(W / 32, S), 256, 0, st>>>(Dl[l], V, W, b.s, rows, b.part);
         k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W, c, grad + ob, accumulate);
     }
-    // output layer: w_out from relu(z_L), b_out from the scales alone
-    colsum<1, true>(Zl[L], V, W, b.s, nullptr, S, b.part, st);
-    k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W, c, grad + ow, accumulate);
-    colsum<1, false>(nullptr, V, 1, b.s, nullptr, S, b.part, st);
-    k_adj_reduce<<<1, 32, 0, st>>>(b.part, S, 1, c, grad + ow + W, accumulate);
 }
-
-void adjoint_fill_ones(float *p, long long n, cudaStream_t st) { k_fill<<<256, 256, 0, st>>>(p, n, 1.f); }
 
 // ---------------------------------------------------------------------------
 // Adjoint of an analytic (CSG) SDB.  The min / max fold selects one
