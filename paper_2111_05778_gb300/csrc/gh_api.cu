@@ -542,9 +542,9 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
     return GH_OK;
 }
 
-// The culling masks of an analytic SDB on an N-grid.
-static int ensure_cull(gh_sdb *s, int N) {
-    const long long need = s->kind == GH_SDB_CSG ? cull_words(N, s->nprim) : 0;
+// The culling masks of an analytic SDB (sized once, for every grid).
+static int ensure_cull(gh_sdb *s) {
+    const long long need = s->kind == GH_SDB_CSG ? cull_words(s->nprim) : 0;
     if (s->scr.cap_cull >= need) return GH_OK;
     if (s->scr.cull) cudaFree(s->scr.cull);
     s->scr.cull = nullptr;
@@ -732,7 +732,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         return GH_OK;
     }
     if (s->kind == GH_SDB_CSG) {
-        if (cull_words(g.N, s->nprim) > 0) {
+        if (cull_words(s->nprim) > 0) {
             launch_cull(s->d_item, 1, s->nprim, st);
             ++launches;
         }
@@ -813,7 +813,7 @@ extern "C" int gh_polygonize(const gh_grid *grid, const gh_sdb *csdb, const gh_o
     long long want_m = 8 * N2 > (1 << 16) ? 8 * N2 : (1 << 16);
     long long want_v = 2 * want_m;
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((rc = ensure_scratch(s, g.N, want_m, want_v)) || (rc = ensure_cull(s, g.N))) return rc;
+        if ((rc = ensure_scratch(s, g.N, want_m, want_v)) || (rc = ensure_cull(s))) return rc;
         if (o.method == GH_METHOD_ENUM && (rc = ensure_lattice(s, g.N))) return rc;
         if (wants_index(*out) && (rc = ensure_index(s))) return rc;
         if ((rc = enqueue_once(s, g, o, *out, nsm, st))) return rc;
@@ -1185,7 +1185,7 @@ extern "C" int gh_polygonize_batch(int B, const gh_grid *grids, const gh_sdb *co
     for (int attempt = 0; attempt < 4; ++attempt) {
         for (int b = 0; b < B; ++b)
             if ((rc = ensure_scratch(sd[b], P.g[b].N, want_m[b], want_v[b])) ||
-                (rc = ensure_cull(sd[b], P.g[b].N)) ||
+                (rc = ensure_cull(sd[b])) ||
                 (wants_index(outs[b]) && (rc = ensure_index(sd[b])))) {
                 cudaFree(d_items);
                 return rc;

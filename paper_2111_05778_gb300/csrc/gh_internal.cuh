@@ -221,7 +221,7 @@ unsigned long long wait_limit_ns();
 cudaError_t upload_mc_table(const int32_t *ntri, const int32_t *edges);  // k_pipeline.cu
 void launch_init(Scratch &s, cudaStream_t st);
 void launch_stage_prims(const Prim *src, Prim *dst, int nprim, cudaStream_t st);  // records + bounding radii
-long long cull_words(int N, int nprim);  // words of Scratch::cull (0: no masks)
+long long cull_words(int nprim);  // words of Scratch::cull, whatever the grid (0: no masks)
 void launch_cull(const Item *items, int n, int max_prims, cudaStream_t st);
 void launch_hop_csg(const Item *items, int n_items, int max_prims, int nsm, int block, cudaStream_t st);
 void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st);

@@ -215,9 +215,11 @@ static constexpr int CULL_NB = 32, CULL_MIN = 6;
 __host__ __device__ inline int cull_edge(int N) { return (N + CULL_NB - 1) / CULL_NB; }  // cells per block and axis
 __host__ __device__ inline int cull_blocks(int N) { return (N + cull_edge(N) - 1) / cull_edge(N); }
 
-long long cull_words(int N, int nprim) {
-    const long long nb = cull_blocks(N);
-    return nprim < CULL_MIN ? 0 : nb * nb * nb * ((nprim + 31) / 32);
+// Words of the masks' buffer.  It holds any grid's masks, so that a scene's
+// buffer never moves: a captured batch graph keeps its address, and the number
+// of blocks is not monotone in N (29 per axis at N = 200, 32 at N = 64).
+long long cull_words(int nprim) {
+    return nprim < CULL_MIN ? 0 : (long long)CULL_NB * CULL_NB * CULL_NB * ((nprim + 31) / 32);
 }
 
 // The block index of a cell or lattice index i: i / cull_edge(N), the last
