@@ -38,6 +38,11 @@ enum : unsigned long long {
     FLAG_TIMEOUT = 32ull,        // a bounded device wait gave up
 };
 
+// Flags after which an item's lists must not be read: they overflowed, or a
+// wait ran out and columns were left without a count, tiles without a prefix.
+// Every kernel between hopping and the status words stops on them.
+constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW | FLAG_TIMEOUT;
+
 // Grid parameters as the kernels see them (FP32).
 struct GridP {
     int N;

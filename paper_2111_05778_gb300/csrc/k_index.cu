@@ -23,8 +23,6 @@ namespace gh {
 
 namespace {
 
-constexpr unsigned long long STOPF = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
-
 // index of lattice point c of vertical line `line` in the vertex list, or -1
 __device__ __forceinline__ long long find_point(const Scratch &s, uint32_t line, uint32_t c) {
     uint32_t lo = s.lineoff[line], hi = s.lineoff[line + 1];
@@ -113,11 +111,11 @@ constexpr int EDGE_T = 256, EDGE_E = 4, EDGE_TILE = EDGE_T * EDGE_E;
 __global__ void __launch_bounds__(EDGE_T) k_edges(GridP g, Scratch s, gh_mesh out) {
     __shared__ uint32_t wsum[EDGE_T / 32], base_s;
     __shared__ unsigned long long tile_s;
-    if (s.ctr->flags & STOPF) return;
     const unsigned long long V = s.ctr->verts;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (;;) {
-        if (threadIdx.x == 0) tile_s = atomicAdd(&s.ctr->tick[2], 1ull);
+        // one thread reads the flags: another block's wait may run out meanwhile
+        if (threadIdx.x == 0) tile_s = (s.ctr->flags & STOP_FLAGS) ? V : atomicAdd(&s.ctr->tick[2], 1ull);
         __syncthreads();
         const unsigned long long tile = tile_s, v0 = tile * EDGE_TILE + (unsigned long long)threadIdx.x * EDGE_E;
         if (tile * EDGE_TILE >= V) return;
@@ -170,7 +168,7 @@ __global__ void __launch_bounds__(256) k_edge_count_b(const Item *__restrict__ i
     const unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
     for (int b = 0; b < n; ++b) {
         const Item &it = items[b];
-        if (!wants_index(it.out) || (it.s.ctr->flags & STOPF)) continue;
+        if (!wants_index(it.out) || (it.s.ctr->flags & STOP_FLAGS)) continue;
         const unsigned long long V = it.s.ctr->verts;
         for (unsigned long long v = t; v < V; v += (unsigned long long)gridDim.x * blockDim.x) {
             long long hint[2] = {-1, -1};
@@ -185,7 +183,7 @@ __global__ void __launch_bounds__(256) k_emit_vertices_b(const Item *__restrict_
     const unsigned long long t = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
     for (int b = 0; b < n; ++b) {
         const Item &it = items[b];
-        if (!it.out.vert_xyz || (it.s.ctr->flags & STOPF)) continue;
+        if (!it.out.vert_xyz || (it.s.ctr->flags & STOP_FLAGS)) continue;
         const unsigned long long V = it.s.ctr->verts;
         for (unsigned long long v = t; v < V; v += (unsigned long long)gridDim.x * blockDim.x) {
             if (!it.s.vflag[v]) continue;

@@ -49,7 +49,6 @@ constexpr int EPI_T0 = 64;   // first epilogue thread (warp 2)
 constexpr int TM = 128;      // rows per tile
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint32_t NONE = 0xFFFFFFFFu;
-constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
 
 enum { MODE_HOP = 0, MODE_VERTS = 1, MODE_POINTS = 2 };
 
@@ -171,7 +170,7 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, c
     SmemB<W, TILES> &sm = *reinterpret_cast<SmemB<W, TILES> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *ctl = &sm.ctl;
-    Counters *ctr0 = items[0].s.ctr;  // error flags of a timeout go to the first item
+    Counters *ctr0 = items[0].s.ctr;  // a timeout is flagged here at once, in every item at the end
     const int n_mid = items[0].m.n_mid;
 
     // ---- set-up ----------------------------------------------------------
@@ -647,6 +646,8 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (tid == 0 && (*ctl & CTL_ABORT))  // no item's lists may be read after this
+        for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }

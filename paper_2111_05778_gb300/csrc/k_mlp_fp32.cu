@@ -29,7 +29,6 @@ constexpr int KC = 32;    // K rows per weight chunk
 constexpr int NT = 256;   // threads per CTA
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint32_t NONE = 0xFFFFFFFFu;
-constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
 
 constexpr unsigned long long WAIT_NS = 2000000000ull;
 

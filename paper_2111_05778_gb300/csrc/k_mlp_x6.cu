@@ -63,7 +63,6 @@ constexpr int EPI_T0 = 64;  // first epilogue thread (warp 2)
 constexpr int MAXMID = 8;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint32_t NONE = 0xFFFFFFFFu;
-constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
 constexpr int BAR_EPI = 1;  // named barrier of the epilogue threads
 
 enum { XM_HOP = 0, XM_VERTS = 1, XM_REFINE = 2, XM_POINTS = 3, XM_LATTICE = 4, XM_ADJ = 5 };
@@ -226,7 +225,7 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
     SmemX<W> &sm = *reinterpret_cast<SmemX<W> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *ctl = &sm.ctl;
-    Counters *ctr0 = items[0].s.ctr;  // error flags of a timeout go to the first item
+    Counters *ctr0 = items[0].s.ctr;  // a timeout is flagged here at once, in every item at the end
     const int n_mid = items[0].m.n_mid;
     const int n_gemm = MODE == XM_ADJ ? 2 * n_mid : n_mid;  // products per tile (adjoint: there and back)
 
@@ -691,6 +690,8 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (tid == 0 && (*ctl & CTL_ABORT))  // no item's lists may be read after this
+        for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }

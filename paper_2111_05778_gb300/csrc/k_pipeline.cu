@@ -44,7 +44,6 @@ cudaError_t upload_mc_table(const int32_t *ntri, const int32_t *edges) {
 
 static constexpr uint32_t NONE = 0xFFFFFFFFu;
 static constexpr unsigned FULL = 0xFFFFFFFFu;
-static constexpr unsigned long long STOP_FLAGS = FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW;
 
 // ---------------------------------------------------------------------------
 // Analytic SDB evaluation: exact distances of the seven primitives of
@@ -600,9 +599,10 @@ __device__ __forceinline__ void scan_apply_tile(const uint32_t *__restrict__ in,
 __global__ void __launch_bounds__(SCAN_T) k_scan_columns(Scratch s, long long n) {
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t prefix, tile_s;
-    if (s.ctr->flags & STOP_FLAGS) return;
-    if (threadIdx.x == 0) tile_s = (uint32_t)atomicAdd(&s.ctr->tick[0], 1ull);
+    // one thread reads the flags: another block's wait may run out meanwhile
+    if (threadIdx.x == 0) tile_s = (s.ctr->flags & STOP_FLAGS) ? NONE : (uint32_t)atomicAdd(&s.ctr->tick[0], 1ull);
     __syncthreads();
+    if (tile_s == NONE) return;
     const long long tile = tile_s, base = tile * SCAN_TILE + (long long)threadIdx.x * SCAN_IPT;
     uint32_t v[SCAN_IPT], sum = 0;
 #pragma unroll
@@ -733,9 +733,9 @@ __device__ __forceinline__ void emit_line(const Scratch &s, const uint32_t *bits
 __global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s, long long lb0) {
     extern __shared__ uint32_t lbits[];
     __shared__ uint32_t wsum[LINES_T / 32], base_s, group_s;
-    if (s.ctr->flags & STOP_FLAGS) return;
-    if (threadIdx.x == 0) group_s = (uint32_t)atomicAdd(&s.ctr->tick[1], 1ull);
+    if (threadIdx.x == 0) group_s = (s.ctr->flags & STOP_FLAGS) ? NONE : (uint32_t)atomicAdd(&s.ctr->tick[1], 1ull);
     __syncthreads();
+    if (group_s == NONE) return;
     const int NW = (g.N + 1 + 31) >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t *bits = lbits + wid * NW * 32;
     const long long tiles = line_tiles(g.N), t = (long long)group_s * (LINES_T / 32) + wid;

@@ -1,0 +1,65 @@
+"""What a run-out wait leaves behind: no kernel after it may read the lists it
+left unfinished, whatever the scratch held before (a new SDB's uninitialised
+buffers, another grid's), and every item of the launch reports it.  With the
+limit at 0 every wait on the engines' own work runs out at once; nothing is
+made to hang."""
+import contextlib
+
+import numpy as np
+import pytest
+
+import meshutil
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2111_05778_gb300 import gh, synth  # noqa: E402
+
+
+@contextlib.contextmanager
+def no_waiting():
+    gh.set_wait_limit_ns(0)
+    try:
+        yield
+    finally:
+        torch.cuda.synchronize()
+        gh.set_wait_limit_ns(2_000_000_000)
+
+
+def _tris(m):
+    return meshutil.canonical_tris(m.tri_keys.cpu().numpy())
+
+
+@pytest.mark.parametrize("width", [64, 128, 256])
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_new_sdb_and_another_grid(width, precision):
+    p = synth.mlp_params(2, width)
+    eps = gh.MlpSdb(p, width).calibrate(48) if precision == "bf16" else None
+    gh.release_cache()
+    sdb = gh.MlpSdb(p, width)  # its scratch is allocated by the failing call
+    for N in (48, 33, 70):
+        with no_waiting(), pytest.raises(gh.GhError) as e:
+            gh.polygonize(sdb, N, precision=precision, eps=eps, indexed=True)
+        assert e.value.code == gh.GH_ERR_CUDA and "timed out" in str(e.value)
+    ref = gh.MlpSdb(p, width)
+    for N in (33, 70):
+        m = gh.polygonize(sdb, N, precision=precision, eps=eps, indexed=True)
+        r = gh.polygonize(ref, N, precision=precision, eps=eps, indexed=True)
+        assert m.n_tris > 0 and np.array_equal(_tris(m), _tris(r))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_every_item_of_a_batch_reports_it(precision):
+    sdbs = [gh.MlpSdb(synth.mlp_params(s, 64), 64) for s in (1, 2, 3)] + [gh.CsgSdb(synth.csg_prims(0))]
+    Ns = [40, 33, 48, 40]
+    bt = gh.Batch(sdbs, Ns, [16 * n * n + 4096 for n in Ns], precision=precision, eps=1e-3, indexed=True)
+    with no_waiting():
+        assert bt.run(sync=False) == gh.GH_OK
+        torch.cuda.synchronize()
+        st = [b.stats_dict() for b in bt.bufs]
+    assert [s["status"] for s in st] == [gh.GH_ERR_CUDA] * 3 + [gh.GH_OK]
+    assert all(s["triangles"] == 0 for s in st[:3]) and st[3]["triangles"] > 0
+    assert bt.run() == gh.GH_OK
+    for b, (s, n) in enumerate(zip(sdbs, Ns)):
+        single = gh.polygonize(s, n, precision=precision if b < 3 else "fp32", eps=1e-3, indexed=True)
+        assert np.array_equal(_tris(bt.mesh(b)), _tris(single))
