@@ -408,7 +408,11 @@ int gh_last_profile(gh_profile *out);
  * keeps waiting for its copy; the call then reports GH_ERR_CUDA ("a bounded
  * device wait timed out") and the SDB stays usable.  Default and maximum 2 s
  * (2e9); 0 makes every such wait run out at once, satisfied or not -- a way
- * to exercise the timeout path.  Process-wide; later launches take it. */
+ * to exercise the timeout path.  Process-wide; later launches take it.
+ * The one-pass scans of gh_polygonize and gh_polygonize_csg_noalloc wait too
+ * (a block for the sums of the blocks before it), analytic SDBs included: for up
+ * to 2 s whatever the limit, and with a limit of 0 not at all, so that these
+ * calls report GH_ERR_CUDA then. */
 int gh_set_wait_limit_ns(uint64_t ns);
 
 /* Copies the library's Marching Cubes table to host memory: ntri[256] and

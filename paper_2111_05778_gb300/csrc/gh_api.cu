@@ -1461,6 +1461,8 @@ extern "C" int gh_polygonize_csg_noalloc(const gh_grid *grid, const gh_csg_prim 
     Counters h;
     GH_CUDA(cudaMemcpyAsync(&h, c.ctr, sizeof(h), cudaMemcpyDeviceToHost, st));
     GH_CUDA(cudaStreamSynchronize(st));
+    // a wait that ran out leaves the other counters meaningless
+    if (h.flags & FLAG_TIMEOUT) return fail(GH_ERR_CUDA, "a bounded device wait timed out");
     if (h.flags & FLAG_MARK_OVERFLOW)
         return fail(GH_ERR_CAPACITY, "scene marks %llu cells; the no-allocation scratch holds %lld", h.marks,
                     c.cap_marks);

@@ -596,7 +596,7 @@ __device__ __forceinline__ void scan_apply_tile(const uint32_t *__restrict__ in,
 }
 
 // Column counts -> column offsets of one call, in one pass.
-__global__ void __launch_bounds__(SCAN_T) k_scan_columns(Scratch s, long long n) {
+__global__ void __launch_bounds__(SCAN_T) k_scan_columns(Scratch s, long long n, bool expire) {
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t prefix, tile_s;
     // one thread reads the flags: another block's wait may run out meanwhile
@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_columns(Scratch s, long long n)
     uint32_t tot;
     const uint32_t loc = block_excl_scan(sum, wsum, tot);
     if (threadIdx.x < 32) {
-        const uint32_t p = lb_prefix(s.lb + 1, s.lb[0], tile, tot, s.ctr);
+        const uint32_t p = lb_prefix(s.lb + 1, s.lb[0], tile, tot, s.ctr, expire);
         if (threadIdx.x == 0) prefix = p;
     }
     __syncthreads();
@@ -730,7 +730,7 @@ __device__ __forceinline__ void emit_line(const Scratch &s, const uint32_t *bits
 }
 
 // One call: gather, count, scan and emit in one pass, a block per four tiles.
-__global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s, long long lb0) {
+__global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s, long long lb0, bool expire) {
     extern __shared__ uint32_t lbits[];
     __shared__ uint32_t wsum[LINES_T / 32], base_s, group_s;
     if (threadIdx.x == 0) group_s = (s.ctr->flags & STOP_FLAGS) ? NONE : (uint32_t)atomicAdd(&s.ctr->tick[1], 1ull);
@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(LINES_T) k_lines(GridP g, Scratch s, long long
         tot += wsum[q];
     }
     if (wid == 0) {
-        const uint32_t p = lb_prefix(s.lb + lb0, s.lb[0], group_s, tot, s.ctr);
+        const uint32_t p = lb_prefix(s.lb + lb0, s.lb[0], group_s, tot, s.ctr, expire);
         if (lane == 0) base_s = p;
     }
     __syncthreads();
@@ -780,10 +780,11 @@ long long lb_words(int N) { return 1 + column_tiles(N) + line_groups(N); }
 
 void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st) {
     const long long ct = column_tiles(g.N);
-    k_scan_columns<<<(int)ct, SCAN_T, 0, st>>>(s, (long long)g.N * g.N);
+    const bool expire = wait_limit_ns() == 0;
+    k_scan_columns<<<(int)ct, SCAN_T, 0, st>>>(s, (long long)g.N * g.N, expire);
     k_scatter_marks<<<1024, 256, 0, st>>>(s);
     const size_t lsm = (size_t)((g.N + 1 + 31) / 32) * LINES_T * sizeof(uint32_t);  // <= 33 KB at N = 2048
-    k_lines<<<(int)line_groups(g.N), LINES_T, lsm, st>>>(g, s, 1 + ct);
+    k_lines<<<(int)line_groups(g.N), LINES_T, lsm, st>>>(g, s, 1 + ct, expire);
 }
 
 // ---------------------------------------------------------------------------

@@ -3,7 +3,8 @@
 // word, and the block of the next tile adds up its predecessors' words until
 // it meets one that already holds the whole sum before it.  A tile waits only
 // for tiles taken earlier, whose blocks are running, so every wait ends; it is
-// bounded all the same (2 s of %globaltimer, then the timeout flag is set).
+// bounded all the same (2 s of %globaltimer, then the timeout flag is set; with
+// gh_set_wait_limit_ns(0) every such wait runs out at once).
 // A status word is call number << 34 | state << 32 | value, so words of
 // earlier calls read as not written and nothing has to be cleared.
 #pragma once
@@ -18,13 +19,16 @@ namespace {
 constexpr unsigned long long LB_SUM = 1ull << 32, LB_PREFIX = 2ull << 32;
 
 // The sum of the tiles before `tile`; the first warp of the block calls it.
+// expire: give up at once, as if the wait had run out (its caller's test device).
 __device__ __forceinline__ uint32_t lb_prefix(unsigned long long *words, unsigned long long call, long long tile,
-                                              uint32_t sum, Counters *ctr) {
+                                              uint32_t sum, Counters *ctr, bool expire) {
     const int lane = threadIdx.x & 31;
     volatile unsigned long long *w = words;
     const unsigned long long tag = call << 34;
     uint32_t before = 0;
-    if (tile > 0) {
+    if (tile > 0 && expire) {
+        if (lane == 0) atomicOr(&ctr->flags, FLAG_TIMEOUT);
+    } else if (tile > 0) {
         if (lane == 0) w[tile] = tag | LB_SUM | sum;
         for (long long last = tile - 1; last >= 0; last -= 32) {
             const long long t = last - lane;

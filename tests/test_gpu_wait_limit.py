@@ -63,3 +63,23 @@ def test_every_item_of_a_batch_reports_it(precision):
     for b, (s, n) in enumerate(zip(sdbs, Ns)):
         single = gh.polygonize(s, n, precision=precision if b < 3 else "fp32", eps=1e-3, indexed=True)
         assert np.array_equal(_tris(bt.mesh(b)), _tris(single))
+
+
+@pytest.mark.parametrize("N", [64, 200])
+def test_analytic_scans_report_it(N):
+    """The scans of the lists are the analytic pipeline's only waits, in the
+    no-allocation entry point too."""
+    prims = synth.csg_prims(1)
+    sdb, dev = gh.CsgSdb(prims), gh.csg_prims_device(prims)
+    bufs = gh.Buffers(16 * N * N + 4096, keys=True)
+
+    def noalloc():
+        return gh.polygonize_csg_noalloc(dev, len(prims), N, bufs)
+
+    for call in (noalloc, lambda: gh.polygonize(sdb, N, indexed=True)):
+        with no_waiting(), pytest.raises(gh.GhError) as e:
+            call()
+        assert e.value.code == gh.GH_ERR_CUDA and "timed out" in str(e.value)
+    assert noalloc() == gh.GH_OK
+    m = gh.polygonize(sdb, N, indexed=True)
+    assert np.array_equal(_tris(m), meshutil.canonical_tris(bufs.tri_keys[:int(bufs.counts[0])].cpu().numpy()))
