@@ -368,13 +368,17 @@ int64_t gh_column_order(int32_t N, int64_t c);
  * vertices in chunks of GH_ADJOINT_CHUNK (the SDB keeps a work buffer of
  * 2 (n_mid + 1) width floats per chunk vertex); the result is the sum of the
  * chunks' gradients in chunk order, so it equals, bit for bit, the sum of
- * separate calls on those chunks. */
+ * separate calls on those chunks.  The call is asynchronous and has no status
+ * of the device: where a bounded wait ran out (gh_set_wait_limit_ns) the
+ * gradient is NaN. */
 #define GH_ADJOINT_CHUNK 131072
 int gh_backward(const gh_sdb *sdb, const float *verts, const float *dL_dv, int64_t V, float *dL_dtheta,
                 void *stream);
 
 /* Evaluates f at n points p[n][3] (device float32) into out[n] (device
- * float32) with the given precision -- the evaluator the hopper uses. */
+ * float32) with the given precision -- the evaluator the hopper uses.
+ * Asynchronous, without a status of the device: rows for which a bounded wait
+ * ran out (gh_set_wait_limit_ns) are NaN. */
 int gh_eval(const gh_sdb *sdb, const float *p, int64_t n, float *out, int32_t precision, void *stream);
 
 /* Profiling aid.  gh_set_profiling(1) makes every later gh_polygonize on the
@@ -400,15 +404,20 @@ int gh_set_profiling(int enable);
 int gh_last_profile(gh_profile *out);
 
 /* The limit, in nanoseconds, of the bounded waits the neural engines make
- * on their own work (BF16 and split-BF16 tensor-core engines: one role waiting
- * for another through an mbarrier; FP32 engine: a weight copy landing).  When
- * a wait runs out the kernel records it, the BF16 engines' roles leave their
+ * on their own work (BF16 and split-BF16 tensor-core engines, which also run the
+ * adjoint: one role waiting for another through an mbarrier; FFMA engine of the
+ * networks of more than 8 hidden layers: a weight copy landing).  When a wait
+ * runs out the kernel records it.  The tensor-core engines' roles leave their
  * loops (copies in flight land and issued MMAs complete, with a fixed 2 s
- * limit, before tensor memory is freed) and the FP32 engine records it and
- * keeps waiting for its copy; the call then reports GH_ERR_CUDA ("a bounded
- * device wait timed out") and the SDB stays usable.  Default and maximum 2 s
- * (2e9); 0 makes every such wait run out at once, satisfied or not -- a way
- * to exercise the timeout path.  Process-wide; later launches take it.
+ * limit, before tensor memory is freed); no later kernel of the call reads what
+ * they left unfinished, the polygonizing calls report GH_ERR_CUDA ("a bounded
+ * device wait timed out"; asynchronous ones in stats->status, batches in every
+ * item of the launch), and gh_eval and gh_backward, which have no status, write
+ * NaN.  The FFMA engine keeps waiting for its copy: gh_eval and gh_backward give
+ * their usual values, a polygonizing call reports it all the same.  The SDB
+ * stays usable.  Default and maximum 2 s (2e9); 0 makes every such wait run out
+ * at once, satisfied or not -- a way to exercise the timeout path.
+ * Process-wide; later launches take it.
  * The one-pass scans of gh_polygonize and gh_polygonize_csg_noalloc wait too
  * (a block for the sums of the blocks before it), analytic SDBs included: for up
  * to 2 s whatever the limit, and with a limit of 0 not at all, so that these

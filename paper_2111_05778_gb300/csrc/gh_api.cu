@@ -355,7 +355,7 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     auto up = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
     unsigned char *base;
     if (dev_alloc(s, &base, up(sizeof(float) * np) + 2 * up(sizeof(float) * mw) + up(sizeof(float) * h.n_mid * W) +
-                                up(2 * mw) + 2 * up(6 * mw)))
+                                up(2 * mw) + 2 * up(6 * mw) + up(sizeof(Counters))))
         return GH_ERR_CUDA;
     auto take = [&](size_t bytes) {
         unsigned char *p = base;
@@ -366,6 +366,8 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     float *d_wt = (float *)take(sizeof(float) * mw), *d_wtb = (float *)take(sizeof(float) * mw);
     float *d_bm = (float *)take(sizeof(float) * h.n_mid * W);
     uint16_t *d_wbf = (uint16_t *)take(2 * mw), *d_wx6 = (uint16_t *)take(6 * mw), *d_wx6t = (uint16_t *)take(6 * mw);
+    s->mlp.err = (Counters *)take(sizeof(Counters));
+    GH_CUDA(cudaMemsetAsync(s->mlp.err, 0, sizeof(Counters), 0));
     GH_CUDA(cudaMemcpy(s->d_params, P, sizeof(float) * np, cudaMemcpyHostToDevice));
     launch_prep_mlp(s->d_params, W, h.n_mid, d_wt, d_wtb, d_wbf, d_wx6, d_wx6t, d_bm, 0);
     GH_CUDA(cudaGetLastError());

@@ -153,6 +153,7 @@ struct MlpDev {
     const uint16_t *wbf;  // n_mid x BF16 hidden weights in the tensor-core tile layout
     const uint16_t *wx6;  // n_mid x 3 BF16 parts (low, middle, high) of the hidden weights, same layout
     const uint16_t *wx6t; // the same of the transposed weights, last layer first (adjoint)
+    Counters *err;        // where the launches without an item (point lists, adjoint) flag a timeout
 };
 
 // Scratch of one polygonization (device pointers) and its capacities.
@@ -274,6 +275,8 @@ void launch_hop_mlp_x6(const Item *items, int n_items, int width, int nsm, cudaS
 void launch_eval_vertices_mlp_x6(const Item *items, int n_items, int width, int nsm, bool refine_list,
                                  cudaStream_t st);
 void launch_lattice_mlp_x6(const Item *items, int width, int nsm, cudaStream_t st);
+// (a block that gave up a wait writes NaN to all its rows, and flags it in m.err;
+// so do the BF16 points and the adjoint)
 void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, float *out, int nsm, cudaStream_t st);
 // the adjoint's forward pass and delta chain over V vertices: relu(z_l) into
 // A + l*ldl, delta_l into D + l*ldl (l = 0..n_mid), s_v into s; mask is work

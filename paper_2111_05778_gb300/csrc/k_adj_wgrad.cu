@@ -267,7 +267,13 @@ __global__ void __launch_bounds__(NLD + 32, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid < ROWS) bpart[(size_t)unit * BMR + tid] = (sm.bsum[0][tid] + sm.bsum[1][tid]) + (sm.bsum[2][tid] + sm.bsum[3][tid]);
+    if (*ctl & CTL_ABORT) {  // a wait ran out: no sum of this CTA is one, which NaN says
+        const float nan = __int_as_float(0x7FC00000);
+        for (int i = tid; i < ROWS * W; i += blockDim.x) part[(size_t)unit * BMR * W + i] = nan;
+        if (tid < ROWS) bpart[(size_t)unit * BMR + tid] = nan;
+    } else if (tid < ROWS) {
+        bpart[(size_t)unit * BMR + tid] = (sm.bsum[0][tid] + sm.bsum[1][tid]) + (sm.bsum[2][tid] + sm.bsum[3][tid]);
+    }
     if (warp == NLD / 32)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
@@ -325,8 +331,7 @@ size_t adj_wgrad_floats(int W, int n_mid, int nsm) {
 
 void launch_adj_wgrad(const MlpDev &m, const float *A, const float *D, const float *s, long long V, long long ldl,
                       float *part, float c, float *dst, bool accumulate, int nsm, cudaStream_t st) {
-    static thread_local Counters *ctr = nullptr;
-    if (!ctr) cudaMalloc(&ctr, sizeof(Counters));
+    Counters *const ctr = m.err;
     switch (m.width) {
     case 64: wgrad<64>(m.n_mid, A, D, s, V, ldl, part, c, dst, accumulate, ctr, nsm, st); break;
     case 128: wgrad<128>(m.n_mid, A, D, s, V, ldl, part, c, dst, accumulate, ctr, nsm, st); break;

@@ -105,6 +105,8 @@ struct SmemB {
     int ctl;
 };
 
+#define NAN_OUT __int_as_float(0x7FC00000)
+
 __device__ __forceinline__ float outer_f(const MlpDev &m, float x, float y, float z, float g) {
     const float r = sqrtf(fmaf(x, x, fmaf(y, y, z * z)));
     return (fmaf(m.alpha, g, m.radial * r - m.r0) / m.beta) * m.inv_lam;
@@ -158,7 +160,7 @@ __device__ __forceinline__ void load_item(SmemB<W, TILES> &sm, int t, const MlpD
 template <int W, int MODE, int TILES>
 __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, ctas_of<W, TILES>())
     k_mlp_bf16(const Item *__restrict__ items, int n_items, const float *__restrict__ pts, long long npts,
-               float *__restrict__ outv, unsigned long long wait_ns) {
+               float *__restrict__ outv, Counters *err, unsigned long long wait_ns) {
     extern __shared__ uint8_t smem_raw[];
     constexpr int HALVES = halves_of<W, TILES>(), ET = TM * HALVES;  // epilogue threads per row, per tile
     constexpr int KS = ks_of<W>(), KB = W / KS;  // K-blocks per hidden layer
@@ -170,7 +172,7 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, c
     SmemB<W, TILES> &sm = *reinterpret_cast<SmemB<W, TILES> *>(smem_raw + ((1024 - (su32(smem_raw) & 1023)) & 1023));
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *ctl = &sm.ctl;
-    Counters *ctr0 = items[0].s.ctr;  // a timeout is flagged here at once, in every item at the end
+    Counters *ctr0 = MODE == MODE_POINTS ? err : items[0].s.ctr;  // a timeout is flagged here at once, in every item at the end
     const int n_mid = items[0].m.n_mid;
 
     // ---- set-up ----------------------------------------------------------
@@ -468,6 +470,7 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, c
             const bool any = bar_any(bar, ET, live);
             // the abort decision goes through the barrier so that it is uniform
             if (bar_any(bar, ET, (*ctl & CTL_ABORT) != 0)) {
+                if (MODE == MODE_POINTS && own && live) outv[idx] = NAN_OUT;  // taken, not evaluated
                 if (own && row == 0) {
                     vdone[t] = 1;
                     __threadfence_block();
@@ -637,7 +640,7 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, c
                     if (!isfinite(f)) atomicOr(&ctr->flags, FLAG_NONFINITE);
                     it->s.vval[idx] = f;
                 } else {
-                    outv[idx] = f;
+                    outv[idx] = *ctl & CTL_ABORT ? NAN_OUT : f;
                 }
             }
         }
@@ -646,14 +649,28 @@ __global__ void __launch_bounds__(EPI_T0 + TM * halves_of<W, TILES>() * TILES, c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid == 0 && (*ctl & CTL_ABORT))  // no item's lists may be read after this
-        for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
+    if (*ctl & CTL_ABORT) {
+        if (tid == 0)  // no item's lists may be read after this
+            for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
+        // a point list has no status: NaN says that the CTA gave up, in the rows it
+        // had taken (above) and in what is left of the queue, should nobody else take it
+        if (MODE == MODE_POINTS && warp == 0) {
+            for (;;) {
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(&items[0].s.ctr->next_tile, 32ull);
+                base = __shfl_sync(FULL, base, 0);
+                if (base >= (unsigned long long)npts) break;
+                if (base + lane < (unsigned long long)npts) outv[base + lane] = NAN_OUT;
+            }
+        }
+    }
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
 template <int W, int MODE, int TILES>
-void launch_bf16(const Item *items, int n_items, const float *p, long long n, float *out, int nsm, cudaStream_t st) {
+void launch_bf16(const Item *items, int n_items, const float *p, long long n, float *out, Counters *err, int nsm,
+                 cudaStream_t st) {
     const size_t smem = sizeof(SmemB<W, TILES>) + 1024;
     cudaFuncSetAttribute(k_mlp_bf16<W, MODE, TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int grid = nsm * ctas_of<W, TILES>();
@@ -661,7 +678,8 @@ void launch_bf16(const Item *items, int n_items, const float *p, long long n, fl
         const long long tiles = (n + 128 * TILES - 1) / (128 * TILES);
         if (grid > tiles) grid = (int)(tiles < 1 ? 1 : tiles);
     }
-    k_mlp_bf16<W, MODE, TILES><<<grid, EPI_T0 + TM * halves_of<W, TILES>() * TILES, smem, st>>>(items, n_items, p, n, out, wait_limit_ns());
+    k_mlp_bf16<W, MODE, TILES><<<grid, EPI_T0 + TM * halves_of<W, TILES>() * TILES, smem, st>>>(items, n_items, p, n, out, err,
+                                                                                           wait_limit_ns());
 }
 
 }  // namespace
@@ -682,19 +700,19 @@ int bf16_max_mid(int width) { return width == 256 ? maxmid_of<256>() : maxmid_of
 // 0.52 -> 0.54).  At width 128 three CTAs of one tile are slower than one of
 // two from N = 300 on (hop at N = 1000 5.11 against 4.83 ms).
 template <int W, int MODE>
-void launch_tiles(int tiles, const Item *items, int n_items, const float *p, long long n, float *out, int nsm,
-                  cudaStream_t st) {
+void launch_tiles(int tiles, const Item *items, int n_items, const float *p, long long n, float *out, Counters *err,
+                  int nsm, cudaStream_t st) {
     constexpr int T = W == 64 ? 1 : 2;
-    if (tiles == 1) launch_bf16<W, MODE, 1>(items, n_items, p, n, out, nsm, st);
-    else launch_bf16<W, MODE, T>(items, n_items, p, n, out, nsm, st);
+    if (tiles == 1) launch_bf16<W, MODE, 1>(items, n_items, p, n, out, err, nsm, st);
+    else launch_bf16<W, MODE, T>(items, n_items, p, n, out, err, nsm, st);
 }
 
 void launch_hop_mlp_bf16(const Item *items, int n_items, int width, int nsm, int tiles, cudaStream_t st) {
-    GH_BF16_W(width, (launch_tiles<WW, MODE_HOP>(tiles, items, n_items, nullptr, 0, nullptr, nsm, st)))
+    GH_BF16_W(width, (launch_tiles<WW, MODE_HOP>(tiles, items, n_items, nullptr, 0, nullptr, nullptr, nsm, st)))
 }
 
 void launch_eval_vertices_mlp_bf16(const Item *items, int n_items, int width, int nsm, int tiles, cudaStream_t st) {
-    GH_BF16_W(width, (launch_tiles<WW, MODE_VERTS>(tiles, items, n_items, nullptr, 0, nullptr, nsm, st)))
+    GH_BF16_W(width, (launch_tiles<WW, MODE_VERTS>(tiles, items, n_items, nullptr, 0, nullptr, nullptr, nsm, st)))
 }
 
 void launch_eval_points_mlp_bf16(const MlpDev &m, const float *p, long long n, float *out, int nsm,
@@ -710,7 +728,7 @@ void launch_eval_points_mlp_bf16(const MlpDev &m, const float *p, long long n, f
     h.kind = 1;
     cudaMemsetAsync(ctr, 0, sizeof(Counters), st);
     cudaMemcpyAsync(ditem, &h, sizeof(Item), cudaMemcpyHostToDevice, st);
-    GH_BF16_W(m.width, (launch_tiles<WW, MODE_POINTS>(2, ditem, 1, p, n, out, nsm, st)))
+    GH_BF16_W(m.width, (launch_tiles<WW, MODE_POINTS>(2, ditem, 1, p, n, out, m.err, nsm, st)))
 }
 
 }  // namespace gh

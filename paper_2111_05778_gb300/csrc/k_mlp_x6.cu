@@ -690,8 +690,17 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid == 0 && (*ctl & CTL_ABORT))  // no item's lists may be read after this
-        for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
+    if (*ctl & CTL_ABORT) {
+        if (tid == 0)  // no item's lists may be read after this
+            for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
+        // calls without a status: NaN in every row of this CTA says that it gave
+        // up (s_v multiplies every term of the gradient's sums)
+        if ((MODE == XM_POINTS || MODE == XM_ADJ) && tid < TM) {
+            float *const dst = MODE == XM_POINTS ? outv : adj.s;
+            for (long long i = (long long)blockIdx.x * TM + tid; i < npts; i += (long long)gridDim.x * TM)
+                dst[i] = __int_as_float(0x7FC00000);
+        }
+    }
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
@@ -738,13 +747,11 @@ void launch_lattice_mlp_x6(const Item *items, int width, int nsm, cudaStream_t s
 }
 
 // A network's descriptor for the kernels that take points instead of an item
-// (its counters only carry the error flag of a timeout, which nothing reads).
+// (its counters only carry the error flag of a timeout).
 static Item points_item(const MlpDev &m) {
-    static thread_local Counters *ctr = nullptr;
-    if (!ctr) cudaMalloc(&ctr, sizeof(Counters));
     Item h{};
     h.m = m;
-    h.s.ctr = ctr;
+    h.s.ctr = m.err;
     h.kind = 1;
     return h;
 }

@@ -83,3 +83,48 @@ def test_analytic_scans_report_it(N):
     assert noalloc() == gh.GH_OK
     m = gh.polygonize(sdb, N, indexed=True)
     assert np.array_equal(_tris(m), meshutil.canonical_tris(bufs.tri_keys[:int(bufs.counts[0])].cpu().numpy()))
+
+
+def _surface(V):
+    rng = np.random.default_rng(V)
+    u = rng.standard_normal((V, 3))
+    v = (0.6 * u / np.linalg.norm(u, axis=1, keepdims=True)).astype(np.float32)
+    return torch.from_numpy(v).cuda(), torch.from_numpy(rng.standard_normal((V, 3)).astype(np.float32)).cuda()
+
+
+@pytest.mark.parametrize("width", [64, 128, 256])
+def test_calls_without_a_status_give_nan(width):
+    sdb = gh.MlpSdb(synth.mlp_params(2, width), width)
+    for n in (1, 129, 50001):
+        P = torch.from_numpy(synth.uniform_points(3, n)).cuda()
+        for precision in ("fp32", "bf16", "bf16x6"):
+            ref = gh.eval_points(sdb, P, precision)
+            with no_waiting():
+                f = gh.eval_points(sdb, P, precision)
+            assert bool(torch.isnan(f).all()), (n, precision)
+            again = gh.eval_points(sdb, P, precision)
+            if precision == "bf16" and width == 256:
+                # its last bits depend on the tile a row falls into (the order of the
+                # K-blocks follows the ring's reuse between tiles)
+                assert bool(torch.isfinite(again).all())
+            else:
+                assert torch.equal(again, ref)
+    for V in (33, 2080):
+        v, dl = _surface(V)
+        ref = gh.backward(sdb, v, dl)
+        assert bool(torch.isfinite(ref).all())
+        with no_waiting():
+            g = gh.backward(sdb, v, dl)
+        assert bool(torch.isnan(g).all()), V
+        assert torch.equal(gh.backward(sdb, v, dl), ref)
+
+
+def test_deep_networks_keep_waiting():
+    p = synth.pack_layers(synth.mlp_layers(7, 64, 9))
+    sdb = gh.MlpSdb(p, 64, 9)
+    P = torch.from_numpy(synth.uniform_points(3, 5000)).cuda()
+    v, dl = _surface(545)
+    f, g = gh.eval_points(sdb, P), gh.backward(sdb, v, dl)
+    with no_waiting():
+        f0, g0 = gh.eval_points(sdb, P), gh.backward(sdb, v, dl)
+    assert torch.equal(f0, f) and torch.equal(g0, g)
