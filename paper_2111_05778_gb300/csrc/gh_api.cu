@@ -995,6 +995,7 @@ extern "C" int gh_sdb_calibrate(gh_sdb *s, const gh_grid *grid, int64_t n_points
     Counters hc;
     GH_CUDA(cudaMemcpyAsync(&hc, c.ctr, sizeof(hc), cudaMemcpyDeviceToHost, st));
     GH_CUDA(cudaStreamSynchronize(st));
+    if (hc.flags & FLAG_TIMEOUT) return fail(GH_ERR_CUDA, "calibration: a bounded device wait timed out");
     const long long nv = (hc.flags & (FLAG_MARK_OVERFLOW | FLAG_VERT_OVERFLOW)) ? 0 : (long long)hc.verts;
     const long long nmax = n_points > nv ? n_points : nv;
     float *p = nullptr, *f32 = nullptr, *f16 = nullptr;
@@ -1004,6 +1005,7 @@ extern "C" int gh_sdb_calibrate(gh_sdb *s, const gh_grid *grid, int64_t n_points
     GH_CUDA(cudaMalloc((void **)&f16, sizeof(float) * (nmax + 1)));
     GH_CUDA(cudaMalloc((void **)&d_max, sizeof(unsigned int)));
     GH_CUDA(cudaMemsetAsync(d_max, 0, sizeof(unsigned int), st));
+    GH_CUDA(cudaMemsetAsync(s->mlp.err, 0, sizeof(Counters), st));  // the point lists' timeouts are flagged there
     const float ext = g.h * (float)g.N;
     launch_rand_points(p, n_points, g.lo, ext, seed, st);
     rc = bf16_gap(s, p, n_points, f32, f16, d_max, nsm, st);
@@ -1014,8 +1016,10 @@ extern "C" int gh_sdb_calibrate(gh_sdb *s, const gh_grid *grid, int64_t n_points
     unsigned int hmax = 0;
     if (!rc) {
         cudaError_t e = cudaMemcpyAsync(&hmax, d_max, sizeof(hmax), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, s->mlp.err, sizeof(hc), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = fail(GH_ERR_CUDA, "calibration: %s", cudaGetErrorString(e));
+        else if (hc.flags & FLAG_TIMEOUT) rc = fail(GH_ERR_CUDA, "calibration: a bounded device wait timed out");
     }
     cudaFree(p);
     cudaFree(f32);

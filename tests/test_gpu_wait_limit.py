@@ -128,3 +128,16 @@ def test_deep_networks_keep_waiting():
     with no_waiting():
         f0, g0 = gh.eval_points(sdb, P), gh.backward(sdb, v, dl)
     assert torch.equal(f0, f) and torch.equal(g0, g)
+
+
+@pytest.mark.parametrize("width", [64, 256])
+@pytest.mark.parametrize("n_points", [0, 4096])
+def test_calibration_reports_it_and_keeps_its_bound(width, n_points):
+    sdb = gh.MlpSdb(synth.mlp_params(2, width), width)
+    with no_waiting(), pytest.raises(gh.GhError) as e:
+        sdb.calibrate(40, n_points=n_points)
+    assert e.value.code == gh.GH_ERR_CUDA and "timed out" in str(e.value)
+    assert sdb.eps is None
+    with pytest.raises(gh.GhError):  # no bound was stored
+        gh.polygonize(sdb, 40, precision="bf16")
+    assert 0.0 < sdb.calibrate(40, n_points=n_points) < 1e-2
