@@ -450,9 +450,10 @@ static void free_scratch(gh_sdb *s) {
     s->scr_N = 0;
 }
 
-// Adjoint buffers above this (1 GB: 2 (n_mid + 1) width floats per vertex, 85 k
-// vertices at width 256 and 5 hidden layers) stay out of the pool.
-constexpr size_t POOL_ADJ_FLOATS = (size_t)1 << 28;
+// The adjoint buffers in the pool hold no more than this together (2.6 GB: one
+// buffer of any network the tensor-core adjoint takes; 2.5 GB at width 256 and 8
+// hidden layers, 0.8 GB at width 128 and 5); others are freed.
+constexpr size_t POOL_ADJ_FLOATS = (size_t)640 << 20;
 
 extern "C" int gh_destroy_sdb(gh_sdb *s) {
     if (!s) return GH_OK;
@@ -463,7 +464,9 @@ extern "C" int gh_destroy_sdb(gh_sdb *s) {
     if (s->scr.ctr) {
         std::lock_guard<std::mutex> lk(g_pool_mu);
         if (g_pool.size() < POOL_MAX) {
-            const bool keep = s->adj_floats <= POOL_ADJ_FLOATS;
+            size_t held = s->adj_floats;
+            for (const PoolEntry &e : g_pool) held += e.adj_floats;
+            const bool keep = held <= POOL_ADJ_FLOATS;
             g_pool.push_back(PoolEntry{s->scr, s->scr_N, s->device, keep ? s->adj : nullptr, keep ? s->adj_floats : 0});
             s->scr = Scratch{};
             s->scr_N = 0;
@@ -488,8 +491,7 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
                 c = e.scr;
                 s->scr_N = e.N;
                 s->item_valid = false;
-                if (s->adj_floats < e.adj_floats) {
-                    if (s->adj) cudaFree(s->adj);
+                if (!s->adj) {  // (its own buffer stays: a captured gh_backward may hold it)
                     s->adj = e.adj;
                     s->adj_floats = e.adj_floats;
                 } else if (e.adj) {
@@ -1335,11 +1337,14 @@ extern "C" int gh_backward(const gh_sdb *cs, const float *verts, const float *dL
         return GH_OK;
     }
     std::lock_guard<std::mutex> lk(s->mu);
-    const int W = s->mlp.width, L = s->mlp.n_mid, S = 76;  // 2 x 76 weight-gradient tiles: one per SM
-    // vertices per chunk: the stored activations and deltas of a chunk take
-    // 2 (L + 1) W floats per vertex (1.6 GB at W = 256, L = 5, a full chunk; a
-    // smaller mesh takes no more than its vertices need)
-    const int VCHUNK = V < GH_ADJOINT_CHUNK ? (int)((V + 4095) / 4096 * 4096) : GH_ADJOINT_CHUNK;
+    const int W = s->mlp.width, L = s->mlp.n_mid;
+    // vertex ranges of the first and the last layer's sums (and of the FFMA path's
+    // weight sums: 2 x 76 tiles at width 256, one per SM)
+    const int S = 76;
+    // The buffer is sized for a full chunk (2 (L + 1) W floats per vertex, 1.6 GB
+    // at W = 256, L = 5) whatever V, so that no later call of this SDB allocates or
+    // moves it: a call may be captured, and a captured one holds its address.
+    constexpr int VCHUNK = GH_ADJOINT_CHUNK;
     const size_t need = adjoint_buffer_floats(W, L, VCHUNK, S, nsm);
     if (s->adj_floats < need) {
         if (s->adj) cudaFree(s->adj);
