@@ -199,9 +199,12 @@ __device__ __forceinline__ float csg_eval(const float4 *P, int n, float x, float
 //    run's minimum (with the fold before it) by 2 R is never the minimum;
 //  * a subtracted or intersected primitive that is 2 R below the fold before
 //    it never raises it.
-// A margin far above the FP32 rounding of the values (and the 1e-4 by which a
-// rotation may miss orthonormality) is added, so the masked fold gives the
-// full fold's value bit for bit.  Scenes with a primitive whose bounding
+// A margin far above the FP32 rounding of the values is added, so the masked
+// fold gives the full fold's value bit for bit: 4e-5 of the values and the
+// position, and 2e-5 (the skip test's factor) of the largest distance to a
+// centre plus bounding radius, with which a distance's rounding grows (at most
+// about 6e-7 of it: two spheres of radius 2e5 that meet inside a unit scene gave
+// another mesh without this term).  Scenes with a primitive whose bounding
 // radius is infinite (sizes for which the distance may not be 1-Lipschitz)
 // get full masks.  32 blocks per axis at every N: the masks then cost 14 us for
 // 36 primitives, and 4 to 7 of them remain in a warp's union of masks; blocks of
@@ -238,13 +241,16 @@ __device__ void cull_block(const float4 *P, int nprim, const GridP &g, int b, fl
     const float x = fmaf(bi * edge + half, g.h, g.lo[0]), y = fmaf(bj * edge + half, g.h, g.lo[1]),
                 z = fmaf(bk * edge + half, g.h, g.lo[2]);
     const float R = 0.8660255f * edge * g.h * 1.0003f;
-    const float pos = fabsf(x) + fabsf(y) + fabsf(z) + R + 1.f;
     bool full = false;
+    float size = 0.f;  // of |p - c| + rb <= |d| + 2 rb, the largest
     for (int i = 0; i < nprim; ++i) {
         int op;
-        dist[i * T] = prim_dist(P + 5 * i, x, y, z, op);
-        if (!(P[5 * i + 4].y < INFINITY)) full = true;
+        const float d = prim_dist(P + 5 * i, x, y, z, op), rb = P[5 * i + 4].y;
+        dist[i * T] = d;
+        if (!(rb < INFINITY)) full = true;
+        size = fmaxf(size, fmaf(2.f, rb, fabsf(d)));
     }
+    const float margin = fmaf(4e-5f, fabsf(x) + fabsf(y) + fabsf(z) + R + 1.f, 2e-5f * size);
     for (int w = 0; w < nw; ++w) out[w] = full ? 0xFFFFFFFFu : 0u;
     if (full) return;
     float f = 0.f;  // the fold at the centre
@@ -259,12 +265,12 @@ __device__ void cull_block(const float4 *P, int nprim, const GridP &g, int b, fl
             }
             for (; i < e; ++i) {
                 const float d = dist[i * T];
-                if (!(d > m + 2.f * R + 4e-5f * (fabsf(d) + fabsf(m) + pos))) out[i >> 5] |= 1u << (i & 31);
+                if (!(d > m + 2.f * R + fmaf(4e-5f, fabsf(d) + fabsf(m), margin))) out[i >> 5] |= 1u << (i & 31);
             }
             f = m;
         } else {
             const float d = op == GH_OP_SUBTRACT ? -dist[i * T] : dist[i * T];
-            if (!(d < f - 2.f * R - 4e-5f * (fabsf(d) + fabsf(f) + pos))) out[i >> 5] |= 1u << (i & 31);
+            if (!(d < f - 2.f * R - fmaf(4e-5f, fabsf(d) + fabsf(f), margin))) out[i >> 5] |= 1u << (i & 31);
             f = fmaxf(f, d);
             ++i;
         }
