@@ -509,8 +509,10 @@ void launch_cull(const Item *items, int n, int max_prims, cudaStream_t st) {
     if (max_prims < CULL_MIN) return;
     constexpr unsigned blocks = CULL_NB * CULL_NB * CULL_NB;  // at most; an item's surplus ones return at once
     const dim3 grid((blocks + CULL_T - 1) / CULL_T, (unsigned)n);
-    const size_t smem = (size_t)max_prims * (sizeof(Prim) + CULL_T * sizeof(float));
-    cudaFuncSetAttribute(k_cull, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr size_t per_prim = sizeof(Prim) + CULL_T * sizeof(float);
+    const size_t smem = (size_t)max_prims * per_prim;
+    // the limit of the largest scene, whatever this one's: another thread's launch may come between these two calls
+    cudaFuncSetAttribute(k_cull, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(GH_MAX_PRIMS * per_prim));
     k_cull<<<grid, CULL_T, smem, st>>>(items);
 }
 
@@ -1393,7 +1395,7 @@ void launch_cont_csg(const Prim *prims, int nprim, const GridP &g, Scratch &s, c
     // the queue's slots read 0 until written (the scratch holds earlier calls' data)
     cudaMemsetAsync(s.marks_raw, 0, sizeof(unsigned long long) * (size_t)s.cap_marks, st);
     k_cont_seed<<<(n_seeds + 127) / 128, 128, smem, st>>>(prims, nprim, g, s, seeds, n_seeds);
-    cudaFuncSetAttribute(k_cont_csg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (no limit to raise: 20 KB of primitives at most beside 23 KB)
     // one CTA (8 warps) per SM: the crawl's front holds a few thousand cells
     k_cont_csg<<<nsm, 256, smem, st>>>(prims, nprim, g, s, out);
 }
