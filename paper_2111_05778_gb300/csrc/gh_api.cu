@@ -355,7 +355,8 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     auto up = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
     unsigned char *base;
     if (dev_alloc(s, &base, up(sizeof(float) * np) + 2 * up(sizeof(float) * mw) + up(sizeof(float) * h.n_mid * W) +
-                                up(2 * mw) + 2 * up(6 * mw) + up(sizeof(Counters))))
+                                up(2 * mw) + 2 * up(6 * mw) + up(sizeof(Counters)) + up(8) +
+                                up(sizeof(float) * 2 * h.n_mid * W)))
         return GH_ERR_CUDA;
     auto take = [&](size_t bytes) {
         unsigned char *p = base;
@@ -367,11 +368,14 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     float *d_bm = (float *)take(sizeof(float) * h.n_mid * W);
     uint16_t *d_wbf = (uint16_t *)take(2 * mw), *d_wx6 = (uint16_t *)take(6 * mw), *d_wx6t = (uint16_t *)take(6 * mw);
     s->mlp.err = (Counters *)take(sizeof(Counters));
-    GH_CUDA(cudaMemsetAsync(s->mlp.err, 0, sizeof(Counters), 0));
+    uint32_t *d_kbits = (uint32_t *)take(8);  // (next to err: cleared with it)
+    float *d_kap = (float *)take(sizeof(float) * 2 * h.n_mid * W);
+    GH_CUDA(cudaMemsetAsync(s->mlp.err, 0, (size_t)((char *)d_kap - (char *)s->mlp.err), 0));
     GH_CUDA(cudaMemcpy(s->d_params, P, sizeof(float) * np, cudaMemcpyHostToDevice));
-    launch_prep_mlp(s->d_params, W, h.n_mid, d_wt, d_wtb, d_wbf, d_wx6, d_wx6t, d_bm, 0);
+    launch_prep_mlp(s->d_params, W, h.n_mid, d_wt, d_wtb, d_wbf, d_wx6, d_wx6t, d_bm, d_kap, d_kbits, 0);
     GH_CUDA(cudaGetLastError());
-    GH_CUDA(cudaStreamSynchronize(0));  // the layouts are complete before any stream uses them
+    // (waits for stream 0: the layouts are complete before any stream uses them)
+    GH_CUDA(cudaMemcpy(s->mlp.own, d_kbits, sizeof(s->mlp.own), cudaMemcpyDeviceToHost));
     const float *d_w0 = s->d_params, *d_b0 = s->d_params + 3 * W;
     const float *d_wout = s->d_params + (size_t)4 * W + (size_t)h.n_mid * (WW + W);
     MlpDev &m = s->mlp;
@@ -392,6 +396,8 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     m.wbf = d_wbf;
     m.wx6 = d_wx6;
     m.wx6t = d_wx6t;
+    m.kap = d_kap;
+    m.kbits = d_kbits;
     s->nparam = np;
     return GH_OK;
 }
@@ -701,13 +707,16 @@ static constexpr int LAUNCHES_HOP = 2, LAUNCHES_LISTS = 3, LAUNCHES_VERTS = 1, L
 // the FFMA engine for networks deeper than that engine's shared memory takes.
 static bool fp32_on_tensor(const MlpDev &m) { return m.n_mid <= x6_max_mid(); }
 
-static void hop_mlp_fp32(const gh_sdb *first, const Item *di, int n, int nsm, cudaStream_t st) {
-    if (fp32_on_tensor(first->mlp)) launch_hop_mlp_x6(di, n, first->mlp.width, nsm, st);
+// (first: an SDB of the group, for its width and depth; own: some SDB of it has
+// layers with corrections of their own)
+static void hop_mlp_fp32(const gh_sdb *first, bool own, const Item *di, int n, int nsm, cudaStream_t st) {
+    if (fp32_on_tensor(first->mlp)) launch_hop_mlp_x6(di, n, first->mlp.width, own, nsm, st);
     else launch_hop_mlp_fp32(di, n, first->mlp.width, nsm, st);
 }
 
-static void vertices_mlp_fp32(const gh_sdb *first, const Item *di, int n, int nsm, bool refine_list, cudaStream_t st) {
-    if (fp32_on_tensor(first->mlp)) launch_eval_vertices_mlp_x6(di, n, first->mlp.width, nsm, refine_list, st);
+static void vertices_mlp_fp32(const gh_sdb *first, bool own, const Item *di, int n, int nsm, bool refine_list,
+                              cudaStream_t st) {
+    if (fp32_on_tensor(first->mlp)) launch_eval_vertices_mlp_x6(di, n, first->mlp.width, own, nsm, refine_list, st);
     else launch_eval_vertices_mlp_fp32(di, n, first->mlp.width, nsm, refine_list, st);
 }
 
@@ -718,12 +727,13 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
     if (rc) return rc;
     long long launches = LAUNCHES_HOP + LAUNCHES_LISTS + LAUNCHES_VERTS + LAUNCHES_MC;
     const int tiles = o.mlp_tiles == 1 ? 1 : 2;
+    const bool own = s->mlp.own[0] != 0;
     mark_phase(0, st);
     launch_init(c, st);
     if (o.method == GH_METHOD_ENUM) {
         // Sec. 2 enumeration: every lattice point, every cell
         if (s->kind == GH_SDB_CSG) launch_lattice_csg(s->d_prims, s->nprim, g, c, st);
-        else if (fp32_on_tensor(s->mlp)) launch_lattice_mlp_x6(s->d_item, s->mlp.width, nsm, st);
+        else if (fp32_on_tensor(s->mlp)) launch_lattice_mlp_x6(s->d_item, s->mlp.width, own, nsm, st);
         else launch_lattice_mlp_fp32(s->d_item, s->mlp.width, nsm, st);
         launch_enum_stats(g, c, st);
         for (int p = 1; p <= 5; ++p) mark_phase(p, st);
@@ -749,11 +759,11 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(4, st);
         mark_phase(5, st);
     } else if (o.precision == GH_FP32) {
-        hop_mlp_fp32(s, s->d_item, 1, nsm, st);
+        hop_mlp_fp32(s, own, s->d_item, 1, nsm, st);
         mark_phase(1, st);
         launch_build_lists(g, c, st);
         mark_phase(2, st);
-        vertices_mlp_fp32(s, s->d_item, 1, nsm, false, st);
+        vertices_mlp_fp32(s, own, s->d_item, 1, nsm, false, st);
         mark_phase(3, st);
         mark_phase(4, st);
         mark_phase(5, st);
@@ -766,7 +776,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(3, st);
         launch_refine_select(g, c, st);
         mark_phase(4, st);
-        vertices_mlp_fp32(s, s->d_item, 1, nsm, true, st);
+        vertices_mlp_fp32(s, own, s->d_item, 1, nsm, true, st);
         mark_phase(5, st);
         launches += LAUNCHES_REFINE;
     }
@@ -1069,6 +1079,11 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             any_mlp = true;
         }
     }
+    auto own = [&](const std::pair<int, int> &gr) {
+        for (int q = gr.first; q < gr.second; ++q)
+            if (sd[P.order[q]]->mlp.own[0]) return true;
+        return false;
+    };
     long long launches = 1 + 7 + 1 + 1;  // counters, lists, Marching Cubes, status words
     launch_init_b(P.d_items, B, st);
     for (auto &gr : P.groups) {
@@ -1083,7 +1098,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             ++launches;
             launch_hop_csg(di, n, mx, nsm, o.ray_block, st);
         } else if (o.precision == GH_FP32) {
-            hop_mlp_fp32(first, di, n, nsm, st);
+            hop_mlp_fp32(first, own(gr), di, n, nsm, st);
         } else {
             launch_hop_mlp_bf16(di, n, first->mlp.width, nsm, tiles, st);
         }
@@ -1099,7 +1114,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         const Item *di = P.d_items + gr.first;
         const int n = gr.second - gr.first;
         ++launches;
-        if (o.precision == GH_FP32) vertices_mlp_fp32(first, di, n, nsm, false, st);
+        if (o.precision == GH_FP32) vertices_mlp_fp32(first, own(gr), di, n, nsm, false, st);
         else launch_eval_vertices_mlp_bf16(di, n, first->mlp.width, nsm, tiles, st);
     }
     if (any_mlp && o.precision != GH_FP32) {
@@ -1111,7 +1126,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             const Item *di = P.d_items + gr.first;
             const int n = gr.second - gr.first;
             ++launches;
-            vertices_mlp_fp32(first, di, n, nsm, true, st);
+            vertices_mlp_fp32(first, own(gr), di, n, nsm, true, st);
         }
     }
     bool any_index = false;

@@ -154,7 +154,30 @@ struct MlpDev {
     const uint16_t *wx6;  // n_mid x 3 BF16 parts (low, middle, high) of the hidden weights, same layout
     const uint16_t *wx6t; // the same of the transposed weights, last layer first (adjoint)
     Counters *err;        // where the launches without an item (point lists, adjoint) flag a timeout
+    const float *kap;       // split-BF16 engine, up to 8 hidden layers: what its epilogue adds back per output,
+                            // n_mid x [W], then the same of the transposed weights, last layer first
+    const uint32_t *kbits;  // [2]: bit l W/64 + g: not kappa_units(W) throughout columns 64 g .. of layer l
+    uint32_t own[2];        // kbits, known to the host
 };
+
+// Mean shortfall of a truncated tensor-core accumulator over a dense layer, in
+// units of its last place, as a factor of the accumulator's power of two 2^e
+// (its value is m 2^e, 1 <= m < 2).  Measured 0.50 / 0.62 / 1.50 units at width
+// 64 / 128 / 256 for terms of one sign and 0.63 / 1.1 / 2.3 for mixed ones (half
+// of the activations zero); the constants lie between.
+__host__ __device__ constexpr float kappa_units(int W) {
+    return (W == 256 ? 1.9f : (W == 128 ? 0.8f : 0.5f)) * 1.1920929e-7f;
+}
+// ... and for an output with n nonzero weights (pow2: all of them powers of
+// two, so that the sum may be exact: an identity or a selection loses nothing).
+// Measured for n = 1, 2, 4, 8, 16, 32, 64, 128 of 256 inputs: 0.43 0.42 0.46 0.47
+// 0.54 0.63 0.84 1.25 units with any weights, 0 0.11 0.31 0.43 0.47 0.49 0.50 0.50
+// with powers of two (deviation 0.3 to 0.8, and at most 0.3).  With the dense
+// layer's constant an identity layer of width 256 was off by 1.9 units.
+__host__ __device__ inline float kappa_row(int W, int n, bool pow2) {
+    const float u = 1.1920929e-7f, q = n > 0 ? 1.f - 1.f / (float)n : 0.f;
+    return fminf(kappa_units(W), (pow2 ? 0.5f * q * q : 0.43f + 0.0065f * (float)n) * u);
+}
 
 // Scratch of one polygonization (device pointers) and its capacities.
 struct Scratch {
@@ -271,10 +294,11 @@ void launch_eval_points_mlp_bf16(const MlpDev &m, const float *p, long long n, f
 void launch_refine_select(const GridP &g, Scratch &s, cudaStream_t st);  // k_pipeline.cu
 // neural SDB with split-BF16 tensor-core products (k_mlp_x6.cu)
 int x6_max_mid();  // deeper networks run on the FFMA engine
-void launch_hop_mlp_x6(const Item *items, int n_items, int width, int nsm, cudaStream_t st);
-void launch_eval_vertices_mlp_x6(const Item *items, int n_items, int width, int nsm, bool refine_list,
+// (own: some item's MlpDev::own[0] is not 0)
+void launch_hop_mlp_x6(const Item *items, int n_items, int width, bool own, int nsm, cudaStream_t st);
+void launch_eval_vertices_mlp_x6(const Item *items, int n_items, int width, bool own, int nsm, bool refine_list,
                                  cudaStream_t st);
-void launch_lattice_mlp_x6(const Item *items, int width, int nsm, cudaStream_t st);
+void launch_lattice_mlp_x6(const Item *items, int width, bool own, int nsm, cudaStream_t st);
 // (a block that gave up a wait writes NaN to all its rows, and flags it in m.err;
 // so do the BF16 points and the adjoint)
 void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, float *out, int nsm, cudaStream_t st);
@@ -289,7 +313,7 @@ long long lb_words(int N);              // words of Scratch::lb
 long long lbe_words(long long nverts);  // words of Scratch::lbe
 // derived weight layouts of a neural SDB from its packed parameters (k_prep.cu)
 void launch_prep_mlp(const float *params, int W, int n_mid, float *wt, float *wtb, uint16_t *wbf, uint16_t *wx6,
-                     uint16_t *wx6t, float *bm, cudaStream_t st);
+                     uint16_t *wx6t, float *bm, float *kap, uint32_t *kbits, cudaStream_t st);  // kbits: zeroed
 // the indexed mesh's vertices and their numbers, before Marching Cubes, which writes the indices (k_index.cu)
 void launch_index_mesh(const GridP &g, Scratch &s, const gh_mesh &out, int nsm, cudaStream_t st);
 void launch_index_mesh_b(const Item *items, int n, int nsm, cudaStream_t st);

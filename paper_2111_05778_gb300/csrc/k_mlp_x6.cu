@@ -14,11 +14,13 @@
 // The accumulator adds the products from the smallest to the largest in four
 // passes over the layer's inputs: x_h w_l; x_m w_m and x_h w_m; x_l w_h and
 // x_m w_h; x_h w_h.  Only the last pass's W/16 updates are at the size of the
-// result.  The accumulator is truncated toward zero: on layers of like-signed
-// terms it was short by 0.50 / 0.62 / 1.50 units in the last place on average
-// at width 64 / 128 / 256 (0.63 / 1.1 / 2.3 with mixed signs; deviation 0.3 /
-// 0.4 / 0.6), which the epilogue adds back on average (KAPPA).  What remains
-// is below the error of a chain of FP32 FMAs (deviation 1.2 / 1.6 / 2.2).
+// result.  The accumulator is truncated toward zero; the epilogue adds back what
+// that loses on average, by the width and, where an output has few weights, by
+// their number (gh_internal.cuh: kappa_row; a selection loses nothing and gets
+// nothing).  On dense layers what remains is below the error of a chain of FP32
+// FMAs (deviation 0.3 / 0.4 / 0.6 units in the last place at width 64 / 128 / 256
+// for terms of one sign, the chain's 1.2 / 1.6 / 2.2).  Dense weights of which
+// few see a nonzero activation are corrected too much, by at most the constant.
 // The last two passes share the high part's stages in the ring.  Layer 0
 // (3 -> W) and the output layer (W -> 1) run on CUDA cores in FP32.
 //
@@ -85,12 +87,6 @@ constexpr int nst_of() {
     return W == 256 ? 4 : 3;
 }
 
-// Mean shortfall of a truncated accumulator in units of its last place, as a
-// factor of the accumulator's power of two (2^e of its value m 2^e, 1 <= m < 2).
-template <int W>
-constexpr float kappa_of() {
-    return (W == 256 ? 1.9f : (W == 128 ? 0.8f : 0.5f)) * 1.1920929e-7f;
-}
 __device__ __forceinline__ float pow2_of(float v) { return __uint_as_float(__float_as_uint(v) & 0xFF800000u); }
 
 template <int W>
@@ -105,6 +101,7 @@ struct SmemX {
     float red[3][W / 64][TM];      // per column group: output dot products (adjoint: grad_x g)
     unsigned long long full[NST], empty[NST], acc_full, a_h, a_ml, item_ready, drain;
     const uint16_t *cur_w;         // split weights of the current item
+    uint32_t kbits[2];             // layers and column groups whose outputs have their own correction (MlpDev::kbits)
     int done;
     uint32_t tmem_base;
     int ctl;
@@ -130,7 +127,7 @@ __device__ __forceinline__ float outer_f(const MlpDev &m, float x, float y, floa
 }
 
 // Loads an item's layer-0 rows, biases and output weights (epilogue threads).
-template <int W>
+template <int W, bool OWN>
 __device__ __forceinline__ void load_params(SmemX<W> &sm, const MlpDev &mm, int e) {
     for (int o = e; o < W; o += 2 * W) {
         float *q = reinterpret_cast<float *>(&sm.w0b[o & ~1]) + (o & 1);
@@ -141,6 +138,7 @@ __device__ __forceinline__ void load_params(SmemX<W> &sm, const MlpDev &mm, int 
         sm.wout[o] = mm.wout[o];
     }
     for (int i = e; i < mm.n_mid * W; i += 2 * W) sm.bmid[i] = mm.bm[i];
+    if (OWN && e < 2) sm.kbits[e] = mm.kbits[e];
 }
 
 // x[64] (this thread's row, columns 64 grp .., ReLU'd when RELU) -> x_h into
@@ -207,7 +205,23 @@ struct AdjOut {
     const uint16_t *wt6;  // split transposed weights, last layer first
 };
 
-template <int W, int MODE>
+// A CTA's end after a wait ran out: no item's lists may be read any more ...
+__device__ __noinline__ void give_up_items(const Item *items, int n_items) {
+    if (threadIdx.x == 0)
+        for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
+}
+// ... and the calls without a status get NaN in every row of the CTA
+__device__ __noinline__ void give_up_rows(float *dst, long long n, Counters *ctr) {
+    if (threadIdx.x == 0) atomicOr(&ctr->flags, FLAG_TIMEOUT);
+    if (threadIdx.x < TM)
+        for (long long i = (long long)blockIdx.x * TM + threadIdx.x; i < n; i += (long long)gridDim.x * TM)
+            dst[i] = __int_as_float(0x7FC00000);
+}
+
+// OWN: some layer of some item has outputs with corrections of their own
+// (MlpDev::kbits).  Dense networks run the form without: deciding it per layer
+// cost them 5 % (2^20 points at width 256 2.37 -> 2.48 ms: registers).
+template <int W, int MODE, bool OWN>
 __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
     k_mlp_x6(const Item *__restrict__ items_in, int n_items, const __grid_constant__ Item single,
              const float *__restrict__ pts, long long npts, float *__restrict__ outv, AdjOut adj,
@@ -229,7 +243,7 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
     const int n_mid = items[0].m.n_mid;
     const int n_gemm = MODE == XM_ADJ ? 2 * n_mid : n_mid;  // products per tile (adjoint: there and back)
 
-    if (tid >= EPI_T0) load_params<W>(sm, items[0].m, tid - EPI_T0);
+    if (tid >= EPI_T0) load_params<W, OWN>(sm, items[0].m, tid - EPI_T0);
     if (tid == 0) {
         for (int i = 0; i < NST; ++i) {
             mbar_init(&sm.full[i], 1);
@@ -462,7 +476,7 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
                     it = &items[cur];
                     col = NONE;
                     done = false;
-                    load_params<W>(sm, it->m, e);
+                    load_params<W, OWN>(sm, it->m, e);
                     bar_sync(BAR_EPI, EPI);
                     continue;
                 }
@@ -515,7 +529,7 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
             mbar_arrive(&sm.a_ml);
             // 3. the products' results, layer by layer -> the next A operands, and at
             //    the end the output dot product (adjoint: grad_x g)
-            constexpr float KAPPA = kappa_of<W>();
+            constexpr float KAPPA = kappa_units(W);
             const unsigned long long KK = pack2(KAPPA, KAPPA);
             float gs[3] = {0.f, 0.f, 0.f};
             for (int l = 0; l < n_gemm; ++l) {
@@ -537,22 +551,31 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
                         x[32 + c] = __uint_as_float(hi[c]);
                     }
                 }
+                const bool own = OWN && (sm.kbits[back ? 1 : 0] >> ((back ? l - n_mid : l) * G + grp)) & 1u;
                 if (!back) {
                     const float4 *bl = reinterpret_cast<const float4 *>(sm.bmid + l * W + c0);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        const float4 b = bl[c];
-                        // z = acc + (b + KAPPA 2^e(acc)): one rounding at the size of z
+                    // z = acc + (b + kappa 2^e(acc)): one rounding at the size of z
+                    auto put = [&](int c, const float4 &b, unsigned long long k0, unsigned long long k1) {
                         const unsigned long long z0 =
                             fadd2(pack2(x[4 * c], x[4 * c + 1]),
-                                  ffma2(pack2(pow2_of(x[4 * c]), pow2_of(x[4 * c + 1])), KK, pack2(b.x, b.y)));
+                                  ffma2(pack2(pow2_of(x[4 * c]), pow2_of(x[4 * c + 1])), k0, pack2(b.x, b.y)));
                         const unsigned long long z1 =
                             fadd2(pack2(x[4 * c + 2], x[4 * c + 3]),
-                                  ffma2(pack2(pow2_of(x[4 * c + 2]), pow2_of(x[4 * c + 3])), KK, pack2(b.z, b.w)));
+                                  ffma2(pack2(pow2_of(x[4 * c + 2]), pow2_of(x[4 * c + 3])), k1, pack2(b.z, b.w)));
                         x[4 * c] = RELU_CVT ? lo2(z0) : fmaxf(lo2(z0), 0.f);
                         x[4 * c + 1] = RELU_CVT ? hi2(z0) : fmaxf(hi2(z0), 0.f);
                         x[4 * c + 2] = RELU_CVT ? lo2(z1) : fmaxf(lo2(z1), 0.f);
                         x[4 * c + 3] = RELU_CVT ? hi2(z1) : fmaxf(hi2(z1), 0.f);
+                    };
+                    if (!own) {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) put(c, bl[c], KK, KK);
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            const float4 k = __ldg(reinterpret_cast<const float4 *>(m.kap + l * W + c0) + c);
+                            put(c, bl[c], pack2(k.x, k.y), pack2(k.z, k.w));
+                        }
                     }
                     if (MODE == XM_ADJ) {
                         if (rlive) store_row(adj.A + (size_t)(l + 1) * adj.ldl + aoff, x);
@@ -567,9 +590,21 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
                         }
                     }
                 } else {  // delta_{l'} = (W^T delta) [z_{l'} > 0], l' = 2 n_mid - 1 - l
+                    if (!own) {
 #pragma unroll
-                    for (int c = 0; c < 64; ++c)
-                        x[c] = ((c < 32 ? mk.x : mk.y) >> (c & 31)) & 1u ? fmaf(pow2_of(x[c]), KAPPA, x[c]) : 0.f;
+                        for (int c = 0; c < 64; ++c) x[c] = fmaf(pow2_of(x[c]), KAPPA, x[c]);
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) {
+                            const float4 k = __ldg(reinterpret_cast<const float4 *>(m.kap + l * W + c0) + c);
+                            x[4 * c] = fmaf(pow2_of(x[4 * c]), k.x, x[4 * c]);
+                            x[4 * c + 1] = fmaf(pow2_of(x[4 * c + 1]), k.y, x[4 * c + 1]);
+                            x[4 * c + 2] = fmaf(pow2_of(x[4 * c + 2]), k.z, x[4 * c + 2]);
+                            x[4 * c + 3] = fmaf(pow2_of(x[4 * c + 3]), k.w, x[4 * c + 3]);
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < 64; ++c) x[c] = ((c < 32 ? mk.x : mk.y) >> (c & 31)) & 1u ? x[c] : 0.f;
                     if (rlive) store_row(adj.D + (size_t)(2 * n_mid - 1 - l) * adj.ldl + aoff, x);
                 }
                 if (l + 1 < n_gemm) {
@@ -591,8 +626,10 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
                             gs[2] = fmaf(wb.y, x[2 * p + 1], fmaf(wb.x, x[2 * p], gs[2]));
                         }
                     } else {
-                        // eight sums of every eighth column: the roundings of one long
-                        // chain would be the largest error of a narrow network
+                        // eight sums of every eighth column: eight fused multiply-adds in a
+                        // row instead of 64.  (With four, 9 of 8,640 vertices of the
+                        // paper-form network at N = 77 lie beyond 1e-4 h of the FP64 mesh
+                        // instead of 8; an exact evaluator at the FP32 lattice has 9.)
                         const float4 *wp = reinterpret_cast<const float4 *>(sm.wout + c0);
                         float d[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -690,32 +727,33 @@ __global__ void __launch_bounds__(64 + 2 * W, ctas_of<W>())
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (*ctl & CTL_ABORT) {
-        if (tid == 0)  // no item's lists may be read after this
-            for (int b = 0; b < n_items; ++b) atomicOr(&items[b].s.ctr->flags, FLAG_TIMEOUT);
-        // calls without a status: NaN in every row of this CTA says that it gave
-        // up (s_v multiplies every term of the gradient's sums)
-        if ((MODE == XM_POINTS || MODE == XM_ADJ) && tid < TM) {
-            float *const dst = MODE == XM_POINTS ? outv : adj.s;
-            for (long long i = (long long)blockIdx.x * TM + tid; i < npts; i += (long long)gridDim.x * TM)
-                dst[i] = __int_as_float(0x7FC00000);
-        }
+    if (sm.ctl & CTL_ABORT) {
+        if (MODE == XM_POINTS) give_up_rows(outv, npts, ctr0);
+        else if (MODE == XM_ADJ) give_up_rows(adj.s, npts, ctr0);  // s_v multiplies every term of the gradient's sums
+        else give_up_items(items_in, n_items);
     }
-    if (warp == 1)
+    if (threadIdx.x >> 5 == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
-template <int W, int MODE>
-void launch_x6(const Item *items, int n_items, const Item &single, const float *p, long long n, float *out,
+template <int W, int MODE, bool OWN>
+void launch_x6_as(const Item *items, int n_items, const Item &single, const float *p, long long n, float *out,
                const AdjOut &adj, int nsm, cudaStream_t st) {
     const size_t smem = sizeof(SmemX<W>) + 1024;
-    cudaFuncSetAttribute(k_mlp_x6<W, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_mlp_x6<W, MODE, OWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int grid = nsm * ctas_of<W>();
     if (MODE == XM_POINTS || MODE == XM_ADJ) {
         const long long tiles = (n + TM - 1) / TM;
         if (grid > tiles) grid = (int)(tiles < 1 ? 1 : tiles);
     }
-    k_mlp_x6<W, MODE><<<grid, EPI_T0 + 2 * W, smem, st>>>(items, n_items, single, p, n, out, adj, wait_limit_ns());
+    k_mlp_x6<W, MODE, OWN><<<grid, EPI_T0 + 2 * W, smem, st>>>(items, n_items, single, p, n, out, adj, wait_limit_ns());
+}
+
+template <int W, int MODE>
+void launch_x6(bool own, const Item *items, int n_items, const Item &single, const float *p, long long n, float *out,
+               const AdjOut &adj, int nsm, cudaStream_t st) {
+    if (own) launch_x6_as<W, MODE, true>(items, n_items, single, p, n, out, adj, nsm, st);
+    else launch_x6_as<W, MODE, false>(items, n_items, single, p, n, out, adj, nsm, st);
 }
 
 }  // namespace
@@ -729,21 +767,21 @@ void launch_x6(const Item *items, int n_items, const Item &single, const float *
 
 int x6_max_mid() { return MAXMID; }
 
-void launch_hop_mlp_x6(const Item *items, int n_items, int width, int nsm, cudaStream_t st) {
-    GH_X6_W(width, (launch_x6<WW, XM_HOP>(items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+void launch_hop_mlp_x6(const Item *items, int n_items, int width, bool own, int nsm, cudaStream_t st) {
+    GH_X6_W(width, (launch_x6<WW, XM_HOP>(own, items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
 }
 
-void launch_eval_vertices_mlp_x6(const Item *items, int n_items, int width, int nsm, bool refine_list,
+void launch_eval_vertices_mlp_x6(const Item *items, int n_items, int width, bool own, int nsm, bool refine_list,
                                  cudaStream_t st) {
     if (refine_list) {
-        GH_X6_W(width, (launch_x6<WW, XM_REFINE>(items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+        GH_X6_W(width, (launch_x6<WW, XM_REFINE>(own, items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
     } else {
-        GH_X6_W(width, (launch_x6<WW, XM_VERTS>(items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+        GH_X6_W(width, (launch_x6<WW, XM_VERTS>(own, items, n_items, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
     }
 }
 
-void launch_lattice_mlp_x6(const Item *items, int width, int nsm, cudaStream_t st) {
-    GH_X6_W(width, (launch_x6<WW, XM_LATTICE>(items, 1, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
+void launch_lattice_mlp_x6(const Item *items, int width, bool own, int nsm, cudaStream_t st) {
+    GH_X6_W(width, (launch_x6<WW, XM_LATTICE>(own, items, 1, Item{}, nullptr, 0, nullptr, AdjOut{}, nsm, st)))
 }
 
 // A network's descriptor for the kernels that take points instead of an item
@@ -758,14 +796,14 @@ static Item points_item(const MlpDev &m) {
 
 void launch_eval_points_mlp_x6(const MlpDev &m, const float *p, long long n, float *out, int nsm, cudaStream_t st) {
     const Item it = points_item(m);
-    GH_X6_W(m.width, (launch_x6<WW, XM_POINTS>(nullptr, 1, it, p, n, out, AdjOut{}, nsm, st)))
+    GH_X6_W(m.width, (launch_x6<WW, XM_POINTS>(m.own[0] != 0, nullptr, 1, it, p, n, out, AdjOut{}, nsm, st)))
 }
 
 void launch_adj_mlp_x6(const MlpDev &m, const float *P, const float *dL, long long V, float *A, float *D, float *s,
                        uint32_t *mask, long long ldl, int nsm, cudaStream_t st) {
     const Item it = points_item(m);
     const AdjOut a{dL, A, D, s, reinterpret_cast<uint2 *>(mask), ldl, m.wx6t};
-    GH_X6_W(m.width, (launch_x6<WW, XM_ADJ>(nullptr, 1, it, P, V, nullptr, a, nsm, st)))
+    GH_X6_W(m.width, (launch_x6<WW, XM_ADJ>((m.own[0] | m.own[1]) != 0, nullptr, 1, it, P, V, nullptr, a, nsm, st)))
 }
 
 }  // namespace gh

@@ -18,12 +18,16 @@
 //       each part in K-blocks of 64 inputs with the 128-byte swizzle;
 //   wx6t the same of the transposed weights (rows = inputs of the layer, K =
 //       its outputs), layer n_mid first (the adjoint walks down);
-//   bm  hidden biases, n_mid x [W].
+//   bm  hidden biases, n_mid x [W];
+//   kap, kbits  what the split-BF16 engine's epilogue adds back (gh_internal.cuh:
+//       kappa_row, from the number of nonzero weights of each output).
 #include "gh_internal.cuh"
 
 namespace gh {
 
 namespace {
+
+constexpr int x6_mid_limit = 8;  // = x6_max_mid(): 8 layers x W/64 groups are the 32 bits of a word of kbits
 
 __device__ __forceinline__ int perm_pos(int o) {
     const int og = o & 15, m = o >> 4;
@@ -40,7 +44,8 @@ __device__ __forceinline__ float bf16_val(uint16_t b) { return __uint_as_float((
 __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ params, int W, int n_mid,
                                                   float *__restrict__ wt, float *__restrict__ wtb,
                                                   uint16_t *__restrict__ wbf, uint16_t *__restrict__ wx6,
-                                                  uint16_t *__restrict__ wx6t, float *__restrict__ bm) {
+                                                  uint16_t *__restrict__ wx6t, float *__restrict__ bm,
+                                                  float *__restrict__ kap, uint32_t *__restrict__ kbits) {
     const long long WW = (long long)W * W, total = (long long)n_mid * WW;
     const long long mid0 = 4LL * W;  // W0 and b0 come first
     const int KB = W / 64;
@@ -78,13 +83,34 @@ __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ para
         const int l = (int)(e / W), o = (int)(e - (long long)l * W);
         bm[e] = params[mid0 + l * (WW + W) + WW + o];
     }
+    if (n_mid > x6_mid_limit) return;
+    // one warp per output: d = 0 forward, 1 transposed (its layers last first)
+    const int lane = threadIdx.x & 31, nwarp = (int)(gridDim.x * blockDim.x) >> 5;
+    for (int e = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < 2 * n_mid * W; e += nwarp) {
+        const int d = e / (n_mid * W), r = e - d * n_mid * W, l = r / W, o = r - l * W;
+        const float *w = params + mid0 + (d ? n_mid - 1 - l : l) * (WW + W);
+        int n = 0;
+        bool pow2 = true;
+        for (int i = lane; i < W; i += 32) {
+            const float v = d ? w[(long long)i * W + o] : w[(long long)o * W + i];
+            n += v != 0.f;
+            pow2 = pow2 && (__float_as_uint(v) & 0x7FFFFFu) == 0u;
+        }
+        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        pow2 = __all_sync(0xFFFFFFFFu, pow2);
+        if (lane == 0) {
+            const float k = kappa_row(W, n, pow2);
+            kap[e] = k;
+            if (k != kappa_units(W)) atomicOr(kbits + d, 1u << (l * KB + (o >> 6)));
+        }
+    }
 }
 
 }  // namespace
 
 void launch_prep_mlp(const float *params, int W, int n_mid, float *wt, float *wtb, uint16_t *wbf, uint16_t *wx6,
-                     uint16_t *wx6t, float *bm, cudaStream_t st) {
-    k_prep_mlp<<<1024, 256, 0, st>>>(params, W, n_mid, wt, wtb, wbf, wx6, wx6t, bm);
+                     uint16_t *wx6t, float *bm, float *kap, uint32_t *kbits, cudaStream_t st) {
+    k_prep_mlp<<<1024, 256, 0, st>>>(params, W, n_mid, wt, wtb, wbf, wx6, wx6t, bm, kap, kbits);
 }
 
 }  // namespace gh
