@@ -228,6 +228,8 @@ struct gh_sdb {
     // CSG
     Prim *d_prims = nullptr;
     int nprim = 0;
+    int in_runs = 0;        // of these in runs of two or more spheres joined by union
+    bool cullable = false;  // every primitive has a bounding radius
     // MLP
     MlpDev mlp{};
     std::vector<void *> dbufs;
@@ -317,8 +319,14 @@ static int create_csg(gh_sdb *s, const gh_sdb_desc *d) {
     // change the fold), pad[1] the length of the union-sphere run it starts
     std::vector<Prim> q(pr.size());
     memcpy(q.data(), pr.data(), pr.size() * sizeof(Prim));
-    for (size_t i = 0; i < pr.size(); ++i) {
+    s->cullable = true;
+    for (size_t i = 0, end = 0; i < pr.size(); ++i) {
         const int run = prim_sphere_run(q.data(), (int)q.size(), (int)i);
+        if (i >= end && run >= 2) {
+            s->in_runs += run;
+            end = i + run;
+        }
+        s->cullable = s->cullable && isfinite(prim_bound_radius(q[i]));
         pr[i].pad[0] = prim_bound_radius(q[i]);
         memcpy(&pr[i].pad[1], &run, sizeof(run));
         pr[i].pad[2] = 0.f;
@@ -552,9 +560,13 @@ static int ensure_scratch(gh_sdb *s, int N, long long want_marks, long long want
     return GH_OK;
 }
 
+static bool uses_cull(const gh_sdb *s, int N) {
+    return s->kind == GH_SDB_CSG && s->cullable && cull_pays(N, s->nprim, s->in_runs);
+}
+
 // The culling masks of an analytic SDB (sized once, for every grid).
-static int ensure_cull(gh_sdb *s) {
-    const long long need = s->kind == GH_SDB_CSG ? cull_words(s->nprim) : 0;
+static int ensure_cull(gh_sdb *s, int N) {
+    const long long need = uses_cull(s, N) ? cull_words(s->nprim) : 0;
     if (s->scr.cap_cull >= need) return GH_OK;
     if (s->scr.cull) cudaFree(s->scr.cull);
     s->scr.cull = nullptr;
@@ -603,6 +615,7 @@ static Item make_item(const gh_sdb *s, const GridP &g) {
     Item it{};  // zero-initialised, padding included, so descriptors compare bytewise
     it.g = g;
     it.s = s->scr;
+    if (!uses_cull(s, g.N)) it.s.cull = nullptr;  // (held for another grid, or from the pool)
     it.m = s->mlp;
     it.prims = s->d_prims;
     it.nprim = s->nprim;
@@ -725,6 +738,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
     Scratch &c = s->scr;
     int rc = sync_item(s, g, st);
     if (rc) return rc;
+    const bool cull = uses_cull(s, g.N);
     long long launches = LAUNCHES_HOP + LAUNCHES_LISTS + LAUNCHES_VERTS + LAUNCHES_MC;
     const int tiles = o.mlp_tiles == 1 ? 1 : 2;
     const bool own = s->mlp.own[0] != 0;
@@ -746,7 +760,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         return GH_OK;
     }
     if (s->kind == GH_SDB_CSG) {
-        if (cull_words(s->nprim) > 0) {
+        if (cull) {
             launch_cull(s->d_item, 1, s->nprim, st);
             ++launches;
         }
@@ -754,7 +768,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(1, st);
         launch_build_lists(g, c, st);
         mark_phase(2, st);
-        launch_eval_vertices_csg(s->d_prims, s->nprim, g, c, nsm, st);
+        launch_eval_vertices_csg(s->d_prims, s->nprim, g, s->h_item.s, nsm, st);
         mark_phase(3, st);
         mark_phase(4, st);
         mark_phase(5, st);
@@ -827,7 +841,7 @@ extern "C" int gh_polygonize(const gh_grid *grid, const gh_sdb *csdb, const gh_o
     long long want_m = 8 * N2 > (1 << 16) ? 8 * N2 : (1 << 16);
     long long want_v = 2 * want_m;
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((rc = ensure_scratch(s, g.N, want_m, want_v)) || (rc = ensure_cull(s))) return rc;
+        if ((rc = ensure_scratch(s, g.N, want_m, want_v)) || (rc = ensure_cull(s, g.N))) return rc;
         if (o.method == GH_METHOD_ENUM && (rc = ensure_lattice(s, g.N))) return rc;
         if (wants_index(*out) && (rc = ensure_index(s))) return rc;
         if ((rc = enqueue_once(s, g, o, *out, nsm, st))) return rc;
@@ -1092,10 +1106,16 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         const Item *di = P.d_items + gr.first;
         const int n = gr.second - gr.first;
         if (first->kind == GH_SDB_CSG) {
-            int mx = 1;
-            for (int q = gr.first; q < gr.second; ++q) mx = sd[P.order[q]]->nprim > mx ? sd[P.order[q]]->nprim : mx;
-            launch_cull(di, n, mx, st);
-            ++launches;
+            int mx = 1, mc = 0;  // most primitives of an item, of one with masks
+            for (int q = gr.first; q < gr.second; ++q) {
+                const int b = P.order[q];
+                mx = sd[b]->nprim > mx ? sd[b]->nprim : mx;
+                if (uses_cull(sd[b], P.g[b].N)) mc = sd[b]->nprim > mc ? sd[b]->nprim : mc;
+            }
+            if (mc) {
+                launch_cull(di, n, mc, st);
+                ++launches;
+            }
             launch_hop_csg(di, n, mx, nsm, o.ray_block, st);
         } else if (o.precision == GH_FP32) {
             hop_mlp_fp32(first, own(gr), di, n, nsm, st);
@@ -1208,7 +1228,7 @@ extern "C" int gh_polygonize_batch(int B, const gh_grid *grids, const gh_sdb *co
     for (int attempt = 0; attempt < 4; ++attempt) {
         for (int b = 0; b < B; ++b)
             if ((rc = ensure_scratch(sd[b], P.g[b].N, want_m[b], want_v[b])) ||
-                (rc = ensure_cull(sd[b])) ||
+                (rc = ensure_cull(sd[b], P.g[b].N)) ||
                 (wants_index(outs[b]) && (rc = ensure_index(sd[b])))) {
                 cudaFree(d_items);
                 return rc;

@@ -203,7 +203,7 @@ struct Scratch {
     long long cap_vis;              // words of vis
     unsigned long long *lb;         // one-pass scans: [0] call number, then a status word per tile of columns and lines
     unsigned long long *lbe;        // the same per tile of list entries (indexed output)
-    uint32_t *cull;                 // analytic SDBs: primitive masks per block of cells (NULL: fold every primitive)
+    uint32_t *cull;                 // analytic SDBs: primitive masks per block of cells (in a descriptor: NULL to fold every primitive)
     long long cap_cull;             // words of cull
 };
 
@@ -250,7 +250,8 @@ unsigned long long wait_limit_ns();
 cudaError_t upload_mc_table(const int32_t *ntri, const int32_t *edges);  // k_pipeline.cu
 void launch_init(Scratch &s, cudaStream_t st);
 void launch_stage_prims(const Prim *src, Prim *dst, int nprim, cudaStream_t st);  // records + bounding radii
-long long cull_words(int nprim);  // words of Scratch::cull, whatever the grid (0: no masks)
+bool cull_pays(int N, int nprim, int in_runs);  // in_runs: primitives in runs of spheres joined by union
+long long cull_words(int nprim);  // words of Scratch::cull, whatever the grid
 void launch_cull(const Item *items, int n, int max_prims, cudaStream_t st);
 void launch_hop_csg(const Item *items, int n_items, int max_prims, int nsm, int block, cudaStream_t st);
 void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st);

@@ -205,24 +205,42 @@ __device__ __forceinline__ float csg_eval(const float4 *P, int n, float x, float
 // centre plus bounding radius, with which a distance's rounding grows (at most
 // about 6e-7 of it: two spheres of radius 2e5 that meet inside a unit scene gave
 // another mesh without this term).  Scenes with a primitive whose bounding
-// radius is infinite (sizes for which the distance may not be 1-Lipschitz)
-// get full masks.  32 blocks per axis at every N: the masks then cost 14 us for
-// 36 primitives, and 4 to 7 of them remain in a warp's union of masks; blocks of
-// 16 cells left most of them at N = 64 (hop 189 us without masks, 246 with
-// those, 123 with these).  Below CULL_MIN primitives the masks cost more than
-// they save.
+// radius is infinite (sizes for which the distance may not be 1-Lipschitz) have
+// none.  32 blocks per axis at every N: the masks then cost 14 us for 36
+// primitives, and 4 to 7 of them remain in a warp's union of masks; blocks of 16
+// cells left most of them at N = 64 (hop 189 us without masks, 246 with those, 123
+// with these).
 // ---------------------------------------------------------------------------
-static constexpr int CULL_NB = 32, CULL_MIN = 6;
+static constexpr int CULL_NB = 32;
 
 __host__ __device__ inline int cull_edge(int N) { return (N + CULL_NB - 1) / CULL_NB; }  // cells per block and axis
 __host__ __device__ inline int cull_blocks(int N) { return (N + cull_edge(N) - 1) / cull_edge(N); }
 
+// Whether the masks pay.  What they cost is one distance per primitive and
+// block and a slower step (mask loads, the dispatch per primitive); what they save
+// is a primitive's dispatch and skip test per step, or, in a run of spheres joined by
+// union, whose loop has no dispatch, one square root.  Mesh calls without / with
+// masks, n primitives of which s in such runs:
+//   n = 6, s = 0:    N = 32 0.96 to 1.00, 128 1.07 to 1.11, 512 1.17 to 1.24
+//   n = 12, s = 0:   N = 16 1.04, 64 1.17, 512 1.64 to 1.80
+//   n = 64, s = 0:   N = 16 1.26, 64 1.90, 512 2.7
+//   n = s = 24:      N = 64 0.78 to 0.86, 256 0.90, 512 1.00 to 1.04
+//   n = s = 64:      N = 64 0.76, 128 0.90, 256 1.06 to 1.11, 512 1.3
+//   n = s = 128:     N = 32 0.77, 64 0.96 to 0.99, 128 1.35 to 1.45, 512 2.0
+//   n = s = 250:     N = 16 0.56, 64 1.1 to 1.2, 512 2.7
+//   n = 21, s = 16:  N = 64 1.04, 128 1.23, 256 1.27
+//   n = 69, s = 64:  N = 64 0.86, 128 0.98, 256 1.14
+// So: six or more outside of runs that are no small part of the scene, or s + 24
+// (n - s) times N from 16,384 on.
+bool cull_pays(int N, int nprim, int in_runs) {
+    const int other = nprim - in_runs;
+    return nprim >= 6 && ((other >= 6 && 4 * other >= in_runs) || (in_runs + 24 * other) * (long long)N >= 16384);
+}
+
 // Words of the masks' buffer.  It holds any grid's masks, so that a scene's
 // buffer never moves: a captured batch graph keeps its address, and the number
 // of blocks is not monotone in N (29 per axis at N = 200, 32 at N = 64).
-long long cull_words(int nprim) {
-    return nprim < CULL_MIN ? 0 : (long long)CULL_NB * CULL_NB * CULL_NB * ((nprim + 31) / 32);
-}
+long long cull_words(int nprim) { return (long long)CULL_NB * CULL_NB * CULL_NB * ((nprim + 31) / 32); }
 
 // The block index of a cell or lattice index i: i / cull_edge(N), the last
 // lattice point in the last block (the quotient of i + 1/2 is at least 1/128
@@ -241,18 +259,15 @@ __device__ void cull_block(const float4 *P, int nprim, const GridP &g, int b, fl
     const float x = fmaf(bi * edge + half, g.h, g.lo[0]), y = fmaf(bj * edge + half, g.h, g.lo[1]),
                 z = fmaf(bk * edge + half, g.h, g.lo[2]);
     const float R = 0.8660255f * edge * g.h * 1.0003f;
-    bool full = false;
     float size = 0.f;  // of |p - c| + rb <= |d| + 2 rb, the largest
     for (int i = 0; i < nprim; ++i) {
         int op;
         const float d = prim_dist(P + 5 * i, x, y, z, op), rb = P[5 * i + 4].y;
         dist[i * T] = d;
-        if (!(rb < INFINITY)) full = true;
         size = fmaxf(size, fmaf(2.f, rb, fabsf(d)));
     }
     const float margin = fmaf(4e-5f, fabsf(x) + fabsf(y) + fabsf(z) + R + 1.f, 2e-5f * size);
-    for (int w = 0; w < nw; ++w) out[w] = full ? 0xFFFFFFFFu : 0u;
-    if (full) return;
+    for (int w = 0; w < nw; ++w) out[w] = 0u;
     float f = 0.f;  // the fold at the centre
     for (int i = 0; i < nprim;) {
         const int op = i ? __float_as_int(P[5 * i].y) : GH_OP_UNION;
@@ -283,7 +298,7 @@ __global__ void __launch_bounds__(CULL_T) k_cull(const Item *__restrict__ items)
     extern __shared__ float4 sprim[];
     const Item &it = items[blockIdx.y];
     const int nprim = it.nprim, nb = cull_blocks(it.g.N), nblk = nb * nb * nb;
-    if (it.kind != GH_SDB_CSG || !it.s.cull || nprim < CULL_MIN || blockIdx.x * CULL_T >= nblk) return;
+    if (it.kind != GH_SDB_CSG || !it.s.cull || blockIdx.x * CULL_T >= nblk) return;
     const float4 *s4 = reinterpret_cast<const float4 *>(it.prims);
     for (int i = threadIdx.x; i < nprim * 5; i += CULL_T) sprim[i] = s4[i];
     __syncthreads();
@@ -498,15 +513,15 @@ __global__ void __launch_bounds__(512) k_hop_csg(const Item *__restrict__ items,
     for (int cur = 0; cur < n_items; ++cur) {
         const Item &it = items[cur];
         load_prims(sprim, it.prims, it.nprim);  // ends with __syncthreads
-        if (it.s.cull && it.nprim >= CULL_MIN) hop_csg<true>(it, sprim, buf[threadIdx.x >> 5]);
+        if (it.s.cull) hop_csg<true>(it, sprim, buf[threadIdx.x >> 5]);
         else hop_csg<false>(it, sprim, buf[threadIdx.x >> 5]);
         __syncthreads();  // the primitives are restaged only after every warp is done
     }
 }
 
-// The culling masks of n items, before their hopping.
+// The culling masks of those of n items that have some (Scratch::cull), before
+// their hopping; max_prims: of those.
 void launch_cull(const Item *items, int n, int max_prims, cudaStream_t st) {
-    if (max_prims < CULL_MIN) return;
     constexpr unsigned blocks = CULL_NB * CULL_NB * CULL_NB;  // at most; an item's surplus ones return at once
     const dim3 grid((blocks + CULL_T - 1) / CULL_T, (unsigned)n);
     constexpr size_t per_prim = sizeof(Prim) + CULL_T * sizeof(float);
@@ -810,7 +825,7 @@ __device__ __forceinline__ void vertex_pos(const GridP &g, unsigned long long ke
 __device__ __forceinline__ void eval_vertices_csg(const float4 *sprim, int nprim, const GridP &g, const Scratch &s,
                                                   unsigned long long t0, unsigned long long stride) {
     const unsigned long long V = s.ctr->verts;
-    if (s.cull && nprim >= CULL_MIN) {  // whole warps (t0 - lane starts the warp's vertices)
+    if (s.cull) {  // whole warps (t0 - lane starts the warp's vertices)
         const int lane = threadIdx.x & 31, nw = (nprim + 31) / 32, nb = cull_blocks(g.N);
         const float inv_edge = 1.f / (float)cull_edge(g.N);
         const uint32_t N1 = (uint32_t)g.N + 1u;
