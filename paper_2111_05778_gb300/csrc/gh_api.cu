@@ -359,22 +359,24 @@ static int create_mlp(gh_sdb *s, const gh_sdb_desc *d) {
     const size_t WW = (size_t)W * W;
     // (one allocation for all of them: each costs the host tens of microseconds
     // to make and to free, and a training step makes a new SDB)
+    // (the FFMA engine's layouts for the networks it runs, the tensor-core engines' for the others)
     const size_t mw = (size_t)h.n_mid * WW;
+    const bool deep = h.n_mid > x6_max_mid();
+    const size_t fw = deep ? sizeof(float) * mw : 0, bw = deep ? 0 : 2 * mw;  // bytes of an FP32, a BF16 copy
     auto up = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
     unsigned char *base;
-    if (dev_alloc(s, &base, up(sizeof(float) * np) + 2 * up(sizeof(float) * mw) + up(sizeof(float) * h.n_mid * W) +
-                                up(2 * mw) + 2 * up(6 * mw) + up(sizeof(Counters)) + up(8) +
-                                up(sizeof(float) * 2 * h.n_mid * W)))
+    if (dev_alloc(s, &base, up(sizeof(float) * np) + 2 * up(fw) + up(sizeof(float) * h.n_mid * W) + up(bw) +
+                                2 * up(3 * bw) + up(sizeof(Counters)) + up(8) + up(sizeof(float) * 2 * h.n_mid * W)))
         return GH_ERR_CUDA;
     auto take = [&](size_t bytes) {
         unsigned char *p = base;
         base += up(bytes);
-        return (void *)p;
+        return (void *)(bytes ? p : nullptr);
     };
     s->d_params = (float *)take(sizeof(float) * np);
-    float *d_wt = (float *)take(sizeof(float) * mw), *d_wtb = (float *)take(sizeof(float) * mw);
+    float *d_wt = (float *)take(fw), *d_wtb = (float *)take(fw);
     float *d_bm = (float *)take(sizeof(float) * h.n_mid * W);
-    uint16_t *d_wbf = (uint16_t *)take(2 * mw), *d_wx6 = (uint16_t *)take(6 * mw), *d_wx6t = (uint16_t *)take(6 * mw);
+    uint16_t *d_wbf = (uint16_t *)take(bw), *d_wx6 = (uint16_t *)take(3 * bw), *d_wx6t = (uint16_t *)take(3 * bw);
     s->mlp.err = (Counters *)take(sizeof(Counters));
     uint32_t *d_kbits = (uint32_t *)take(8);  // (next to err: cleared with it)
     float *d_kap = (float *)take(sizeof(float) * 2 * h.n_mid * W);
@@ -727,10 +729,14 @@ static void hop_mlp_fp32(const gh_sdb *first, bool own, const Item *di, int n, i
     else launch_hop_mlp_fp32(di, n, first->mlp.width, nsm, st);
 }
 
-static void vertices_mlp_fp32(const gh_sdb *first, bool own, const Item *di, int n, int nsm, bool refine_list,
-                              cudaStream_t st) {
-    if (fp32_on_tensor(first->mlp)) launch_eval_vertices_mlp_x6(di, n, first->mlp.width, own, nsm, refine_list, st);
-    else launch_eval_vertices_mlp_fp32(di, n, first->mlp.width, nsm, refine_list, st);
+static void vertices_mlp_fp32(const gh_sdb *first, bool own, const Item *di, int n, int nsm, cudaStream_t st) {
+    if (fp32_on_tensor(first->mlp)) launch_eval_vertices_mlp_x6(di, n, first->mlp.width, own, nsm, false, st);
+    else launch_eval_vertices_mlp_fp32(di, n, first->mlp.width, nsm, st);
+}
+
+// Refinement of the BF16 path, whose networks all fit the split-BF16 engine.
+static void refine_mlp(const gh_sdb *first, bool own, const Item *di, int n, int nsm, cudaStream_t st) {
+    launch_eval_vertices_mlp_x6(di, n, first->mlp.width, own, nsm, true, st);
 }
 
 static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh_mesh &out, int nsm,
@@ -777,7 +783,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(1, st);
         launch_build_lists(g, c, st);
         mark_phase(2, st);
-        vertices_mlp_fp32(s, own, s->d_item, 1, nsm, false, st);
+        vertices_mlp_fp32(s, own, s->d_item, 1, nsm, st);
         mark_phase(3, st);
         mark_phase(4, st);
         mark_phase(5, st);
@@ -790,7 +796,7 @@ static int enqueue_once(gh_sdb *s, const GridP &g, const gh_options &o, const gh
         mark_phase(3, st);
         launch_refine_select(g, c, st);
         mark_phase(4, st);
-        vertices_mlp_fp32(s, own, s->d_item, 1, nsm, true, st);
+        refine_mlp(s, own, s->d_item, 1, nsm, st);
         mark_phase(5, st);
         launches += LAUNCHES_REFINE;
     }
@@ -1134,7 +1140,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
         const Item *di = P.d_items + gr.first;
         const int n = gr.second - gr.first;
         ++launches;
-        if (o.precision == GH_FP32) vertices_mlp_fp32(first, own(gr), di, n, nsm, false, st);
+        if (o.precision == GH_FP32) vertices_mlp_fp32(first, own(gr), di, n, nsm, st);
         else launch_eval_vertices_mlp_bf16(di, n, first->mlp.width, nsm, tiles, st);
     }
     if (any_mlp && o.precision != GH_FP32) {
@@ -1146,7 +1152,7 @@ static int batch_enqueue(const BatchPlan &P, int B, gh_sdb *const *sd, const gh_
             const Item *di = P.d_items + gr.first;
             const int n = gr.second - gr.first;
             ++launches;
-            vertices_mlp_fp32(first, own(gr), di, n, nsm, true, st);
+            refine_mlp(first, own(gr), di, n, nsm, st);
         }
     }
     bool any_index = false;

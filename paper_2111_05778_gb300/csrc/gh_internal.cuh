@@ -145,16 +145,18 @@ struct MlpDev {
     float radial;  // 1, or 0 without the |p| term (GH_MLP_NO_RADIAL)
     const float *w0;    // [W][3]
     const float *b0;    // [W]
-    const float *wt;    // n_mid x [W(in)][W(out)] transposed FP32 hidden weights
-    const float *wtb;   // n_mid x [W(out)][W(in)] FP32 hidden weights, inputs permuted like wt's outputs
     const float *bm;    // n_mid x [W]
     const float *wout;  // [W]
     float bout;
+    // FFMA engine (more than 8 hidden layers; else NULL)
+    const float *wt;    // n_mid x [W(in)][W(out)] transposed FP32 hidden weights
+    const float *wtb;   // n_mid x [W(out)][W(in)] FP32 hidden weights, inputs permuted like wt's outputs
+    // tensor-core engines (up to 8 hidden layers; else NULL)
     const uint16_t *wbf;  // n_mid x BF16 hidden weights in the tensor-core tile layout
     const uint16_t *wx6;  // n_mid x 3 BF16 parts (low, middle, high) of the hidden weights, same layout
     const uint16_t *wx6t; // the same of the transposed weights, last layer first (adjoint)
     Counters *err;        // where the launches without an item (point lists, adjoint) flag a timeout
-    const float *kap;       // split-BF16 engine, up to 8 hidden layers: what its epilogue adds back per output,
+    const float *kap;       // split-BF16 engine: what its epilogue adds back per output,
                             // n_mid x [W], then the same of the transposed weights, last layer first
     const uint32_t *kbits;  // [2]: bit l W/64 + g: not kappa_units(W) throughout columns 64 g .. of layer l
     uint32_t own[2];        // kbits, known to the host
@@ -279,8 +281,7 @@ void launch_eval_points_csg(const Prim *prims, int nprim, const float *p, long l
 
 // neural SDB, FP32 on the FFMA pipe (k_mlp_fp32.cu)
 void launch_hop_mlp_fp32(const Item *items, int n_items, int width, int nsm, cudaStream_t st);
-void launch_eval_vertices_mlp_fp32(const Item *items, int n_items, int width, int nsm, bool refine_list,
-                                   cudaStream_t st);
+void launch_eval_vertices_mlp_fp32(const Item *items, int n_items, int width, int nsm, cudaStream_t st);
 void launch_eval_points_mlp_fp32(const MlpDev &m, const float *p, long long n, float *out, int nsm,
                                  cudaStream_t st);
 void launch_lattice_mlp_fp32(const Item *items, int width, int nsm, cudaStream_t st);

@@ -12,13 +12,15 @@
 //   dL/dW_l = c sum_v s_v delta_l relu(z_{l-1})^T,  dL/db_l = c sum_v s_v delta_l,
 //   dL/dW_0 = c sum_v s_v delta_0 p^T,  dL/dw = c sum_v s_v relu(z_L),  dL/db = c sum_v s_v.
 // The activations are recomputed from the vertices (nothing is kept from the
-// polygonization).  Over a chunk of vertices the forward pass (storing every
-// z_l) and the delta chain run on the FP32 tile engine of the network's
-// evaluation (k_mlp_fp32.cu); the weight sums are dense FP32 products on the
-// FFMA pipe (k_gemm, 128 x 128 tiles, 8 x 8 per thread in packed FP32 pairs,
-// register-prefetched 16-deep K slices); the
-// sums over vertices use a split over the vertex axis whose partial results
-// are added in a fixed order, so the gradient is deterministic.
+// polygonization).  Over a chunk of vertices, networks of up to 8 hidden layers
+// run the forward pass and the delta chain in one launch of the split-BF16
+// engine (k_mlp_x6.cu, which stores relu(z_l), delta_l and s_v) and the hidden
+// layers' weight sums in another (k_adj_wgrad.cu).  Deeper ones run both passes
+// on the FP32 tile engine (k_mlp_fp32.cu, which stores z_l) and the weight sums
+// as dense FP32 products on the FFMA pipe (k_gemm).  The first and the last
+// layer's sums are k_adj_ends for all.  Sums over vertices are split over the
+// vertex axis and the partial results added in a fixed order, so the gradient is
+// deterministic.
 #include <math.h>
 #include <string.h>
 
@@ -32,17 +34,13 @@ namespace {
 
 constexpr int BM = 128, BN = 128, BK = 16, GT = 256, PADS = 4;
 
-// C[M x N] (+ split z: C + z*M*ldc) = sum_k opA(m,k) opB(k,n) over the k-range
-// [z*kchunk, (z+1)*kchunk) with opA(m,k) = (TA ? A[k*lda+m] : A[m*lda+k]),
-// relu'd if RA and scaled by ksc[k]; opB likewise.  Epilogue: + bias[n],
-// then * [mask[m*ldc+n] > 0].
+// C[M x N] + z*M*N = sum_k ksc[k] A[k*M+m] relu(B[k*N+n]) over the k-range
+// [z*kchunk, (z+1)*kchunk): the FFMA path's weight sums (k = vertices).
 // 128 x 128 tile per CTA, 8 x 8 per thread as packed FP32 pairs
 // (fma.rn.f32x2); the next 16-deep K slice is fetched into registers while
 // the current one is multiplied out of the other shared-memory buffer.
-template <bool TA, bool TB, bool RA, bool RB>
-__global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, const float *__restrict__ A, int lda,
-                                             const float *__restrict__ B, int ldb, float *__restrict__ C, int ldc,
-                                             const float *__restrict__ bias, const float *__restrict__ mask,
+__global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, const float *__restrict__ A,
+                                             const float *__restrict__ B, float *__restrict__ C,
                                              const float *__restrict__ ksc, int kchunk) {
     __shared__ __align__(16) float As[2][BK][BM + PADS];
     __shared__ __align__(16) float Bs[2][BK][BN + PADS];
@@ -50,44 +48,23 @@ __global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, const float *_
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
     const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
     // each thread stages 8 elements of A and 8 of B per slice: element
-    // e = tid + 256 r (r < 8) of the 128 x 16 slice, walking the contiguous
-    // direction of the operand's storage fastest
+    // e = tid + 256 r (r < 8) of the 16 x 128 slice, consecutive lanes on
+    // consecutive columns
     float ra[8], rb[8];
     auto fetch = [&](int k0) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            const int e = tid + r * GT;  // 0..2047
-            {
-                const int mm = TA ? (e & (BM - 1)) : (e >> 4), kk = TA ? (e >> 7) : (e & (BK - 1));
-                const int m = m0 + mm, k = k0 + kk;
-                float v = 0.f;
-                if (m < M && k < ke) {
-                    v = TA ? A[(size_t)k * lda + m] : A[(size_t)m * lda + k];
-                    if (RA) v = fmaxf(v, 0.f);
-                    if (ksc) v *= ksc[k];
-                }
-                ra[r] = v;
-            }
-            {
-                const int nn = TB ? (e >> 4) : (e & (BN - 1)), kk = TB ? (e & (BK - 1)) : (e >> 7);
-                const int n = n0 + nn, k = k0 + kk;
-                float v = 0.f;
-                if (n < N && k < ke) {
-                    v = TB ? B[(size_t)n * ldb + k] : B[(size_t)k * ldb + n];
-                    if (RB) v = fmaxf(v, 0.f);
-                }
-                rb[r] = v;
-            }
+            const int e = tid + r * GT, c = e & (BM - 1), k = k0 + (e >> 7);
+            ra[r] = m0 + c < M && k < ke ? A[(size_t)k * M + m0 + c] * ksc[k] : 0.f;
+            rb[r] = n0 + c < N && k < ke ? fmaxf(B[(size_t)k * N + n0 + c], 0.f) : 0.f;
         }
     };
     auto stash = [&](int buf) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            const int e = tid + r * GT;
-            const int mm = TA ? (e & (BM - 1)) : (e >> 4), ka = TA ? (e >> 7) : (e & (BK - 1));
-            const int nn = TB ? (e >> 4) : (e & (BN - 1)), kbb = TB ? (e & (BK - 1)) : (e >> 7);
-            As[buf][ka][mm] = ra[r];
-            Bs[buf][kbb][nn] = rb[r];
+            const int e = tid + r * GT, c = e & (BM - 1), k = e >> 7;
+            As[buf][k][c] = ra[r];
+            Bs[buf][k][c] = rb[r];
         }
     };
     unsigned long long acc[8][4];
@@ -126,7 +103,7 @@ __global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, const float *_
             buf ^= 1;
         }
     }
-    float *Cz = C + (size_t)blockIdx.z * M * ldc;
+    float *Cz = C + (size_t)blockIdx.z * M * N;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int m = m0 + ty * 8 + i;
@@ -135,25 +112,18 @@ __global__ void __launch_bounds__(GT) k_gemm(int M, int N, int K, const float *_
         for (int j = 0; j < 4; ++j) {
             float lo, hi;
             asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[i][j]));
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int n = n0 + tx * 8 + 2 * j + u;
-                if (n >= N) continue;
-                float v = u ? hi : lo;
-                if (bias) v += bias[n];
-                if (mask && !(mask[(size_t)m * ldc + n] > 0.f)) v = 0.f;
-                Cz[(size_t)m * ldc + n] = v;
-            }
+            const int n = n0 + tx * 8 + 2 * j;
+            if (n < N) Cz[(size_t)m * N + n] = lo;
+            if (n + 1 < N) Cz[(size_t)m * N + n + 1] = hi;
         }
     }
 }
 
-template <bool TA, bool TB, bool RA, bool RB>
-void gemm(int M, int N, int K, const float *A, int lda, const float *B, int ldb, float *C, int ldc, const float *bias,
-          const float *mask, const float *ksc, int splits, cudaStream_t st) {
+void gemm(int M, int N, int K, const float *A, const float *B, float *C, const float *ksc, int splits,
+          cudaStream_t st) {
     const int kchunk = ((K + splits - 1) / splits + BK - 1) / BK * BK;
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, splits);
-    k_gemm<TA, TB, RA, RB><<<grid, GT, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, mask, ksc, kchunk);
+    k_gemm<<<grid, GT, 0, st>>>(M, N, K, A, B, C, ksc, kchunk);
 }
 
 // delta_L = w * [z_L > 0]
@@ -318,11 +288,9 @@ void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, floa
         Dl[l] = b.D + (size_t)l * b.VC * W;
     }
     const int eb = 1024;
-    // forward: pre-activations of every layer; backward chain of g (both on the
-    // FP32 tile engine of the network's evaluation)
+    // forward pass and delta chain; Z holds relu(z) from the first, z from the second
     const long long ldl = (long long)b.VC * W;
     if (L <= x6_max_mid()) {
-        // on the tensor cores, both ways per tile in one launch; Z holds relu(z)
         launch_adj_mlp_x6(m, P, dL, V, b.Z, b.D, b.s, b.mbits, ldl, b.nsm, st);
     } else {
         launch_adj_fwd_fp32(m, P, V, b.Z, ldl, b.mbits, b.nsm, st);
@@ -340,7 +308,7 @@ void adjoint_chunk(const MlpDev &m, const float *P, const float *dL, int V, floa
     if (tensor) launch_adj_wgrad(m, b.Z, b.D, b.s, V, ldl, b.part, c, grad + omid, accumulate, b.nsm, st);
     for (int l = 1; l <= (tensor ? 0 : L); ++l) {
         const size_t oW = omid + (size_t)(l - 1) * ((size_t)W * W + W), ob = oW + (size_t)W * W;
-        gemm<true, false, false, true>(W, W, V, Dl[l], W, Zl[l - 1], W, b.part, W, nullptr, nullptr, b.s, S, st);
+        gemm(W, W, V, Dl[l], Zl[l - 1], b.part, b.s, S, st);
         k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W * W, c, grad + oW, accumulate);
         k_colsum<<<dim3(W / 32, S), 256, 0, st>>>(Dl[l], V, W, b.s, rows, b.part);
         k_adj_reduce<<<gb, 256, 0, st>>>(b.part, S, (long long)W, c, grad + ob, accumulate);

@@ -420,8 +420,8 @@ __global__ void __launch_bounds__(NT, 1) k_hop_mlp_fp32(const Item *__restrict__
 }
 
 // Point lists over a batch of items: MODE 0 = the unique lattice vertices of
-// each item, MODE 1 = each item's refinement list, MODE 2 = explicit points
-// (one item), MODE 3 = all (N+1)^3 lattice points into s.lat (enumeration).
+// each item, MODE 2 = explicit points (one item), MODE 3 = all (N+1)^3 lattice
+// points into s.lat (enumeration).
 template <int W, int MODE>
 __global__ void __launch_bounds__(NT, 1) k_pts_mlp_fp32(const Item *__restrict__ items, int n_items,
                                                          const float *pts, long long npts, float *outv,
@@ -437,14 +437,11 @@ __global__ void __launch_bounds__(NT, 1) k_pts_mlp_fp32(const Item *__restrict__
         const Item &it = items[cur];
         const Scratch &s = it.s;
         const GridP &g = it.g;
-        unsigned long long *counter = MODE == 1 ? &s.ctr->next_tile2 : &s.ctr->next_tile;
         if (tid == 0) {
             const bool stopped = MODE != 2 && (s.ctr->flags & STOP_FLAGS);
             const unsigned long long nl = (unsigned long long)(g.N + 1) * (g.N + 1) * (g.N + 1);
-            total_s = stopped ? 0ull
-                              : (MODE == 0 ? s.ctr->verts
-                                           : (MODE == 1 ? s.ctr->refine : (MODE == 3 ? nl : (unsigned long long)npts)));
-            tile_s = total_s ? atomicAdd(counter, 1ull) : 0ull;
+            total_s = stopped ? 0ull : (MODE == 0 ? s.ctr->verts : (MODE == 3 ? nl : (unsigned long long)npts));
+            tile_s = total_s ? atomicAdd(&s.ctr->next_tile, 1ull) : 0ull;
         }
         __syncthreads();
         const unsigned long long t = tile_s, total = total_s;
@@ -465,7 +462,7 @@ __global__ void __launch_bounds__(NT, 1) k_pts_mlp_fp32(const Item *__restrict__
                     p = make_float4(fmaf((float)a, g.h, g.lo[0]), fmaf((float)b, g.h, g.lo[1]),
                                     fmaf((float)c, g.h, g.lo[2]), 0.f);
                 } else {
-                    const unsigned long long key = s.vkey[MODE == 1 ? (unsigned long long)s.rlist[r] : r];
+                    const unsigned long long key = s.vkey[r];
                     const int N1 = g.N + 1;
                     const uint32_t line = (uint32_t)(key & 0xFFFFFFFFull), c = (uint32_t)(key >> 32);
                     const uint32_t a = line / (uint32_t)N1, b = line - a * (uint32_t)N1;
@@ -483,7 +480,6 @@ __global__ void __launch_bounds__(NT, 1) k_pts_mlp_fp32(const Item *__restrict__
                 const float f = outer_f(it.m, sm.p[tid], sm.g[tid]);
                 if (MODE != 2 && !isfinite(f)) atomicOr(&s.ctr->flags, FLAG_NONFINITE);
                 if (MODE == 0) s.vval[r] = f;
-                else if (MODE == 1) s.vval[s.rlist[r]] = f;
                 else if (MODE == 3) s.lat[r] = f;
                 else outv[r] = f;
             }
@@ -569,17 +565,11 @@ void launch_hop_mlp_fp32(const Item *items, int n_items, int width, int nsm, cud
     })
 }
 
-void launch_eval_vertices_mlp_fp32(const Item *items, int n_items, int width, int nsm, bool refine_list,
-                                   cudaStream_t st) {
+void launch_eval_vertices_mlp_fp32(const Item *items, int n_items, int width, int nsm, cudaStream_t st) {
     GH_DISPATCH_W(width, {
         const size_t smem = sizeof(Smem<WW>);
-        if (refine_list) {
-            const int grid = occupancy_grid(k_pts_mlp_fp32<WW, 1>, smem, nsm);
-            k_pts_mlp_fp32<WW, 1><<<grid, NT, smem, st>>>(items, n_items, nullptr, 0, nullptr, wait_limit_ns());
-        } else {
-            const int grid = occupancy_grid(k_pts_mlp_fp32<WW, 0>, smem, nsm);
-            k_pts_mlp_fp32<WW, 0><<<grid, NT, smem, st>>>(items, n_items, nullptr, 0, nullptr, wait_limit_ns());
-        }
+        const int grid = occupancy_grid(k_pts_mlp_fp32<WW, 0>, smem, nsm);
+        k_pts_mlp_fp32<WW, 0><<<grid, NT, smem, st>>>(items, n_items, nullptr, 0, nullptr, wait_limit_ns());
     })
 }
 

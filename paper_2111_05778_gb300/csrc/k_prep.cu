@@ -1,7 +1,9 @@
 // Derived layouts of a neural SDB's weights, built on the device from the
 // packed parameter block W0[W][3] b0[W] { W_l[W][W] b_l[W] } x n_mid w_out[W]
 // b_out, so that creating an SDB costs one upload and one launch.
-//   wt  (FP32 evaluation engine): per layer [input i][output o], the outputs
+// Networks of more than 8 hidden layers run on the FFMA engine and get wt and
+// wtb (wt != NULL), the others the rest:
+//   wt  (FFMA engine): per layer [input i][output o], the outputs
 //       of a row permuted so that position q*64 + og*4 + e holds output
 //       og + 16(4q + e);
 //   wtb (adjoint delta chain): per layer [output o][input i], the inputs
@@ -19,15 +21,13 @@
 //   wx6t the same of the transposed weights (rows = inputs of the layer, K =
 //       its outputs), layer n_mid first (the adjoint walks down);
 //   bm  hidden biases, n_mid x [W];
-//   kap, kbits  what the split-BF16 engine's epilogue adds back (gh_internal.cuh:
+//   kap, kbits  (8 layers of W/64 groups at most fit a word) what the split-BF16 engine's epilogue adds back (gh_internal.cuh:
 //       kappa_row, from the number of nonzero weights of each output).
 #include "gh_internal.cuh"
 
 namespace gh {
 
 namespace {
-
-constexpr int x6_mid_limit = 8;  // = x6_max_mid(): 8 layers x W/64 groups are the 32 bits of a word of kbits
 
 __device__ __forceinline__ int perm_pos(int o) {
     const int og = o & 15, m = o >> 4;
@@ -55,8 +55,11 @@ __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ para
         const long long r = e - l * WW;
         const int o = (int)(r / W), i = (int)(r - (long long)o * W);  // W_l[o][i]
         const float v = params[mid0 + l * (WW + W) + r];
-        wt[l * WW + (long long)i * W + perm_pos(o)] = v;
-        wtb[l * WW + (long long)o * W + perm_pos(i)] = v;
+        if (wt) {  // a network for the FFMA engine
+            wt[l * WW + (long long)i * W + perm_pos(o)] = v;
+            wtb[l * WW + (long long)o * W + perm_pos(i)] = v;
+            continue;
+        }
         const int kb = i >> 6, kk = i & 63;
         const int byte = (o >> 3) * 1024 + (o & 7) * 128 + (((kk >> 3) ^ (o & 7)) << 4) + (kk & 7) * 2;
         const uint16_t hi = bf16_rne(v);
@@ -83,7 +86,7 @@ __global__ void __launch_bounds__(256) k_prep_mlp(const float *__restrict__ para
         const int l = (int)(e / W), o = (int)(e - (long long)l * W);
         bm[e] = params[mid0 + l * (WW + W) + WW + o];
     }
-    if (n_mid > x6_mid_limit) return;
+    if (wt) return;
     // one warp per output: d = 0 forward, 1 transposed (its layers last first)
     const int lane = threadIdx.x & 31, nwarp = (int)(gridDim.x * blockDim.x) >> 5;
     for (int e = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < 2 * n_mid * W; e += nwarp) {
