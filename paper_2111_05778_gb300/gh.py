@@ -283,7 +283,7 @@ class Buffers:
         self.cap_cells = int(cap_cells)
         self.cap_verts = int(cap_verts)
         if cap_verts:
-            keys = True  # the face indices are derived from the edge keys
+            keys = True  # the library writes face indices only beside edge keys
         self.tri_xyz = torch.empty((max(self.cap_tris, 1), 3, 3), dtype=torch.float32, device=dev)
         self.tri_keys = torch.empty((max(self.cap_tris, 1), 3), dtype=torch.int64, device=dev) if keys else None
         self.cell_ids = torch.empty(max(self.cap_cells, 1), dtype=torch.int64, device=dev) if cap_cells else None
@@ -353,8 +353,10 @@ def polygonize(sdb: Sdb, N, lo=-1.0, hi=1.0, precision="fp32", tau_mode=GH_TAU_D
     keys = bool(keys) or bool(indexed)
     key = (int(N), keys, bool(cells), bool(indexed))
     # first guess of the triangles: 4 per column for one closed surface, 8 for a
-    # scene (a guess too small costs a second polygonization)
-    cap = sdb._cap.get(key, (8 if sdb.kind == GH_SDB_CSG else 4) * int(N) * int(N) + 4096)
+    # scene of several primitives (a guess too small costs a second
+    # polygonization, one too large memory that the mesh keeps: 1.2 GB at N = 2048)
+    scene = sdb.kind == GH_SDB_CSG and sdb.prims.shape[0] > 1
+    cap = sdb._cap.get(key, (8 if scene else 4) * int(N) * int(N) + 4096)
     for _ in range(3):
         capv = cap // 2 + 4096 if indexed else 0
         bufs = Buffers(cap, keys=keys, cap_cells=cap if cells else 0, cap_verts=capv)
