@@ -138,9 +138,9 @@ typedef struct {
  * is there; a sum of a few terms is truncated where an FMA rounds (deviation
  * about 0.3 units in the last place for one to eight terms, the FMA chain's 0.3
  * to 0.45, and up to 0.5 units low where no bias is added).  A network of more
- * than 8 hidden layers (identities added, for instance) gets the FMA chain.  A
- * hidden activation that overflows float32 makes f NaN
- * (GH_ERR_NONFINITE).  Deeper networks run on FP32 FMAs.
+ * than 8 hidden layers (identities added, for instance) gets the FMA chain.
+ * Where a sum of a hidden layer overflows float32, below zero as well as above,
+ * f may become NaN or inf (GH_ERR_NONFINITE), although the ReLU cuts it off.
  * GH_BF16_REFINE_X6: as GH_BF16_REFINE; it names the split-BF16 evaluator
  * explicitly (networks it does not take are refused), gh_eval takes it too. */
 #define GH_BF16_REFINE_X6 2
@@ -163,7 +163,8 @@ typedef struct {
     int32_t ray_block; /* tuning: threads per CTA of the analytic hopper      */
                        /* (128, 256 or 512; 0 = 256)                          */
     int32_t mlp_tiles; /* tuning: 128-row tiles per CTA of the BF16 engine    */
-                       /* (1 or 2; 0 = 2)                                     */
+                       /* (1 or 2; 0 = 2).  Width 64 always runs one tile and */
+                       /* four CTAs on an SM                                  */
     int32_t method;    /* GH_METHOD_HOP (Algorithm 1, default) or             */
                        /* GH_METHOD_ENUM: f at all (N+1)^3 lattice points and */
                        /* Marching Cubes on all N^3 cells (Sec. 2), FP32 only */
@@ -270,10 +271,11 @@ int gh_polygonize(const gh_grid *grid, const gh_sdb *sdb, const gh_options *opts
 
 /* Polygonizes B SDBs, each on its own grid (Algorithm 1 for every item).
  * The ray hopping of all analytic items runs in one persistent launch, and
- * that of all neural items of one width in one persistent launch, each fed by
- * device work queues (every CTA walks the items in order and takes columns
+ * that of all neural items of one width and depth in one persistent launch, each
+ * fed by device work queues (every CTA walks the items in order and takes columns
  * from the current item's queue); lattice-vertex evaluation of the neural
- * items is batched the same way; lists and Marching Cubes run per item.
+ * items is batched the same way; lists and Marching Cubes are one launch per step
+ * over all items.
  * grids[b], sdbs[b], outs[b] as in gh_polygonize; every item needs its own
  * SDB object (B distinct pointers).  opts->precision applies to the neural
  * items (analytic items always run in FP32); BF16 items use opts->eps when
@@ -283,7 +285,9 @@ int gh_polygonize(const gh_grid *grid, const gh_sdb *sdb, const gh_options *opts
  * captures the same launch sequence into a CUDA graph and writes its
  * cudaGraphExec_t to *graph without running it again; replay it with
  * cudaGraphLaunch on a stream, and release it with gh_batch_graph_free.  The
- * SDBs, grids and output buffers stay bound to the graph. */
+ * SDBs, grids and output buffers stay bound to the graph.  The SDBs may be used
+ * otherwise between replays, on grids no larger than the captured ones (a larger
+ * grid, or a call that overflows the scratch, reallocates what the graph holds). */
 int gh_polygonize_batch(int B, const gh_grid *grids, const gh_sdb *const *sdbs, const gh_options *opts,
                         gh_mesh *outs, void *stream, void **graph);
 

@@ -1,6 +1,6 @@
 """Autotuner for batched polygonization: picks the analytic hopper's CTA size
-(ray tile: 128, 256 or 512 rays per CTA) and the BF16 engine's GEMM tile (128
-or 256 rows per weight K-block) by timing the actual batch, and caches the
+(ray tile: 128, 256 or 512 rays per CTA) and, for networks wider than 64, the
+BF16 engine's GEMM tile (128 or 256 rows per weight K-block) by timing the actual batch, and caches the
 choice per GPU and batch signature in a JSON file
 ($GH_TUNE_CACHE, default ~/.cache/gridhop-gb300/tune.json)."""
 from __future__ import annotations
@@ -58,10 +58,10 @@ def tune_batch(sdbs, Ns, precision="fp32", eps=None, repeats=2, use_cache=True):
     if key in cache:
         c = cache[key]
         return c["ray_block"], c["mlp_tiles"], c.get("timings_ms", {})
-    has_mlp = any(hasattr(s, "width") for s in sdbs)
     has_csg = any(not hasattr(s, "width") for s in sdbs)
-    cands = [(rb, mt) for rb, mt in CANDIDATES if (has_csg or rb == 256) and
-             ((has_mlp and precision == "bf16") or mt == 2)]
+    # (width 64 runs one tile per CTA whatever is asked for)
+    has_tiles = precision == "bf16" and any(getattr(s, "width", 64) > 64 for s in sdbs)
+    cands = [(rb, mt) for rb, mt in CANDIDATES if (has_csg or rb == 256) and (has_tiles or mt == 2)]
     base = gh.polygonize_batch(sdbs, Ns, precision=precision, eps=eps)
     caps = [int(c * 1.05) + 4096 for c in base.counts()]
     timings = {}
