@@ -27,10 +27,13 @@
 //                thread owns the row (one ray or one point): the layer-0
 //                operand, the grid-hopping step of Algorithm 1 (with the eps
 //                shrink) or the store of f.
-// What bounds it at width 256 is the SM's shared-memory port: per tile and
-// layer 192 KB of operand reads, 64 or 128 KB of weights and 64 KB of
-// activations written and 32 KB of biases read are about 3,000 cycles at 128
-// bytes a cycle, against 2,048 of the products; a phase takes 3,200.
+// At width 256 a phase takes 3,200 cycles against 2,048 of its products.  By the
+// bytes the SM's shared-memory port comes next: per tile and layer 192 KB of
+// operand reads, 64 or 128 KB of weights and 64 KB of activations written and 32
+// KB of biases read are about 3,000 cycles at 128 bytes a cycle.  The counters
+// agree on the bytes (89 a cycle read and written with the tensor pipe at 49 %)
+// but rate the banks at a third of their peak and the load/store pipe at 41 %, so
+// they leave open whether the port or the hand-overs between the roles bind.
 // Every wait is bounded (2 s of %globaltimer); a timeout sets an error flag,
 // makes all roles leave their loops, drains the copies in flight, and frees
 // TMEM before the kernel returns.
