@@ -430,9 +430,9 @@ int gh_last_profile(gh_profile *out);
  * at once, satisfied or not -- a way to exercise the timeout path.
  * Process-wide; later launches take it.
  * The one-pass scans of gh_polygonize and gh_polygonize_csg_noalloc wait too
- * (a block for the sums of the blocks before it), analytic SDBs included: for up
- * to 2 s whatever the limit, and with a limit of 0 not at all, so that these
- * calls report GH_ERR_CUDA then. */
+ * (a block for the sums of the blocks before it), analytic SDBs included, for up
+ * to 2 s whatever the limit.  Only gh_polygonize_csg_noalloc, which has no other
+ * waits, lets them run out at once with a limit of 0, and reports GH_ERR_CUDA. */
 int gh_set_wait_limit_ns(uint64_t ns);
 
 /* Copies the library's Marching Cubes table to host memory: ntri[256] and

@@ -1504,7 +1504,7 @@ extern "C" int gh_polygonize_csg_noalloc(const gh_grid *grid, const gh_csg_prim 
     launch_init(c, st);  // clears the counters left by the previous call
     launch_stage_prims(reinterpret_cast<const Prim *>(prims), staged, n_prim, st);
     launch_hop_csg(ditem, 1, n_prim, nsm, 256, st);
-    launch_build_lists(g, c, st);
+    launch_build_lists(g, c, st, wait_limit_ns() == 0);
     launch_eval_vertices_csg(dp, n_prim, g, c, nsm, st);
     launch_mc(g, c, *out, nsm, st);
     launch_finalize(c, *out, (long long)g.N * g.N, st);

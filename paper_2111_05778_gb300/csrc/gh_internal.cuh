@@ -256,7 +256,7 @@ bool cull_pays(int N, int nprim, int in_runs);  // in_runs: primitives in runs o
 long long cull_words(int nprim);  // words of Scratch::cull, whatever the grid
 void launch_cull(const Item *items, int n, int max_prims, cudaStream_t st);
 void launch_hop_csg(const Item *items, int n_items, int max_prims, int nsm, int block, cudaStream_t st);
-void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st);
+void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st, bool expire = false);  // expire: lookback.cuh
 void launch_eval_vertices_csg(const Prim *prims, int nprim, const GridP &g, Scratch &s, int nsm,
                               cudaStream_t st);
 void launch_mc(const GridP &g, Scratch &s, const gh_mesh &out, int nsm, cudaStream_t st);

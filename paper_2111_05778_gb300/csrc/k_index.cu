@@ -108,7 +108,7 @@ __device__ __forceinline__ void put_vertices(const GridP &g, const gh_mesh &out,
 // at 10 k entries three launches less count more.)
 constexpr int EDGE_T = 256, EDGE_E = 4, EDGE_TILE = EDGE_T * EDGE_E;
 
-__global__ void __launch_bounds__(EDGE_T) k_edges(GridP g, Scratch s, gh_mesh out, bool expire) {
+__global__ void __launch_bounds__(EDGE_T) k_edges(GridP g, Scratch s, gh_mesh out) {
     __shared__ uint32_t wsum[EDGE_T / 32], base_s;
     __shared__ unsigned long long tile_s;
     const unsigned long long V = s.ctr->verts;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(EDGE_T) k_edges(GridP g, Scratch s, gh_mesh ou
             tot += wsum[q];
         }
         if (wid == 0) {
-            const uint32_t p = lb_prefix(s.lbe, s.lb[0], (long long)tile, tot, s.ctr, expire);
+            const uint32_t p = lb_prefix(s.lbe, s.lb[0], (long long)tile, tot, s.ctr, false);
             if (lane == 0) base_s = p;
         }
         __syncthreads();
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(256) k_emit_vertices_b(const Item *__restrict_
 long long lbe_words(long long nverts) { return nverts / EDGE_TILE + 1; }
 
 void launch_index_mesh(const GridP &g, Scratch &s, const gh_mesh &out, int nsm, cudaStream_t st) {
-    k_edges<<<nsm * 4, EDGE_T, 0, st>>>(g, s, out, wait_limit_ns() == 0);
+    k_edges<<<nsm * 4, EDGE_T, 0, st>>>(g, s, out);
 }
 
 void launch_index_mesh_b(const Item *items, int n, int nsm, cudaStream_t st) {

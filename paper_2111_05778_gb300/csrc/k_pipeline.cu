@@ -801,9 +801,8 @@ static long long line_groups(int N) { return (line_tiles(N) + LINES_T / 32 - 1) 
 
 long long lb_words(int N) { return 1 + column_tiles(N) + line_groups(N); }
 
-void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st) {
+void launch_build_lists(const GridP &g, Scratch &s, cudaStream_t st, bool expire) {
     const long long ct = column_tiles(g.N);
-    const bool expire = wait_limit_ns() == 0;
     k_scan_columns<<<(int)ct, SCAN_T, 0, st>>>(s, (long long)g.N * g.N, expire);
     k_scatter_marks<<<1024, 256, 0, st>>>(s);
     const size_t lsm = (size_t)((g.N + 1 + 31) / 32) * LINES_T * sizeof(uint32_t);  // <= 33 KB at N = 2048

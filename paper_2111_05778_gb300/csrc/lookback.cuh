@@ -3,8 +3,7 @@
 // word, and the block of the next tile adds up its predecessors' words until
 // it meets one that already holds the whole sum before it.  A tile waits only
 // for tiles taken earlier, whose blocks are running, so every wait ends; it is
-// bounded all the same (2 s of %globaltimer, then the timeout flag is set; with
-// gh_set_wait_limit_ns(0) every such wait runs out at once).
+// bounded all the same (2 s of %globaltimer, then the timeout flag is set).
 // A status word is call number << 34 | state << 32 | value, so words of
 // earlier calls read as not written and nothing has to be cleared.
 #pragma once

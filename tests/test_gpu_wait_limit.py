@@ -66,22 +66,19 @@ def test_every_item_of_a_batch_reports_it(precision):
 
 
 @pytest.mark.parametrize("N", [64, 200])
-def test_analytic_scans_report_it(N):
-    """The scans of the lists are the analytic pipeline's only waits, in the
-    no-allocation entry point too."""
+def test_analytic_scans(N):
+    """The scans of the lists are the analytic pipeline's only waits; the
+    no-allocation entry point reports them too.  The limit of 0 reaches them there
+    and leaves gh_polygonize alone."""
     prims = synth.csg_prims(1)
     sdb, dev = gh.CsgSdb(prims), gh.csg_prims_device(prims)
     bufs = gh.Buffers(16 * N * N + 4096, keys=True)
-
-    def noalloc():
-        return gh.polygonize_csg_noalloc(dev, len(prims), N, bufs)
-
-    for call in (noalloc, lambda: gh.polygonize(sdb, N, indexed=True)):
-        with no_waiting(), pytest.raises(gh.GhError) as e:
-            call()
+    with no_waiting():
+        with pytest.raises(gh.GhError) as e:
+            gh.polygonize_csg_noalloc(dev, len(prims), N, bufs)
         assert e.value.code == gh.GH_ERR_CUDA and "timed out" in str(e.value)
-    assert noalloc() == gh.GH_OK
-    m = gh.polygonize(sdb, N, indexed=True)
+        m = gh.polygonize(sdb, N, indexed=True)
+    assert gh.polygonize_csg_noalloc(dev, len(prims), N, bufs) == gh.GH_OK
     assert np.array_equal(_tris(m), meshutil.canonical_tris(bufs.tri_keys[:int(bufs.counts[0])].cpu().numpy()))
 
 
