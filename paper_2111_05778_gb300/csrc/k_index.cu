@@ -111,11 +111,13 @@ constexpr int EDGE_T = 256, EDGE_E = 4, EDGE_TILE = EDGE_T * EDGE_E;
 __global__ void __launch_bounds__(EDGE_T) k_edges(GridP g, Scratch s, gh_mesh out) {
     __shared__ uint32_t wsum[EDGE_T / 32], base_s;
     __shared__ unsigned long long tile_s;
+    // one decision for the block: another block's wait may run out at any time (which
+    // leaves the list as readable as it was)
+    if (__syncthreads_or((s.ctr->flags & STOP_FLAGS) != 0ull)) return;
     const unsigned long long V = s.ctr->verts;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (;;) {
-        // one thread reads the flags: another block's wait may run out meanwhile
-        if (threadIdx.x == 0) tile_s = (s.ctr->flags & STOP_FLAGS) ? V : atomicAdd(&s.ctr->tick[2], 1ull);
+        if (threadIdx.x == 0) tile_s = atomicAdd(&s.ctr->tick[2], 1ull);
         __syncthreads();
         const unsigned long long tile = tile_s, v0 = tile * EDGE_TILE + (unsigned long long)threadIdx.x * EDGE_E;
         if (tile * EDGE_TILE >= V) return;
